@@ -109,6 +109,7 @@ struct lbm_ctx {
     std::vector<uint8_t> host_solid_in;  // unpitched mask (re-initialisation)
     void* stage = nullptr;             // pinned staging buffer for host transfers
     size_t stage_bytes = 0;
+    unsigned* stage_status = nullptr;  // status word of the last macroscopic read (tail of the staging buffer)
     int timing_every = 0;
     // same-step chi (Eq. 23 at t + dt): outlet-node state between the general
     // tiles and d2q9_outlet_chi_kernel, [slot][OC_STRIDE]
@@ -542,49 +543,41 @@ lbm_status download_f(lbm_ctx* c, double* fh) {
     return LBM_OK;
 }
 
-lbm_status check_status(lbm_ctx* c) {
-    unsigned int st = 0;
-    CK(cudaMemcpyAsync(&st, c->status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+lbm_status status_result(lbm_ctx* c, unsigned st) {
     if (st & 4u) return fail(c, LBM_ERR_CUDA, "a bulk-copy destination was not 128-byte aligned; nothing was copied");
     if (st & 2u) return fail(c, LBM_ERR_TIMEOUT, "a bounded wait for a bulk copy ran out");
     if (st) return fail(c, LBM_ERR_DIVERGED, "non-finite density or velocity produced");
     return LBM_OK;
 }
 
-template <typename R>
-lbm_status copy_macros(lbm_ctx* c, void* rho, void* u, bool to_double, bool dst_dev) {
+lbm_status check_status(lbm_ctx* c) {
+    unsigned int st = 0;
+    CK(cudaMemcpyAsync(&st, c->status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    return status_result(c, st);
+}
+
+// The macroscopic fields as dense O arrays: one kernel writes them into the
+// caller's device buffers, or into the pinned staging buffer for a host
+// reader, with the status word beside them (one launch, one synchronisation).
+template <typename R, typename O>
+lbm_status copy_macros(lbm_ctx* c, O* rho, O* u, bool dst_dev) {
     const size_t N = (size_t)c->nx * c->ny;
+    const bool direct = dst_dev && kernel_writable(rho) && kernel_writable(u);
+    O* r = direct ? rho : static_cast<O*>(c->stage);
+    O* v = direct ? u : r + 2 * N;
+    CK((launch_d2q9_macros<R, O>(static_cast<const R*>(c->macro), c->info, c->nx, c->ny, c->pitch, c->plane,
+                                 c->status, r, v, c->stage_status, c->stream)));
     CK(cudaStreamSynchronize(c->stream));
-    const R* buf = static_cast<const R*>(c->stage);
-    CK(cudaMemcpyAsync(c->stage, c->macro, (size_t)4 * c->plane * sizeof(R), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    std::vector<float> fr, fu;
-    if (!to_double) {
-        fr.resize(2 * N);
-        fu.resize(2 * N);
-    }
-    for (int q = 0; q < 4; ++q)
-        for (int y = 0; y < c->ny; ++y)
-            for (int x = 0; x < c->nx; ++x) {
-                const size_t d = (size_t)y * c->pitch + x;
-                double v = c->host_solid[d] ? 0.0 : (double)buf[(size_t)q * c->plane + d];
-                const size_t h = (size_t)(q & 1) * N + (size_t)y * c->nx + x;
-                if (to_double) {
-                    (q < 2 ? static_cast<double*>(rho) : static_cast<double*>(u))[h] = v;
-                } else {
-                    (q < 2 ? fr : fu)[h] = (float)v;
-                }
-            }
-    if (!to_double) {
-        if (dst_dev) {
-            CK(cudaMemcpyAsync(rho, fr.data(), fr.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-            CK(cudaMemcpyAsync(u, fu.data(), fu.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-            CK(cudaStreamSynchronize(c->stream));
-        } else {
-            std::memcpy(rho, fr.data(), fr.size() * sizeof(float));
-            std::memcpy(u, fu.data(), fu.size() * sizeof(float));
-        }
+    lbm_status st = status_result(c, *static_cast<volatile unsigned*>(c->stage_status));
+    if (st != LBM_OK) return st;
+    if (!dst_dev) {
+        std::memcpy(rho, r, 2 * N * sizeof(O));
+        std::memcpy(u, v, 2 * N * sizeof(O));
+    } else if (!direct) {
+        CK(cudaMemcpyAsync(rho, r, 2 * N * sizeof(O), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemcpyAsync(u, v, 2 * N * sizeof(O), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
     }
     return LBM_OK;
 }
@@ -1615,7 +1608,8 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
     for (int y = 0; y < ny; ++y)
         for (int x = 0; x < nx; ++x) c->host_solid[(size_t)y * c->pitch + x] = sol[(size_t)y * nx + x];
     c->stage_bytes = std::max((size_t)18 * c->plane * c->sbytes, (size_t)4 * c->plane * c->rbytes);
-    e = cudaMallocHost(&c->stage, c->stage_bytes);
+    e = cudaMallocHost(&c->stage, c->stage_bytes + 64);
+    if (e == cudaSuccess) c->stage_status = reinterpret_cast<unsigned*>(static_cast<char*>(c->stage) + c->stage_bytes);
     if (e != cudaSuccess) {
         c->stage = nullptr;
         const std::string msg = std::string("pinned staging allocation: ") + cudaGetErrorString(e);
@@ -1779,19 +1773,15 @@ lbm_status lbm_set_chi_timing(lbm_ctx* c, int same_step) {
 lbm_status lbm_get_macros(lbm_ctx* c, float* rho, float* u, int dst_is_device) {
     if (!c || !rho || !u) return fail(c, LBM_ERR_INVALID_ARG, "NULL argument");
     if (c->d3) return lbm3::get_macros(c->d3, rho, u, dst_is_device);
-    lbm_status st = check_status(c);
-    if (st != LBM_OK) return st;
-    if (c->rbytes == 8) return copy_macros<double>(c, rho, u, false, dst_is_device != 0);
-    return copy_macros<float>(c, rho, u, false, dst_is_device != 0);
+    if (c->rbytes == 8) return copy_macros<double, float>(c, rho, u, dst_is_device != 0);
+    return copy_macros<float, float>(c, rho, u, dst_is_device != 0);
 }
 
 lbm_status lbm_get_macros_f64(lbm_ctx* c, double* rho, double* u) {
     if (!c || !rho || !u) return fail(c, LBM_ERR_INVALID_ARG, "NULL argument");
     if (c->d3) return lbm3::get_macros_f64(c->d3, rho, u);
-    lbm_status st = check_status(c);
-    if (st != LBM_OK) return st;
-    if (c->rbytes == 8) return copy_macros<double>(c, rho, u, true, false);
-    return copy_macros<float>(c, rho, u, true, false);
+    if (c->rbytes == 8) return copy_macros<double, double>(c, rho, u, false);
+    return copy_macros<float, double>(c, rho, u, false);
 }
 
 lbm_status lbm_get_populations(lbm_ctx* c, double* f) {

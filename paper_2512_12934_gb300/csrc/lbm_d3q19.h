@@ -107,6 +107,14 @@ template <typename S>
 cudaError_t launch_step(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st,
                         cudaEvent_t mid_a = nullptr, cudaEvent_t mid_b = nullptr);
 
+// Dense macroscopic fields rho [2][nz][ny][nx] and u [3][nz][ny][nx] in float,
+// 0 at solid nodes, from the density pairs and u^eq.  Nothing is written when
+// *status is set; *status_out (mapped host memory) receives it either way.
+template <typename R>
+cudaError_t launch_macros(const R* rho_pairs, const R* umac, const uint32_t* info, int nx, int ny, int nz, int pitch,
+                          long long plane, const unsigned* status, float* rho, float* u, unsigned* status_out,
+                          cudaStream_t st);
+
 // FP64 sums over fluid nodes of each component's populations and the
 // largest |u|^2: partial [nblocks][3].  FP16 storage decodes every
 // population with the reference density of the node that reads it (rref).

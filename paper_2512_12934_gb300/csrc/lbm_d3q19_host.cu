@@ -13,6 +13,7 @@
 
 #include "lbm.h"
 #include "lbm_d3q19.h"
+#include "lbm_internal.h"
 #include "lbm_d3q19_host.h"
 
 namespace lbm3 {
@@ -91,6 +92,7 @@ struct Ctx3 {
     double* flux = nullptr;
     double* scal[2] = {nullptr, nullptr};
     unsigned int* status = nullptr;
+    unsigned int* hstatus = nullptr;  // pinned: the status word of the last macroscopic read
     // FP32: tensor map of the density field as 8-byte (rho_1, rho_2) pairs,
     // box (36, 8, 8) = one collide tile and its halo
     CUtensorMap rho_map{};
@@ -363,14 +365,18 @@ void make_rho_map(Ctx3* c) {
     c->have_rho_map = r == CUDA_SUCCESS ? 1 : 0;
 }
 
-lbm_status check_status3(Ctx3* c) {
-    unsigned int st = 0;
-    CK3(cudaMemcpyAsync(&st, c->status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
-    CK3(cudaStreamSynchronize(c->stream));
+lbm_status status_result3(Ctx3* c, unsigned st) {
     if (st & STATUS3_TIMEOUT)
         return fail3(c, nullptr, LBM_ERR_TIMEOUT, "a bounded wait on the density-box tensor copy ran out");
     if (st) return fail3(c, nullptr, LBM_ERR_DIVERGED, "non-finite density or velocity produced");
     return LBM_OK;
+}
+
+lbm_status check_status3(Ctx3* c) {
+    unsigned int st = 0;
+    CK3(cudaMemcpyAsync(&st, c->status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
+    CK3(cudaStreamSynchronize(c->stream));
+    return status_result3(c, st);
 }
 
 }  // namespace
@@ -384,6 +390,7 @@ void destroy(Ctx3* c) {
         if (q) cudaFree(q);
     for (__half* q : c->rref)
         if (q) cudaFree(q);
+    if (c->hstatus) cudaFreeHost(c->hstatus);
     for (cudaEvent_t e : c->ev)
         if (e) cudaEventDestroy(e);
     delete c;
@@ -623,6 +630,7 @@ lbm_status create(const lbm_grid* g, const lbm_params* p, const lbm_open_bc* bcs
     alloc((void**)&c->scal[0], SC3_N * sizeof(double));
     alloc((void**)&c->scal[1], SC3_N * sizeof(double));
     alloc((void**)&c->status, sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hstatus, sizeof(unsigned int));
     c->mass_blocks = 304;
     alloc((void**)&c->mass_partial, (size_t)c->mass_blocks * 3 * sizeof(double));
     if (e != cudaSuccess) {
@@ -738,43 +746,56 @@ lbm_status kernel_time_split(Ctx3* c, double* pull_ms, double* collide_ms, int64
     return LBM_OK;
 }
 
+// Host readers: the pitched fields are copied out and reordered here.
 template <typename T, typename O>
-static lbm_status macros_impl(Ctx3* c, O* rho, O* u, bool dst_dev) {
+static lbm_status macros_impl(Ctx3* c, O* rho, O* u) {
     const long long N = (long long)c->nx * c->ny * c->nz;
     CK3(cudaStreamSynchronize(c->stream));
     std::vector<T> r((size_t)2 * c->plane), uu((size_t)3 * c->plane);
     CK3(cudaMemcpy(r.data(), c->rho, r.size() * sizeof(T), cudaMemcpyDeviceToHost));
     CK3(cudaMemcpy(uu.data(), c->umac, uu.size() * sizeof(T), cudaMemcpyDeviceToHost));
-    std::vector<O> ro((size_t)2 * N), uo((size_t)3 * N);
     for (int z = 0; z < c->nz; ++z)
         for (int y = 0; y < c->ny; ++y)
             for (int x = 0; x < c->nx; ++x) {
                 const long long h = hidx(c, x, y, z), d = didx(c, x, y, z);
                 const bool s = c->solid[h] != 0;
-                for (int k = 0; k < 2; ++k) ro[(size_t)k * N + h] = s ? O(0) : (O)r[2 * (size_t)d + k];
-                for (int a = 0; a < 3; ++a) uo[(size_t)a * N + h] = s ? O(0) : (O)uu[(size_t)a * c->plane + d];
+                for (int k = 0; k < 2; ++k) rho[(size_t)k * N + h] = s ? O(0) : (O)r[2 * (size_t)d + k];
+                for (int a = 0; a < 3; ++a) u[(size_t)a * N + h] = s ? O(0) : (O)uu[(size_t)a * c->plane + d];
             }
-    if (dst_dev) {
-        CK3(cudaMemcpy(rho, ro.data(), ro.size() * sizeof(O), cudaMemcpyHostToDevice));
-        CK3(cudaMemcpy(u, uo.data(), uo.size() * sizeof(O), cudaMemcpyHostToDevice));
-    } else {
-        std::memcpy(rho, ro.data(), ro.size() * sizeof(O));
-        std::memcpy(u, uo.data(), uo.size() * sizeof(O));
-    }
     return LBM_OK;
 }
 
+// Device readers: one kernel writes the caller's buffers and the status word.
+template <typename T>
+static lbm_status macros_device(Ctx3* c, float* rho, float* u) {
+    CK3(launch_macros<T>(static_cast<const T*>(c->rho), static_cast<const T*>(c->umac), c->info, c->nx, c->ny, c->nz,
+                         c->pitch, c->plane, c->status, rho, u, c->hstatus, c->stream));
+    CK3(cudaStreamSynchronize(c->stream));
+    return status_result3(c, *static_cast<volatile unsigned*>(c->hstatus));
+}
+
 lbm_status get_macros(Ctx3* c, float* rho, float* u, int dst_is_device) {
+    if (dst_is_device && lbm::kernel_writable(rho) && lbm::kernel_writable(u))
+        return c->rb == 8 ? macros_device<double>(c, rho, u) : macros_device<float>(c, rho, u);
     lbm_status st = check_status3(c);
     if (st != LBM_OK) return st;
-    return c->rb == 8 ? macros_impl<double, float>(c, rho, u, dst_is_device != 0)
-                      : macros_impl<float, float>(c, rho, u, dst_is_device != 0);
+    if (dst_is_device) {
+        const size_t N = (size_t)c->nx * c->ny * c->nz;
+        std::vector<float> r(2 * N), v(3 * N);
+        st = c->rb == 8 ? macros_impl<double, float>(c, r.data(), v.data())
+                        : macros_impl<float, float>(c, r.data(), v.data());
+        if (st != LBM_OK) return st;
+        CK3(cudaMemcpy(rho, r.data(), r.size() * sizeof(float), cudaMemcpyHostToDevice));
+        CK3(cudaMemcpy(u, v.data(), v.size() * sizeof(float), cudaMemcpyHostToDevice));
+        return LBM_OK;
+    }
+    return c->rb == 8 ? macros_impl<double, float>(c, rho, u) : macros_impl<float, float>(c, rho, u);
 }
 
 lbm_status get_macros_f64(Ctx3* c, double* rho, double* u) {
     lbm_status st = check_status3(c);
     if (st != LBM_OK) return st;
-    return c->rb == 8 ? macros_impl<double, double>(c, rho, u, false) : macros_impl<float, double>(c, rho, u, false);
+    return c->rb == 8 ? macros_impl<double, double>(c, rho, u) : macros_impl<float, double>(c, rho, u);
 }
 
 template <typename S>

@@ -178,6 +178,29 @@ cudaError_t launch_d2q9_march(const D2Args<float, float>& a, const void* tmap, c
                               const uint8_t* run_flags, int nruns, cudaStream_t st);
 constexpr int D2Q9_MARCH_BOX_W = 44, D2Q9_MARCH_BOX_H = 10;
 
+// Whether a kernel on the current device can store floats at p: device memory
+// of this device, managed or pinned host memory, 4-byte aligned.  Anything
+// else a caller names as a device destination goes through cudaMemcpy, which
+// copies it or reports the error.
+inline bool kernel_writable(const void* p) {
+    cudaPointerAttributes at{};
+    int dev = 0;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (reinterpret_cast<uintptr_t>(p) & 3u) == 0 &&
+           ((at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged ||
+            at.type == cudaMemoryTypeHost);
+}
+
+// Dense macroscopic fields rho [2][ny][nx], u [2][ny][nx] from macro [4][plane]
+// (0 at solid nodes); rho and u may be device or mapped host memory.  Nothing
+// is written when *status is set; *status_out (mapped host memory) receives it.
+template <typename R, typename O>
+cudaError_t launch_d2q9_macros(const R* macro, const uint16_t* info, int nx, int ny, int pitch, int plane,
+                               const unsigned* status, O* rho, O* u, unsigned* status_out, cudaStream_t st);
+
 // FP64 diagnostics over the current populations and macro buffer:
 // per-block partials [nblocks][3] = mass1, mass2, max |u|^2.
 // (FP16 storage decodes each population with its destination's reference
