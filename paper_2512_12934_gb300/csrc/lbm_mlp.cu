@@ -3,13 +3,10 @@
 // runs the two hidden layers on the tcgen05 tensor cores (FP32-accurate
 // split products; the default inference path).
 //
-// One CTA owns TILE samples of one ensemble member.  Forward: the four layers
-// run back to back on activations held in shared memory; each 128x128 weight
-// matrix is staged transposed so a thread's 4x4 output block reads its four
-// weights as one conflict-free float4.  Backward: the whole chain rule for the
-// tile (output error, dZ3, dW3, dA2, dZ2, dW2, dA1, dZ1, dW1 and the biases)
-// stays on chip; the tile writes its gradient partial with plain stores.  Adam
-// sums the tiles' partials in a fixed order (deterministic) and updates.
+// Training runs whole epochs inside thread-block clusters, one or more per
+// member (mlp_train_kernel): the chain rule and Adam stay on chip and in L2,
+// every sum has a fixed order (deterministic).
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -27,280 +24,432 @@
 namespace {
 
 constexpr int I = 4, H = 128, O = 2;
-constexpr int TILE = 32;        // samples per CTA
-constexpr int NTH = 256;        // threads per CTA
 constexpr int oW1 = 0, ob1 = oW1 + H * I, oW2 = ob1 + H, ob2 = oW2 + H * H, oW3 = ob2 + H, ob3 = oW3 + H * H;
 constexpr int oW4 = ob3 + H, ob4 = oW4 + O * H, P = ob4 + O;
 // Device stride of one member's parameters: P rounded up to 32 floats so that
 // every member (and every weight matrix in it) starts 128-byte aligned.
 constexpr int PS = (P + 31) & ~31;
-constexpr size_t SMEM_BYTES = (size_t)(H * H + 2 * TILE * H) * sizeof(float);
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.3989422804014327f * expf(-0.5f * z * z);
+// GELU and its derivative of one pre-activation.
+__device__ __forceinline__ void gelu_both(float z, float& a, float& d) {
+    const float t = 1.0f + erff(z * 0.70710678118654752f);
+    a = 0.5f * z * t;
+    d = 0.5f * t + z * 0.3989422804014327f * expf(-0.5f * z * z);
 }
 
-// Stage W [H][H] (row = output neuron) transposed into smem Wt[k][j].
-__device__ __forceinline__ void stage_transposed(float* Wt, const float* __restrict__ W) {
-    for (int idx = threadIdx.x; idx < H * H; idx += NTH) {
-        const int k = idx / H, j = idx % H;  // consecutive threads: consecutive j -> conflict-free store
-        Wt[k * H + j] = __ldg(W + j * H + k);
+// One Adam update (c1, c2: 1 - beta^t).
+__device__ __forceinline__ void adam_update(float& w, float& m, float& v, float g, float lr, float b1, float b2,
+                                            float c1, float c2, float eps) {
+    m = b1 * m + (1.0f - b1) * g;
+    v = b2 * v + (1.0f - b2) * g * g;
+    w -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
+// ---- training: forward, backward and Adam inside thread-block clusters ----
+// One cluster of CL CTAs trains one member; a launch runs many steps.  Every
+// CTA holds the member's whole parameter set in shared memory (136 KB) and
+// takes its share of each minibatch through forward and backward in chunks of
+// TS samples; the two 128x128 weight gradients accumulate in registers (64 per
+// thread).  At the end of a step each CTA writes its partial gradient (L2
+// resident), CTA r sums slice r of all partials in rank order (deterministic),
+// applies Adam to it, and every CTA reloads the parameters: two cluster
+// barriers a step, no launches.
+// What bounds it: a minibatch of 64 is 4 samples per CTA, so a step is a chain
+// of eleven short phases (6 us) and the exchange of 140 KB per CTA (6 us); a
+// full batch is bound by shared-memory reads of the weights (16 us per chunk
+// of 16 samples).  Exchanging over distributed shared memory instead of L2
+// took 11 us (8 CTAs) and 15 us (16 CTAs).  The form before this, one CTA per
+// 32 samples and three launches per step, left all but 10 SMs idle at a
+// minibatch of 64 and staged transposed weights with uncoalesced reads.
+// Step of 5 members, before -> now: minibatch 64 109 -> 15 us, 256 111 -> 28
+// us, 1024 161 -> 68 us, 4096 449 -> 206 us.
+constexpr int TT = 512;                        // threads per CTA
+constexpr int WS = H + 4;                      // padded weight row: 16-byte accesses of 8 rows or of one row
+constexpr int iW2 = 0, iW3 = iW2 + H * WS;     // shared parameter image (floats)
+constexpr int iW1 = iW3 + H * WS, ib1 = iW1 + H * I, ib2 = ib1 + H, ib3 = ib2 + H, iW4 = ib3 + H, ib4 = iW4 + O * H;
+constexpr int IMG = (ib4 + O + 3) & ~3;
+static_assert(oW1 % 4 == 0 && oW2 % 4 == 0 && oW3 % 4 == 0 && oW4 % 4 == 0 && ob4 % 4 == 0 && PS >= ob4 + 4,
+              "a group of four image floats must be a group of four parameters");
+
+// Parameter offset of image group q (four floats from 4 q), -1 for row padding.
+__device__ __forceinline__ int img_param(int q) {
+    const int i = 4 * q;
+    if (i < iW1) {
+        const int l = i >= iW3, t = i - l * iW3, r = t / WS, c = t % WS;
+        return c < H ? (l ? oW3 : oW2) + r * H + c : -1;
     }
+    if (i < ib2) return i - iW1 + oW1;  // W1, b1
+    if (i < ib3) return i - ib2 + ob2;
+    return i - ib3 + ob3;  // b3, W4, b4
 }
 
-// Stage W [H][H] as is into smem (used when the contraction runs over the row index).
-__device__ __forceinline__ void stage_plain(float* Ws, const float* __restrict__ W) {
-    for (int idx = threadIdx.x; idx < H * H / 4; idx += NTH)
-        reinterpret_cast<float4*>(Ws)[idx] = __ldg(reinterpret_cast<const float4*>(W) + idx);
+// The parameter image from global memory (other SMs write it during a launch:
+// read through L2).
+__device__ __forceinline__ void load_image(float* img, const float* p) {
+    // both weight matrices: rows of 32 groups, one row per warp and pass
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int r = 0; r < 2 * H; r += TT / 32) {
+        const int row = r + w, l = row / H, j = row % H;
+        *reinterpret_cast<float4*>(img + l * iW3 + j * WS + 4 * lane) =
+            __ldcg(reinterpret_cast<const float4*>(p + (l ? oW3 : oW2) + j * H) + lane);
+    }
+    for (int q = iW1 / 4 + (int)threadIdx.x; q < IMG / 4; q += TT)
+        reinterpret_cast<float4*>(img)[q] = __ldcg(reinterpret_cast<const float4*>(p + img_param(q)));
 }
 
-// out[s][j] = bias[j] + sum_k in[s][k] * M[k][j] for the tile; M in smem laid out
-// [k][j].  Thread: samples 4*sg..+3, columns 4*ng..+3.
-__device__ __forceinline__ void tile_gemm(const float* in, const float* M, const float* bias, float (&acc)[4][4]) {
-    const int sg = threadIdx.x / 32, ng = threadIdx.x % 32;
+struct TrainArgs {
+    float *params, *m, *v;    // [E][PS]
+    const float *X, *T;       // data rows
+    const int* idx;           // row order (NULL: rows 0, 1, ...)
+    const float2* coef;       // per step: 1 - beta1^t, 1 - beta2^t
+    float* part;              // [E][clusters][CL][IMG] partial gradients
+    float* out;               // gradient sums [E][clusters][P] instead of Adam (NULL: Adam)
+    int B, nsteps;            // minibatch rows, steps of this launch
+    int n, spe;               // rows of one epoch in idx, steps per epoch
+    float lr, b1, b2, eps;
+};
+
+// Samples of a chunk (TS = 4, 8 or 16): the chunk runs through the network
+// together.  Wider chunks reuse each weight read more; 4 is what a CTA gets of
+// a minibatch of 64.
+template <int TS>
+struct TrainSmem {
+    static constexpr int ACT = TS * H;
+    static constexpr int PART = 16 * 4 * H;  // partial sums of the split contractions
+    static constexpr size_t BYTES = (size_t)(IMG + 6 * ACT + PART + 2 * TS * (I + O) + TS * O) * 4;
+};
+
+__device__ __forceinline__ float dot4(float4 a, float4 b, float c) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+}
+
+// part[g][s][j] = sum over contraction group g of a[s][k] W[j][k]: a warp owns
+// four samples and 8 SG of the 128 terms, a lane the outputs j = lane + 32 r.
+template <int TS>
+__device__ __forceinline__ void train_gemm_nt(const float* W, const float* a, float* part) {
+    constexpr int SG = TS / 4;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sg = w % SG, g = w / SG;
+    float acc[4][4] = {};
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int k = g * 8 * SG; k < (g + 1) * 8 * SG; k += 4) {
+        float4 av[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = bias ? __ldg(bias + 4 * ng + c) : 0.0f;
-#pragma unroll 4
-    for (int k = 0; k < H; ++k) {
-        const float4 w = reinterpret_cast<const float4*>(M + k * H)[ng];
+        for (int s = 0; s < 4; ++s) av[s] = *reinterpret_cast<const float4*>(a + (4 * sg + s) * H + k);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const float a = in[(4 * sg + r) * H + k];
-            acc[r][0] = fmaf(a, w.x, acc[r][0]);
-            acc[r][1] = fmaf(a, w.y, acc[r][1]);
-            acc[r][2] = fmaf(a, w.z, acc[r][2]);
-            acc[r][3] = fmaf(a, w.w, acc[r][3]);
+            const float4 wv = *reinterpret_cast<const float4*>(W + (lane + 32 * r) * WS + k);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) acc[r][s] = dot4(av[s], wv, acc[r][s]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) part[(g * TS + 4 * sg + s) * H + lane + 32 * r] = acc[r][s];
+}
+
+// part[g][s][k] = sum over contraction group g of z[s][j] W[j][k]; a lane owns
+// the outputs k = 4 lane .. 4 lane + 3.
+template <int TS>
+__device__ __forceinline__ void train_gemm_nn(const float* W, const float* z, float* part) {
+    constexpr int SG = TS / 4;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sg = w % SG, g = w / SG;
+    float4 acc[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) acc[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = g * 8 * SG; j < (g + 1) * 8 * SG; j += 4) {
+        float4 zv[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) zv[s] = *reinterpret_cast<const float4*>(z + (4 * sg + s) * H + j);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 wv = *reinterpret_cast<const float4*>(W + (j + q) * WS + 4 * lane);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const float t = q == 0 ? zv[s].x : (q == 1 ? zv[s].y : (q == 2 ? zv[s].z : zv[s].w));
+                acc[s].x = fmaf(t, wv.x, acc[s].x);
+                acc[s].y = fmaf(t, wv.y, acc[s].y);
+                acc[s].z = fmaf(t, wv.z, acc[s].z);
+                acc[s].w = fmaf(t, wv.w, acc[s].w);
+            }
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) *reinterpret_cast<float4*>(part + (g * TS + 4 * sg + s) * H + 4 * lane) = acc[s];
+}
+
+// Sum of the contraction groups of output o = s * H + j, in group order.
+template <int TS>
+__device__ __forceinline__ float train_fold(const float* part, int o) {
+    float z = part[o];
+#pragma unroll
+    for (int g = 1; g < 64 / TS; ++g) z += part[g * TS * H + o];
+    return z;
+}
+
+// dw[a][c] += sum_s z[s][8 warp + a] x[s][4 lane + c]
+template <int TS>
+__device__ __forceinline__ void train_outer(const float* z, const float* x, float (&dw)[8][4]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll 2
+    for (int s = 0; s < TS; ++s) {
+        const float4 z0 = *reinterpret_cast<const float4*>(z + s * H + 8 * w);
+        const float4 z1 = *reinterpret_cast<const float4*>(z + s * H + 8 * w + 4);
+        const float4 xv = *reinterpret_cast<const float4*>(x + s * H + 4 * lane);
+        const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            dw[a][0] = fmaf(zz[a], xv.x, dw[a][0]);
+            dw[a][1] = fmaf(zz[a], xv.y, dw[a][1]);
+            dw[a][2] = fmaf(zz[a], xv.z, dw[a][2]);
+            dw[a][3] = fmaf(zz[a], xv.w, dw[a][3]);
         }
     }
 }
 
-// Forward pass of TILE samples for one member.  idx (optional) selects rows of X.
-// TRAIN: pre-activations Z1..Z3 [E][B][H] are kept for the backward pass.
-template <bool TRAIN>
-__global__ void __launch_bounds__(NTH) mlp_forward_kernel(const float* __restrict__ params, const float* __restrict__ X,
-                                                          const int* __restrict__ idx, int B, float* __restrict__ Y,
-                                                          float* __restrict__ Z) {
+template <int TS>
+__device__ __forceinline__ float train_column_sum(const float* z, int j) {
+    float t = 0.f;
+#pragma unroll
+    for (int s = 0; s < TS; ++s) t += z[s * H + j];
+    return t;
+}
+
+template <int TS, int CL>
+__global__ void __launch_bounds__(TT, 1) mlp_train_kernel(const TrainArgs a) {
     extern __shared__ __align__(16) float smem[];
-    float* Wt = smem;               // [H][H]
-    float* actA = smem + H * H;     // [TILE][H]
-    float* actB = actA + TILE * H;  // [TILE][H]
-    const int e = blockIdx.y, s0 = blockIdx.x * TILE;
-    const float* p = params + (size_t)e * PS;
-    const int sg = threadIdx.x / 32, ng = threadIdx.x % 32;
-    // layer 1 (K = 4) straight from global
-    for (int q = threadIdx.x; q < TILE * H; q += NTH) {
-        const int s = q / H, j = q % H, b = s0 + s;
-        float z = __ldg(p + ob1 + j);
-        if (b < B) {
-            const int row = idx ? idx[b] : b;
-#pragma unroll
-            for (int k = 0; k < I; ++k) z = fmaf(__ldg(p + oW1 + j * I + k), __ldg(X + (size_t)row * I + k), z);
+    using SM = TrainSmem<TS>;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    float* img = smem;
+    float *A1 = img + IMG, *A2 = A1 + SM::ACT, *A3 = A2 + SM::ACT;     // activations
+    float *D1 = A3 + SM::ACT, *D2 = D1 + SM::ACT, *D3 = D2 + SM::ACT;  // GELU', then dZ
+    float* part = D3 + SM::ACT;
+    float* xs = part + SM::PART;      // [2][TS][I]
+    float* ts = xs + 2 * TS * I;      // [2][TS][O]
+    float* dY = ts + 2 * TS * O;      // [TS][O]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int e = blockIdx.z, rank = (int)cluster.block_rank();
+    const float* p = a.params + (size_t)e * PS;
+    load_image(img, p);
+    // rows of this cluster and of this CTA in every minibatch
+    const int c0 = (int)((long long)a.B * blockIdx.y / gridDim.y);
+    const int c1 = (int)((long long)a.B * (blockIdx.y + 1) / gridDim.y);
+    const int r0 = c0 + (int)((long long)(c1 - c0) * rank / CL), r1 = c0 + (int)((long long)(c1 - c0) * (rank + 1) / CL);
+    const int nch = (r1 - r0 + TS - 1) / TS;
+    const float scale = 2.0f / ((float)a.B * (float)O);
+    // Rows travel two chunks ahead of their use: threads [0, TS) look up the data
+    // row of the chunk after next and load the inputs of the next one, so
+    // neither of the two dependent reads is waited for.  Chunk position (ps,
+    // pc); a negative row stands for a sample past the end (zeros).
+    int ps = 0, pc = 0;
+    auto lookup = [&]() -> int {
+        int row = r0 + pc * TS + tid;
+        if (ps >= a.nsteps || row >= r1) row = -1;
+        else if (a.idx) row = a.idx[(long long)(ps / a.spe) * a.n + (long long)(ps % a.spe) * a.B + row];
+        if (++pc >= nch) {
+            pc = 0;
+            ++ps;
         }
-        if (TRAIN && b < B) Z[((size_t)e * 3 + 0) * B * H + (size_t)b * H + j] = z;
-        actA[s * H + j] = gelu(z);
+        return row;
+    };
+    auto fetch = [&](int row, float4& x, float2& t) {
+        x = make_float4(0.f, 0.f, 0.f, 0.f);
+        t = make_float2(0.f, 0.f);
+        if (row >= 0) {
+            x = *reinterpret_cast<const float4*>(a.X + (size_t)row * I);
+            t = *reinterpret_cast<const float2*>(a.T + (size_t)row * O);
+        }
+    };
+    auto put = [&](int buf, const float4& x, const float2& t) {
+        *reinterpret_cast<float4*>(xs + (buf * TS + tid) * I) = x;
+        *reinterpret_cast<float2*>(ts + (buf * TS + tid) * O) = t;
+    };
+    int buf = 0, row_next = -1;
+    if (tid < TS) {
+        float4 x;
+        float2 t;
+        fetch(lookup(), x, t);
+        put(0, x, t);
+        row_next = lookup();
     }
-    // layers 2 and 3
-    const float* in = actA;
-    float* out = actB;
+    __syncthreads();
 #pragma unroll 1
-    for (int l = 0; l < 2; ++l) {
-        __syncthreads();
-        stage_transposed(Wt, p + (l == 0 ? oW2 : oW3));
-        __syncthreads();
-        float acc[4][4];
-        tile_gemm(in, Wt, p + (l == 0 ? ob2 : ob3), acc);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int s = 4 * sg + r, b = s0 + s;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int j = 4 * ng + c;
-                if (TRAIN && b < B) Z[((size_t)e * 3 + 1 + l) * B * H + (size_t)b * H + j] = acc[r][c];
-                out[s * H + j] = gelu(acc[r][c]);
-            }
-        }
-        const float* t = in;
-        in = out;
-        out = const_cast<float*>(t);
-    }
-    __syncthreads();
-    // layer 4 (2 outputs): one warp per group of 4 samples, lanes split k
-    {
-        const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int s = 4 * w + r, b = s0 + s;
-            float y0 = 0.0f, y1 = 0.0f;
-#pragma unroll
-            for (int q = 0; q < H / 32; ++q) {
-                const int k = lane + 32 * q;
-                const float a = in[s * H + k];
-                y0 = fmaf(a, __ldg(p + oW4 + k), y0);
-                y1 = fmaf(a, __ldg(p + oW4 + H + k), y1);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                y0 += __shfl_down_sync(0xffffffffu, y0, o);
-                y1 += __shfl_down_sync(0xffffffffu, y1, o);
-            }
-            if (lane == 0 && b < B) {
-                Y[((size_t)e * B + b) * O + 0] = y0 + __ldg(p + ob4);
-                Y[((size_t)e * B + b) * O + 1] = y1 + __ldg(p + ob4 + 1);
-            }
-        }
-    }
-}
-
-// Backward pass of TILE samples of one member; writes this tile's gradient
-// partial gp[e][tile][P].  T: targets indexed like X (through idx); the MSE is
-// normalised by B * O.
-__global__ void __launch_bounds__(NTH) mlp_backward_kernel(const float* __restrict__ params, const float* __restrict__ X,
-                                                           const float* __restrict__ T, const int* __restrict__ idx, int B,
-                                                           const float* __restrict__ Y, const float* __restrict__ Z,
-                                                           float* __restrict__ gp) {
-    extern __shared__ __align__(16) float smem[];
-    float* Ws = smem;               // [H][H] weights (plain layout)
-    float* dZ = smem + H * H;       // [TILE][H]
-    float* A = dZ + TILE * H;       // [TILE][H] activations of the layer below
-    __shared__ float dY[TILE][O];
-    const int e = blockIdx.y, tile = blockIdx.x, s0 = tile * TILE, ntile = gridDim.x;
-    const float* p = params + (size_t)e * PS;
-    float* g = gp + ((size_t)e * ntile + tile) * P;
-    const float* Z1 = Z + ((size_t)e * 3 + 0) * B * H;
-    const float* Z2 = Z + ((size_t)e * 3 + 1) * B * H;
-    const float* Z3 = Z + ((size_t)e * 3 + 2) * B * H;
-    const float scale = 2.0f / (float)(B * O);
-    if (threadIdx.x < TILE * O) {
-        const int s = threadIdx.x / O, o = threadIdx.x % O, b = s0 + s;
-        float d = 0.0f;
-        if (b < B) {
-            const int row = idx ? idx[b] : b;
-            d = scale * (Y[((size_t)e * B + b) * O + o] - __ldg(T + (size_t)row * O + o));
-        }
-        dY[s][o] = d;
-    }
-    // A <- A3 = gelu(Z3)
-    for (int q = threadIdx.x; q < TILE * H; q += NTH) {
-        const int s = q / H, j = q % H, b = s0 + s;
-        A[q] = b < B ? gelu(Z3[(size_t)b * H + j]) : 0.0f;
-    }
-    __syncthreads();
-    // output layer: dW4, db4 and dZ3 = (dY W4) * gelu'(Z3)
-    for (int q = threadIdx.x; q < O * H; q += NTH) {
-        const int o = q / H, k = q % H;
-        float acc = 0.0f;
-        for (int s = 0; s < TILE; ++s) acc = fmaf(dY[s][o], A[s * H + k], acc);
-        g[oW4 + q] = acc;
-    }
-    if (threadIdx.x < O) {
-        float acc = 0.0f;
-        for (int s = 0; s < TILE; ++s) acc += dY[s][threadIdx.x];
-        g[ob4 + threadIdx.x] = acc;
-    }
-    for (int q = threadIdx.x; q < TILE * H; q += NTH) {
-        const int s = q / H, k = q % H, b = s0 + s;
-        const float da = dY[s][0] * __ldg(p + oW4 + k) + dY[s][1] * __ldg(p + oW4 + H + k);
-        dZ[q] = b < B ? da * gelu_grad(Z3[(size_t)b * H + k]) : 0.0f;
-    }
-    __syncthreads();
-    // hidden layers 3 and 2: dW = dZ^T A (A = gelu of the layer below), db,
-    // then dZ_below = (dZ W) * gelu'(Z_below)
+    for (int step = 0; step < a.nsteps; ++step) {
+        float dw2[8][4] = {}, dw3[8][4] = {};
+        float dw1 = 0.f, dw4 = 0.f, db1v = 0.f, db2v = 0.f, db3v = 0.f, db4v = 0.f;
 #pragma unroll 1
-    for (int l = 0; l < 2; ++l) {
-        const int oW = l == 0 ? oW3 : oW2, ob = l == 0 ? ob3 : ob2;
-        const float* Zb = l == 0 ? Z2 : Z1;
-        for (int q = threadIdx.x; q < TILE * H; q += NTH) {
-            const int s = q / H, j = q % H, b = s0 + s;
-            A[q] = b < B ? gelu(Zb[(size_t)b * H + j]) : 0.0f;
-        }
-        stage_plain(Ws, p + oW);
-        __syncthreads();
-        {
-            // dW[j][k] = sum_s dZ[s][j] A[s][k]: thread -> 8 j x 8 k
-            const int jg = threadIdx.x / 16, kg = threadIdx.x % 16;
-            float acc[8][8];
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[a][c] = 0.0f;
-            for (int s = 0; s < TILE; ++s) {
-                const float4 z0 = reinterpret_cast<const float4*>(dZ + s * H + 8 * jg)[0];
-                const float4 z1 = reinterpret_cast<const float4*>(dZ + s * H + 8 * jg)[1];
-                const float4 a0 = reinterpret_cast<const float4*>(A + s * H + 8 * kg)[0];
-                const float4 a1 = reinterpret_cast<const float4*>(A + s * H + 8 * kg)[1];
-                const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
-                const float aa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-#pragma unroll
-                for (int a = 0; a < 8; ++a)
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) acc[a][c] = fmaf(zz[a], aa[c], acc[a][c]);
+        for (int ch = 0; ch < nch; ++ch) {
+            const float* x = xs + buf * TS * I;
+            float4 nx_;
+            float2 nt;
+            if (tid < TS) {
+                fetch(row_next, nx_, nt);
+                row_next = lookup();
             }
+            const int live = r1 - (r0 + ch * TS);  // samples of this chunk that exist
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+            for (int o = tid; o < TS * H; o += TT) {
+                const int s = o / H, j = o % H;
+                const float z = dot4(*reinterpret_cast<const float4*>(x + s * I),
+                                     *reinterpret_cast<const float4*>(img + iW1 + j * I), img[ib1 + j]);
+                gelu_both(z, A1[o], D1[o]);
+            }
+            __syncthreads();
+            train_gemm_nt<TS>(img + iW2, A1, part);
+            __syncthreads();
 #pragma unroll
-                for (int c = 0; c < 8; ++c) g[oW + (8 * jg + a) * H + 8 * kg + c] = acc[a][c];
-        }
-        if (threadIdx.x < H) {
-            float acc = 0.0f;
-            for (int s = 0; s < TILE; ++s) acc += dZ[s * H + threadIdx.x];
-            g[ob + threadIdx.x] = acc;
-        }
-        // dA[s][k] = sum_j dZ[s][j] W[j][k]  (W plain: row j contiguous over k)
-        float acc[4][4];
-        tile_gemm(dZ, Ws, nullptr, acc);
-        __syncthreads();  // everyone is done reading dZ
-        {
-            const int sg = threadIdx.x / 32, ng = threadIdx.x % 32;
+            for (int o = tid; o < TS * H; o += TT) gelu_both(train_fold<TS>(part, o) + img[ib2 + o % H], A2[o], D2[o]);
+            __syncthreads();
+            train_gemm_nt<TS>(img + iW3, A2, part);
+            __syncthreads();
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int s = 4 * sg + r, b = s0 + s;
+            for (int o = tid; o < TS * H; o += TT) gelu_both(train_fold<TS>(part, o) + img[ib3 + o % H], A3[o], D3[o]);
+            __syncthreads();
+            // output layer and dZ3: one warp per sample
+            if (w < TS) {
+                const float4 av = *reinterpret_cast<const float4*>(A3 + w * H + 4 * lane);
+                const float4 u0 = *reinterpret_cast<const float4*>(img + iW4 + 4 * lane);
+                const float4 u1 = *reinterpret_cast<const float4*>(img + iW4 + H + 4 * lane);
+                float y0 = dot4(av, u0, 0.f), y1 = dot4(av, u1, 0.f);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int k = 4 * ng + c;
-                    dZ[s * H + k] = b < B ? acc[r][c] * gelu_grad(Zb[(size_t)b * H + k]) : 0.0f;
+                for (int o = 16; o > 0; o >>= 1) {
+                    y0 += __shfl_xor_sync(0xffffffffu, y0, o);
+                    y1 += __shfl_xor_sync(0xffffffffu, y1, o);
                 }
+                const float* t = ts + (buf * TS + w) * O;
+                const bool in = w < live;
+                const float d0 = in ? scale * (y0 + img[ib4] - t[0]) : 0.f;
+                const float d1 = in ? scale * (y1 + img[ib4 + 1] - t[1]) : 0.f;
+                if (lane == 0) {
+                    dY[w * O] = d0;
+                    dY[w * O + 1] = d1;
+                }
+                float4* dz = reinterpret_cast<float4*>(D3 + w * H + 4 * lane);
+                const float4 gv = *dz;
+                *dz = in ? make_float4((d0 * u0.x + d1 * u1.x) * gv.x, (d0 * u0.y + d1 * u1.y) * gv.y,
+                                       (d0 * u0.z + d1 * u1.z) * gv.z, (d0 * u0.w + d1 * u1.w) * gv.w)
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
             }
+            __syncthreads();
+            train_gemm_nn<TS>(img + iW3, D3, part);
+            train_outer<TS>(D3, A2, dw3);
+            if (tid < O * H) {
+#pragma unroll
+                for (int s = 0; s < TS; ++s) dw4 = fmaf(dY[s * O + tid / H], A3[s * H + tid % H], dw4);
+            } else if (tid < O * H + H) {
+                db3v += train_column_sum<TS>(D3, tid - O * H);
+            } else if (tid < O * H + H + O) {
+#pragma unroll
+                for (int s = 0; s < TS; ++s) db4v += dY[s * O + tid - O * H - H];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int o = tid; o < TS * H; o += TT) D2[o] = o / H < live ? train_fold<TS>(part, o) * D2[o] : 0.f;
+            __syncthreads();
+            train_gemm_nn<TS>(img + iW2, D2, part);
+            train_outer<TS>(D2, A1, dw2);
+            if (tid < H) db2v += train_column_sum<TS>(D2, tid);
+            __syncthreads();
+#pragma unroll
+            for (int o = tid; o < TS * H; o += TT) D1[o] = o / H < live ? train_fold<TS>(part, o) * D1[o] : 0.f;
+            __syncthreads();
+            {
+                const int j = tid / I, i = tid % I;
+#pragma unroll
+                for (int s = 0; s < TS; ++s) dw1 = fmaf(D1[s * H + j], x[s * I + i], dw1);
+            }
+            if (tid < H) db1v += train_column_sum<TS>(D1, tid);
+            buf ^= 1;
+            if (tid < TS) put(buf, nx_, nt);
+            __syncthreads();
         }
+        // this CTA's partial gradient, in the order of the parameter image
+        float* gp = a.part + (size_t)((e * gridDim.y + blockIdx.y) * CL + rank) * IMG;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            __stcg(reinterpret_cast<float4*>(gp + iW2 + (8 * w + r) * WS + 4 * lane),
+                   make_float4(dw2[r][0], dw2[r][1], dw2[r][2], dw2[r][3]));
+            __stcg(reinterpret_cast<float4*>(gp + iW3 + (8 * w + r) * WS + 4 * lane),
+                   make_float4(dw3[r][0], dw3[r][1], dw3[r][2], dw3[r][3]));
+        }
+        gp[iW1 + tid] = dw1;
+        if (tid < O * H) gp[iW4 + tid] = dw4;
+        else if (tid < O * H + H) gp[ib3 + tid - O * H] = db3v;
+        else if (tid < O * H + H + O) gp[ib4 + tid - O * H - H] = db4v;
+        if (tid < H) {
+            gp[ib1 + tid] = db1v;
+            gp[ib2 + tid] = db2v;
+        }
+        cluster.sync();
+        // slice of this rank: partials summed in rank order, Adam
+        constexpr int PER = (IMG / 4 + CL - 1) / CL;
+        const float* g0 = a.part + (size_t)((e * gridDim.y + blockIdx.y) * CL) * IMG;
+        const float2 cf = a.out ? make_float2(1.f, 1.f) : a.coef[step];
+#pragma unroll 1
+        for (int i = tid; i < PER; i += TT) {
+            const int q = rank * PER + i, o = q < IMG / 4 ? img_param(q) : -1;
+            if (o < 0) continue;
+            const size_t n = (size_t)e * PS + o;
+            float4 t[CL], wv, mv, vv;
+#pragma unroll
+            for (int c = 0; c < CL; ++c) t[c] = __ldcg(reinterpret_cast<const float4*>(g0 + (size_t)c * IMG) + q);
+            if (!a.out) {
+                wv = *reinterpret_cast<const float4*>(a.params + n);
+                mv = *reinterpret_cast<const float4*>(a.m + n);
+                vv = *reinterpret_cast<const float4*>(a.v + n);
+            }
+            float4 g = t[0];
+#pragma unroll
+            for (int c = 1; c < CL; ++c) {
+                g.x += t[c].x;
+                g.y += t[c].y;
+                g.z += t[c].z;
+                g.w += t[c].w;
+            }
+            if (a.out) {
+                float* go = a.out + ((size_t)e * gridDim.y + blockIdx.y) * P + o;
+                const float gv[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (o + k < P) go[k] = gv[k];
+                continue;
+            }
+            adam_update(wv.x, mv.x, vv.x, g.x, a.lr, a.b1, a.b2, cf.x, cf.y, a.eps);
+            adam_update(wv.y, mv.y, vv.y, g.y, a.lr, a.b1, a.b2, cf.x, cf.y, a.eps);
+            adam_update(wv.z, mv.z, vv.z, g.z, a.lr, a.b1, a.b2, cf.x, cf.y, a.eps);
+            adam_update(wv.w, mv.w, vv.w, g.w, a.lr, a.b1, a.b2, cf.x, cf.y, a.eps);
+            __stcg(reinterpret_cast<float4*>(a.params + n), wv);
+            *reinterpret_cast<float4*>(a.m + n) = mv;
+            *reinterpret_cast<float4*>(a.v + n) = vv;
+        }
+        if (step + 1 == a.nsteps) break;
+        cluster.sync();
+        load_image(img, p);
         __syncthreads();
-    }
-    // first layer: dW1[j][i] = sum_s dZ1[s][j] x[s][i], db1
-    for (int q = threadIdx.x; q < H * I; q += NTH) {
-        const int j = q / I, i = q % I;
-        float acc = 0.0f;
-        for (int s = 0; s < TILE; ++s) {
-            const int b = s0 + s;
-            if (b < B) acc = fmaf(dZ[s * H + j], __ldg(X + (size_t)(idx ? idx[b] : b) * I + i), acc);
-        }
-        g[oW1 + q] = acc;
-    }
-    if (threadIdx.x < H) {
-        float acc = 0.0f;
-        for (int s = 0; s < TILE; ++s) acc += dZ[s * H + threadIdx.x];
-        g[ob1 + threadIdx.x] = acc;
     }
 }
 
-// Sum of the tiles' partials in tile order -> gradient (and optional Adam).
+// Sum of the clusters' gradient partials gp [E][np][P] in cluster order ->
+// gradient (grad_out) or an Adam update.
 __global__ void __launch_bounds__(256) mlp_adam_kernel(float* __restrict__ params, float* __restrict__ m,
-                                                       float* __restrict__ v, const float* __restrict__ gp, int ntile,
+                                                       float* __restrict__ v, const float* __restrict__ gp, int np,
                                                        float lr, float b1, float b2, float c1, float c2, float eps,
-                                                       int adam, float* __restrict__ grad_out) {
+                                                       float* __restrict__ grad_out) {
     const int e = blockIdx.y;
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= P) return;
     float g = 0.0f;
-    for (int t = 0; t < ntile; ++t) g += gp[((size_t)e * ntile + t) * P + q];
+    for (int t = 0; t < np; ++t) g += gp[((size_t)e * np + t) * P + q];
+    if (grad_out) {
+        grad_out[(size_t)e * P + q] = g;
+        return;
+    }
     const size_t n = (size_t)e * PS + q;
-    if (grad_out) grad_out[(size_t)e * P + q] = g;
-    if (!adam) return;
-    const float mm = b1 * m[n] + (1.0f - b1) * g;
-    const float vv = b2 * v[n] + (1.0f - b2) * g * g;
-    m[n] = mm;
-    v[n] = vv;
-    params[n] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+    adam_update(params[n], m[n], v[n], g, lr, b1, b2, c1, c2, eps);
 }
 
 // ---- inference kernel: 128 samples per CTA, 8x8 register tiles -----------
@@ -744,6 +893,7 @@ struct lbm_mlp {
     unsigned* status = nullptr;      // device status word of the tensor-core inference
     int infer_path = LBM_MLP_INFER_TENSOR;
     int sms = 1;  // SMs of the device (persistent tensor-core grid)
+    int clusters8 = 0, clusters16 = 0;  // training clusters of 8 / 16 CTAs that fit on the device at once
     long long wait_limit = TC_WAIT_LIMIT;  // SM cycles a tensor-core wait may take
     void* ws = nullptr;       // grow-only device workspace of the per-call buffers
     size_t ws_bytes = 0;
@@ -764,22 +914,26 @@ lbm_status mfail(lbm_mlp* m, lbm_status st, const std::string& msg) {
         if (e_ != cudaSuccess) return mfail(mm, LBM_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+template <int TS, int CL>
+cudaError_t train_attr() {
+    cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel<TS, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)TrainSmem<TS>::BYTES);
+    if (e == cudaSuccess && CL > 8)
+        e = cudaFuncSetAttribute(mlp_train_kernel<TS, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
 std::once_flag g_attr_once;
 cudaError_t g_attr_err = cudaSuccess;
 
 cudaError_t set_smem_attrs() {
     std::call_once(g_attr_once, [] {
-        g_attr_err = cudaFuncSetAttribute(mlp_forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)SMEM_BYTES);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(mlp_forward_kernel<false>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+        for (cudaError_t e : {train_attr<4, 8>(), train_attr<8, 8>(), train_attr<16, 8>(), train_attr<4, 16>(),
+                              train_attr<8, 16>(), train_attr<16, 16>()})
+            if (g_attr_err == cudaSuccess) g_attr_err = e;
         if (g_attr_err == cudaSuccess)
             g_attr_err = cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)SMEM_BIG);
-        if (g_attr_err == cudaSuccess)
-            g_attr_err = cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)SMEM_BYTES);
         if (g_attr_err == cudaSuccess)
             g_attr_err = cudaFuncSetAttribute(mlp_infer_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)TC_SMEM);
@@ -790,14 +944,15 @@ cudaError_t set_smem_attrs() {
 // Per-call device buffers, carved out of the ensemble's workspace (grown, never
 // shrunk; reallocated only after the stream has drained).
 struct Scratch {
-    float *X = nullptr, *T = nullptr, *Y = nullptr, *Z = nullptr, *gp = nullptr, *grad = nullptr;
+    float *X = nullptr, *T = nullptr, *Y = nullptr, *gp = nullptr, *grad = nullptr;
+    float2* coef = nullptr;
     int* idx = nullptr;
 };
 
-// Element counts of X, T, Y, Z, gp, grad (floats) and idx (ints).
-lbm_status carve(lbm_mlp* mm, Scratch& s, size_t nX, size_t nT, size_t nY, size_t nZ, size_t ngp, size_t ngrad,
+// Element counts of X, T, Y, gp, grad (floats), coef (pairs) and idx (ints).
+lbm_status carve(lbm_mlp* mm, Scratch& s, size_t nX, size_t nT, size_t nY, size_t ngp, size_t ngrad, size_t ncoef,
                  size_t nidx) {
-    const size_t cnt[7] = {nX, nT, nY, nZ, ngp, ngrad, nidx};
+    const size_t cnt[7] = {nX, nT, nY, ngp, ngrad, 2 * ncoef, nidx};
     size_t off[7], total = 0;
     for (int k = 0; k < 7; ++k) {
         off[k] = total;
@@ -818,8 +973,9 @@ lbm_status carve(lbm_mlp* mm, Scratch& s, size_t nX, size_t nT, size_t nY, size_
         mm->ws_bytes = want;
     }
     char* b = static_cast<char*>(mm->ws);
-    float** fp[6] = {&s.X, &s.T, &s.Y, &s.Z, &s.gp, &s.grad};
-    for (int k = 0; k < 6; ++k) *fp[k] = cnt[k] ? reinterpret_cast<float*>(b + off[k]) : nullptr;
+    float** fp[5] = {&s.X, &s.T, &s.Y, &s.gp, &s.grad};
+    for (int k = 0; k < 5; ++k) *fp[k] = cnt[k] ? reinterpret_cast<float*>(b + off[k]) : nullptr;
+    s.coef = cnt[5] ? reinterpret_cast<float2*>(b + off[5]) : nullptr;
     s.idx = cnt[6] ? reinterpret_cast<int*>(b + off[6]) : nullptr;
     return LBM_OK;
 }
@@ -830,24 +986,77 @@ lbm_status carve(lbm_mlp* mm, Scratch& s, size_t nX, size_t nT, size_t nY, size_
         if (cs_ != LBM_OK) return cs_;               \
     } while (0)
 
-// One training (or gradient-only) step on rows idx[0..B) of the device data.
-lbm_status run_step(lbm_mlp* mm, Scratch& s, int B, const int* idx, bool adam, double lr, float* grad_out) {
-    const int ntile = (B + TILE - 1) / TILE;
-    const dim3 grid(ntile, mm->E);
-    mlp_forward_kernel<true><<<grid, NTH, SMEM_BYTES, mm->stream>>>(mm->params, s.X, idx, B, s.Y, s.Z);
-    MCK(cudaGetLastError());
-    mlp_backward_kernel<<<grid, NTH, SMEM_BYTES, mm->stream>>>(mm->params, s.X, s.T, idx, B, s.Y, s.Z, s.gp);
-    MCK(cudaGetLastError());
-    float c1 = 1.0f, c2 = 1.0f;
-    if (adam) {
-        mm->t += 1;
-        c1 = (float)(1.0 - std::pow(0.9, (double)mm->t));
-        c2 = (float)(1.0 - std::pow(0.999, (double)mm->t));
+// How a minibatch of B rows is trained: clusters of `cl` CTAs, `nc` of them per
+// member, chunks of `ts` samples.
+struct TrainPlan {
+    int cl, nc, ts;
+};
+
+// The plan with the smallest estimated step: waves of clusters times (a fixed
+// 11 us for the exchange and barriers, plus the chunks: 4 us for up to four
+// rows per CTA, 7.5 us for up to eight, 16 us for each sixteen), plus 10 us for
+// the second launch when several clusters share a member.  Measured on GB300
+// for 1 to 8 members and minibatches of 16 to 4096: the choice is within a few
+// percent of the best plan tried (e.g. 5 members: minibatch 64 16x1 15 us, 8x1
+// 19 us; 4096 8x3 206 us, 16x1 277 us, 8x1 516 us; 8 members, minibatch 64: 8x1
+// 19 us, 16x1, of which 7 clusters fit, 31 us).
+TrainPlan train_plan(const lbm_mlp* mm, int B) {
+    TrainPlan best{8, 1, 16};
+    double best_us = 1e300;
+    for (int cl : {8, 16}) {
+        const int fit = cl == 16 ? mm->clusters16 : mm->clusters8;
+        if (cl == 16 && fit < 1) continue;
+        for (int nc = 1; nc == 1 || nc * mm->E <= fit; ++nc) {
+            const int rows = (B + cl * nc - 1) / (cl * nc), waves = (mm->E * nc + std::max(1, fit) - 1) / std::max(1, fit);
+            const double chunks = rows <= 4 ? 4.0 : (rows <= 8 ? 7.5 : 16.0 * ((rows + 15) / 16));
+            const double us = waves * (11.0 + chunks) + (nc > 1 ? 10.0 : 0.0);
+            if (us < best_us) {
+                best_us = us;
+                best = {cl, nc, rows <= 4 ? 4 : (rows <= 8 ? 8 : 16)};
+            }
+        }
     }
-    mlp_adam_kernel<<<dim3((P + 255) / 256, mm->E), 256, 0, mm->stream>>>(
-        mm->params, mm->m, mm->v, s.gp, ntile, (float)lr, 0.9f, 0.999f, c1, c2, 1e-8f, adam ? 1 : 0, grad_out);
-    MCK(cudaGetLastError());
-    return LBM_OK;
+    return best;
+}
+
+template <int TS, int CL>
+cudaError_t launch_train(const TrainArgs& a, int nc, int E, cudaStream_t st, int* max_clusters = nullptr) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)CL, (unsigned)nc, (unsigned)E);
+    cfg.blockDim = dim3(TT);
+    cfg.dynamicSmemBytes = TrainSmem<TS>::BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)CL, 1, 1};
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, mlp_train_kernel<TS, CL>, &cfg);
+    return cudaLaunchKernelEx(&cfg, mlp_train_kernel<TS, CL>, a);
+}
+
+template <int CL>
+cudaError_t launch_train_cl(const TrainArgs& a, const TrainPlan& p, int E, cudaStream_t st) {
+    return p.ts == 4   ? launch_train<4, CL>(a, p.nc, E, st)
+           : p.ts == 8 ? launch_train<8, CL>(a, p.nc, E, st)
+                       : launch_train<16, CL>(a, p.nc, E, st);
+}
+
+cudaError_t run_train(const TrainArgs& a, const TrainPlan& p, int E, cudaStream_t st) {
+    return p.cl == 16 ? launch_train_cl<16>(a, p, E, st) : launch_train_cl<8>(a, p, E, st);
+}
+
+// Gradient exchange of a plan: the CTAs' partials, then (several clusters per
+// member) the clusters' sums.
+size_t part_floats(const lbm_mlp* mm, const TrainPlan& p) {
+    return (size_t)mm->E * p.nc * p.cl * IMG + (p.nc > 1 ? (size_t)mm->E * p.nc * P : 0);
+}
+float* cluster_sums(const lbm_mlp* mm, const TrainPlan& p, float* gp) { return gp + (size_t)mm->E * p.nc * p.cl * IMG; }
+
+constexpr float kBeta1 = 0.9f, kBeta2 = 0.999f, kEps = 1e-8f;
+
+float2 adam_coef(int64_t t) {
+    return make_float2((float)(1.0 - std::pow(0.9, (double)t)), (float)(1.0 - std::pow(0.999, (double)t)));
 }
 
 // Refresh the k-major copy of the hidden weights after any parameter change.
@@ -905,6 +1114,14 @@ lbm_status lbm_mlp_create(int members, uint64_t seed, void* cuda_stream, lbm_mlp
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&mm->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = launch_train<16, 8>(TrainArgs{}, 1, members, mm->stream, &mm->clusters8);
+    if (e == cudaSuccess) {
+        // 16 CTAs exceed the portable cluster size: a device may refuse them
+        if (launch_train<16, 16>(TrainArgs{}, 1, members, mm->stream, &mm->clusters16) != cudaSuccess) {
+            cudaGetLastError();
+            mm->clusters16 = 0;
+        }
+    }
     const size_t bytes = (size_t)members * PS * sizeof(float);
     if (e == cudaSuccess) e = cudaMalloc((void**)&mm->params, bytes);
     if (e == cudaSuccess) e = cudaMalloc((void**)&mm->m, bytes);
@@ -984,14 +1201,19 @@ lbm_status lbm_mlp_forward(lbm_mlp* mm, const float* X, int n, float* Y) {
 
 lbm_status lbm_mlp_gradient(lbm_mlp* mm, const float* X, const float* T, int n, float* grad) {
     if (!mm || !X || !T || !grad || n < 1) return mfail(mm, LBM_ERR_INVALID_ARG, "bad gradient request");
+    const TrainPlan p = train_plan(mm, n);
     Scratch s;
-    const int ntile = (n + TILE - 1) / TILE;
-    CARVE((size_t)n * I, (size_t)n * O, (size_t)mm->E * n * O, (size_t)mm->E * 3 * n * H,
-          (size_t)mm->E * ntile * P, (size_t)mm->E * P, 0);
+    CARVE((size_t)n * I, (size_t)n * O, 0, part_floats(mm, p), (size_t)mm->E * P, 0, 0);
     MCK(cudaMemcpyAsync(s.X, X, (size_t)n * I * sizeof(float), cudaMemcpyHostToDevice, mm->stream));
     MCK(cudaMemcpyAsync(s.T, T, (size_t)n * O * sizeof(float), cudaMemcpyHostToDevice, mm->stream));
-    lbm_status st = run_step(mm, s, n, nullptr, false, 0.0, s.grad);
-    if (st != LBM_OK) return st;
+    TrainArgs a{mm->params, mm->m, mm->v, s.X, s.T, nullptr, nullptr, s.gp, p.nc > 1 ? cluster_sums(mm, p, s.gp) : s.grad,
+                n, 1, n, 1, 0.f, kBeta1, kBeta2, kEps};
+    MCK(run_train(a, p, mm->E, mm->stream));
+    if (p.nc > 1) {
+        mlp_adam_kernel<<<dim3((P + 255) / 256, mm->E), 256, 0, mm->stream>>>(
+            mm->params, mm->m, mm->v, a.out, p.nc, 0.f, kBeta1, kBeta2, 1.f, 1.f, kEps, s.grad);
+        MCK(cudaGetLastError());
+    }
     MCK(cudaMemcpyAsync(grad, s.grad, (size_t)mm->E * P * sizeof(float), cudaMemcpyDeviceToHost, mm->stream));
     MCK(cudaStreamSynchronize(mm->stream));
     return LBM_OK;
@@ -1002,26 +1224,57 @@ lbm_status lbm_mlp_train(lbm_mlp* mm, const float* X, const float* T, int n, int
     if (!mm || !X || !T || n < 1 || epochs < 0 || batch < 1 || !(lr > 0.0))
         return mfail(mm, LBM_ERR_INVALID_ARG, "bad training request");
     batch = std::min(batch, n);
+    const TrainPlan p = train_plan(mm, batch);
+    const int spe = n / batch;  // steps per epoch (a ragged tail is dropped)
+    // epochs per launch: as many as about a megabyte of row order holds
+    const int group = (int)std::max<int64_t>(1, std::min<int64_t>(epochs, (1 << 18) / n));
     Scratch s;
-    const int ntile = (batch + TILE - 1) / TILE;
-    CARVE((size_t)n * I, (size_t)n * O, (size_t)mm->E * batch * O, (size_t)mm->E * 3 * batch * H,
-          (size_t)mm->E * ntile * P, 0, (size_t)n);
+    CARVE((size_t)n * I, (size_t)n * O, 0, part_floats(mm, p), 0, (size_t)group * spe, (size_t)group * n);
     MCK(cudaMemcpyAsync(s.X, X, (size_t)n * I * sizeof(float), cudaMemcpyHostToDevice, mm->stream));
     MCK(cudaMemcpyAsync(s.T, T, (size_t)n * O * sizeof(float), cudaMemcpyHostToDevice, mm->stream));
-    std::vector<int> perm(n);
+    // two host buffers: a group is drawn while the previous one's upload and
+    // training may still be running
+    std::vector<int> order[2];
+    std::vector<float2> coefs[2];
+    for (int b = 0; b < (group < epochs ? 2 : 1); ++b) {
+        order[b].resize((size_t)group * n);
+        coefs[b].resize((size_t)group * spe);
+    }
     uint64_t rs = shuffle_seed;
-    for (int ep = 0; ep < epochs; ++ep) {
-        for (int i = 0; i < n; ++i) perm[i] = i;
-        for (int i = n - 1; i > 0; --i) {  // Fisher-Yates with splitmix64
-            const int j = (int)(splitmix64(rs) % (uint64_t)(i + 1));
-            std::swap(perm[i], perm[j]);
+    for (int ep = 0; ep < epochs; ep += group) {
+        std::vector<int>& perm = order[(ep / group) & 1];
+        std::vector<float2>& coef = coefs[(ep / group) & 1];
+        const int ne = std::min(group, epochs - ep);
+        for (int g = 0; g < ne; ++g) {
+            int* q = perm.data() + (size_t)g * n;
+            for (int i = 0; i < n; ++i) q[i] = i;
+            for (int i = n - 1; i > 0; --i) {  // Fisher-Yates with splitmix64
+                const int j = (int)(splitmix64(rs) % (uint64_t)(i + 1));
+                std::swap(q[i], q[j]);
+            }
         }
-        MCK(cudaStreamSynchronize(mm->stream));  // the previous epoch's kernels read s.idx
-        MCK(cudaMemcpy(s.idx, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice));
-        for (int b0 = 0; b0 + batch <= n; b0 += batch) {
-            lbm_status st = run_step(mm, s, batch, s.idx + b0, true, lr, nullptr);
-            if (st != LBM_OK) return st;
+        const int steps = ne * spe;
+        for (int i = 0; i < steps; ++i) coef[i] = adam_coef(mm->t + 1 + i);
+        MCK(cudaStreamSynchronize(mm->stream));  // the previous group reads s.idx and s.coef
+        MCK(cudaMemcpyAsync(s.idx, perm.data(), (size_t)ne * n * sizeof(int), cudaMemcpyHostToDevice, mm->stream));
+        MCK(cudaMemcpyAsync(s.coef, coef.data(), (size_t)steps * sizeof(float2), cudaMemcpyHostToDevice, mm->stream));
+        TrainArgs a{mm->params, mm->m, mm->v, s.X, s.T, s.idx, s.coef, s.gp, nullptr,
+                    batch, steps, n, spe, (float)lr, kBeta1, kBeta2, kEps};
+        if (p.nc == 1) {
+            MCK(run_train(a, p, mm->E, mm->stream));
+        } else {
+            a.out = cluster_sums(mm, p, s.gp);
+            a.nsteps = 1;
+            for (int i = 0; i < steps; ++i) {
+                a.idx = s.idx + (size_t)(i / spe) * n + (size_t)(i % spe) * batch;
+                MCK(run_train(a, p, mm->E, mm->stream));
+                mlp_adam_kernel<<<dim3((P + 255) / 256, mm->E), 256, 0, mm->stream>>>(
+                    mm->params, mm->m, mm->v, a.out, p.nc, (float)lr, kBeta1, kBeta2, coef[i].x, coef[i].y, kEps,
+                    nullptr);
+                MCK(cudaGetLastError());
+            }
         }
+        mm->t += steps;
     }
     lbm_status st = refresh_wt(mm);
     if (st != LBM_OK) return st;
@@ -1033,7 +1286,7 @@ lbm_status lbm_mlp_predict(lbm_mlp* mm, const float* X, int n, float* mean, floa
     if (!mm || !X || !mean || !spread || n < 1) return mfail(mm, LBM_ERR_INVALID_ARG, "bad predict request");
     Scratch s;
     const size_t hn = dst_is_device ? 0 : (size_t)n;
-    CARVE(hn * I, hn * O, (size_t)mm->E * n * O, 0, 0, hn, 0);
+    CARVE(hn * I, hn * O, (size_t)mm->E * n * O, 0, hn, 0, 0);
     const float* dX = X;
     float *dm = mean, *ds = spread;
     if (!dst_is_device) {
