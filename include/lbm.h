@@ -168,7 +168,7 @@ lbm_status lbm_reset(lbm_ctx* ctx, const double* rho_init, const double* u_init)
  * face) and one for the other tiles, plus one for the column-marching runs
  * under tile variant 4 (FP32); the persistent schedule runs up to 1024
  * steps per launch.  D3Q19: five launches per step (pulls, face pulls,
- * collision, outlet, reduction).  Returns without waiting for the GPU;
+ * collision, outlet, reduction), runs of 16 steps replayed from graphs.  Returns without waiting for the GPU;
  * launch errors are reported at once, divergence (LBM_ERR_DIVERGED) or a
  * bounded device wait that ran out (LBM_ERR_TIMEOUT) by the next call that
  * synchronises (lbm_sync, lbm_get_*). */

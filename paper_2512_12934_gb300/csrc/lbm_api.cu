@@ -1993,7 +1993,7 @@ lbm_status lbm_tile_stats(lbm_ctx* c, int* variant, int* fast_tiles, int* genera
 
 lbm_status lbm_set_graph_mode(lbm_ctx* c, int use_graphs) {
     if (!c) return fail(nullptr, LBM_ERR_INVALID_ARG, "ctx is NULL");
-    if (c->d3) return LBM_OK;  // D3Q19 steps are plain launches
+    if (c->d3) return lbm3::set_graphs(c->d3, use_graphs);
     c->use_graphs = use_graphs ? 1 : 0;
     return LBM_OK;
 }

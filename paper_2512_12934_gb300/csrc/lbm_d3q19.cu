@@ -1,7 +1,8 @@
 // D3Q19 two-component MRT pseudopotential step with the corrected open faces
 // (the three-dimensional counterpart of lbm_d2q9.cu).
 //
-// One time step is five launches on the context's stream:
+// One time step is five launches (plain, or replayed from graphs in two
+// branches: launch_step_forked):
 //   A  d3q_pull_kernel      pull streaming (Eq. 2) with halfway bounce-back
 //                           (Eq. B1) and periodic wrap (Eq. B2) of interior
 //                           nodes; component densities rho_k (= psi_k) to a
@@ -10,8 +11,8 @@
 //                           then inlet reconstruction (Eq. 13 over the 5
 //                           unknowns, alpha correction Eqs. 15-19) or the
 //                           convective outlet (Eq. 20); densities.
-//   B  d3q_collide_kernel   rho and the solid indicator of a 32x4xTZ tile plus
-//                           a 2-node halo (ghost mirrors of Eqs. 24-25) staged
+//   B  d3q_collide_kernel   (FP32: d3q_collide_f32_kernel) rho of a 32x4x2 tile
+//                           plus a 2-node halo (ghost mirrors of Eqs. 24-25) staged
 //                           in shared memory; forces of Eqs. 10-11 on the
 //                           92-vector 8th-order isotropic stencil; common
 //                           velocity (Eqs. 7-8); MRT collision with forcing
@@ -116,14 +117,12 @@ __device__ __forceinline__ void acc_c(R& acc, R v) {
 }
 
 // ---- tiles of the collide kernel -----------------------------------------
-// Tiles are TX x TY x TZ nodes; FP32 storage takes TZ = 4 (512 threads, two
-// CTAs per SM: a staged halo of 4.5 sites per node instead of 6.75), the
-// others TZ = 2 (FP64 needs 140 registers a thread, FP16 storage 80).
+// Tiles are TX x TY x TZ nodes of one thread each.
 constexpr int TX = 32, TY = 4;
 constexpr int HX = TX + 4, HY = TY + 4;
 template <typename S>
 struct Tile3 {
-    static constexpr int TZ = std::is_same<S, float>::value ? 4 : 2;
+    static constexpr int TZ = 2;
     static constexpr int HZ = TZ + 4;
     static constexpr int HN = HX * HY * HZ;
     static constexpr int NT = TX * TY * TZ;
@@ -181,52 +180,68 @@ __device__ __forceinline__ long long node_index(const D3Args<S>& a, int x, int y
     return ((long long)z * a.ny + y) * a.pitch + x;
 }
 
-// Pull the 19 populations of component k at (x, y, z) (Eq. 2, Eq. B1, Eq. B2).
-// Away from periodic edges the source of direction i is n minus a fixed
-// offset (e_x + e_y pitch + e_z ny pitch); across an edge it is wrapped.
-template <typename S, typename R, bool FAST = true>
+template <typename S>
+__device__ __forceinline__ void st_at(S* base, unsigned off, S v) {
+    *reinterpret_cast<S*>(reinterpret_cast<char*>(base) + off) = v;
+}
+
+// One stored population at a uniform base plus the thread's byte offset.
+template <typename S>
+__device__ __forceinline__ S ld_at(const S* base, unsigned off) {
+    return __ldg(reinterpret_cast<const S*>(reinterpret_cast<const char*>(base) + off));
+}
+
+// Raw pull of the 19 populations of component k at node n = (x, y, z) (Eq. 2,
+// Eq. B1, Eq. B2).  Most nodes have no blocked direction and no wrap: straight
+// loads from the shifted planes.  The others select each source first, so
+// that their 19 loads are in flight together too (a branch per direction made
+// every load wait for the one before it).  The offsets are 32-bit: n * 8 bytes
+// stays below 2^32 for every grid that fits the device.
+template <typename S>
+__device__ __forceinline__ void pull_raw(const D3Args<S>& a, int k, int x, int y, int z, long long n, uint32_t info,
+                                         S (&v)[Q]) {
+    const unsigned off = (unsigned)n * (unsigned)sizeof(S);
+    if ((info & (0x7FFFFu | INFO3_WRAP)) == 0u) {
+        static_for<0, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            v[i] = ld_at(a.src[k][i], off);
+        });
+    } else if (!(info & INFO3_WRAP)) {
+        const S* own = a.fin + (size_t)k * Q * a.plane;
+        static_for<0, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            const S* p = (info & (1u << i)) ? own + (size_t)opp_(i) * a.plane : a.src[k][i];
+            v[i] = ld_at(p, off);
+        });
+    } else {
+        const S* own = a.fin + (size_t)k * Q * a.plane;
+        const int xm = wrap(x - 1, a.nx), xp = wrap(x + 1, a.nx), ym = wrap(y - 1, a.ny), yp = wrap(y + 1, a.ny),
+                  zm = wrap(z - 1, a.nz), zp = wrap(z + 1, a.nz);
+        static_for<0, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            const int xs = ex_(i) == 1 ? xm : (ex_(i) == -1 ? xp : x);
+            const int ys = ey_(i) == 1 ? ym : (ey_(i) == -1 ? yp : y);
+            const int zs = ez_(i) == 1 ? zm : (ez_(i) == -1 ? zp : z);
+            const bool bb = (info & (1u << i)) != 0;
+            const long long m = bb ? n : node_index(a, xs, ys, zs);
+            v[i] = __ldg(own + (size_t)(bb ? opp_(i) : i) * a.plane + m);
+        });
+    }
+}
+
+// Pull of component k as real values.
+template <typename S, typename R>
 __device__ __forceinline__ void pull(const D3Args<S>& a, int k, int x, int y, int z, uint32_t info, R (&f)[Q]) {
-    const S* __restrict__ fin = a.fin + (size_t)k * Q * a.plane;
     const long long n = node_index(a, x, y, z);
-    const long long sy = a.pitch, sz = (long long)a.ny * a.pitch;
-    const bool wrapped = (info & INFO3_WRAP) != 0;
     // FP16 storage: every value this node pulls was encoded against its
     // reference density (the writer used the same half-rounded density)
     R ref = 0;
     if constexpr (is_half<S>()) ref = __half2float(a.rref_in[(size_t)k * a.plane + n]);
-    if (FAST && !wrapped && (info & 0x7FFFFu) == 0u) {
-        // no blocked direction, no wrap (most fluid nodes): straight neighbour loads
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            long long src = n;
-            if constexpr (ex_(i) != 0) src -= ex_(i);
-            if constexpr (ey_(i) == 1) src -= sy;
-            if constexpr (ey_(i) == -1) src += sy;
-            if constexpr (ez_(i) == 1) src -= sz;
-            if constexpr (ez_(i) == -1) src += sz;
-            f[i] = (R)ld_pop(fin[(size_t)i * a.plane + src]);
-            if constexpr (is_half<S>()) f[i] += ((R)w36_(i) / (R)36) * ref;
-        });
-        return;
-    }
+    S v[Q];
+    pull_raw<S>(a, k, x, y, z, n, info, v);
     static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        if (info & (1u << i)) {
-            f[i] = (R)ld_pop(fin[(size_t)opp_(i) * a.plane + n]);
-        } else if (!wrapped) {
-            long long src = n;
-            if constexpr (ex_(i) != 0) src -= ex_(i);
-            if constexpr (ey_(i) == 1) src -= sy;
-            if constexpr (ey_(i) == -1) src += sy;
-            if constexpr (ez_(i) == 1) src -= sz;
-            if constexpr (ez_(i) == -1) src += sz;
-            f[i] = (R)ld_pop(fin[(size_t)i * a.plane + src]);
-        } else {
-            const int xs = ex_(i) ? wrap(x - ex_(i), a.nx) : x;
-            const int ys = ey_(i) ? wrap(y - ey_(i), a.ny) : y;
-            const int zs = ez_(i) ? wrap(z - ez_(i), a.nz) : z;
-            f[i] = (R)ld_pop(fin[(size_t)i * a.plane + node_index(a, xs, ys, zs)]);
-        }
+        f[i] = (R)ld_pop(v[i]);
         if constexpr (is_half<S>()) f[i] += ((R)w36_(i) / (R)36) * ref;
     });
 }
@@ -439,7 +454,7 @@ __device__ void face_reconstruct(const D3Args<S>& a, int fid, int x, int y, int 
 }
 
 template <typename S>
-__global__ void __launch_bounds__(256, 4) d3q_pull_kernel(D3Args<S> a) {
+__global__ void __launch_bounds__(256, 3) d3q_pull_kernel(D3Args<S> a) {
     using R = typename Store<S>::R;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -452,41 +467,26 @@ __global__ void __launch_bounds__(256, 4) d3q_pull_kernel(D3Args<S> a) {
         return;
     }
     if ((info >> INFO3_FACE_SHIFT) & 7u) return;  // open-face nodes: d3q_face_pull_kernel
+    R r[2];
     if constexpr (is_half<S>()) {
         // sum w_i = 1: rho_k = rho_ref + the sum of the stored deviations
-        const long long sy = a.pitch, sz = (long long)a.ny * a.pitch;
-        const bool wrapped = (info & INFO3_WRAP) != 0;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const S* __restrict__ fin = a.fin + (size_t)k * Q * a.plane;
+            S v[Q];
+            pull_raw<S>(a, k, x, y, z, n, info, v);
             float acc = 0.0f;
-            static_for<0, Q>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                long long src;
-                int ii = i;
-                if (info & (1u << i)) {
-                    src = n;
-                    ii = opp_(i);
-                } else if (!wrapped) {
-                    src = n - ex_(i) - (long long)ey_(i) * sy - (long long)ez_(i) * sz;
-                } else {
-                    src = node_index(a, ex_(i) ? wrap(x - ex_(i), a.nx) : x, ey_(i) ? wrap(y - ey_(i), a.ny) : y,
-                                     ez_(i) ? wrap(z - ez_(i), a.nz) : z);
-                }
-                acc += __half2float(fin[(size_t)ii * a.plane + src]);
-            });
-            a.rho[2 * n + k] = __half2float(a.rref_in[(size_t)k * a.plane + n]) + acc;
+            static_for<0, Q>([&](auto I) { acc += __half2float(v[decltype(I)::value]); });
+            r[k] = __half2float(a.rref_in[(size_t)k * a.plane + n]) + acc;
         }
     } else {
-        R r[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             R f[Q];
-            pull<S, R, false>(a, k, x, y, z, info, f);
+            pull<S, R>(a, k, x, y, z, info, f);
             r[k] = sum19(f);
         }
-        reinterpret_cast<typename Pair<R>::type*>(a.rho)[n] = typename Pair<R>::type{r[0], r[1]};
     }
+    reinterpret_cast<typename Pair<R>::type*>(a.rho)[n] = typename Pair<R>::type{r[0], r[1]};
 }
 
 // Face slot -> face index and node coordinates; false for solid positions.
@@ -660,13 +660,14 @@ template <typename S, typename DestRho>
 __device__ __forceinline__ void store_pop(const D3Args<S>& a, int k, long long n, const typename Store<S>::R (&f)[Q],
                                           DestRho dest_ref) {
     using R = typename Store<S>::R;
+    const unsigned off = (unsigned)n * (unsigned)sizeof(S);
     static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         if constexpr (is_half<S>()) {
             const R ref = dest_ref(I, k);
-            a.fout[(size_t)(k * Q + i) * a.plane + n] = __float2half_rn(f[i] - ((R)w36_(i) / (R)36) * ref);
+            st_at(a.dst[k][i], off, __float2half_rn(f[i] - ((R)w36_(i) / (R)36) * ref));
         } else {
-            a.fout[(size_t)(k * Q + i) * a.plane + n] = (S)f[i];
+            st_at(a.dst[k][i], off, (S)f[i]);
         }
     });
 }
@@ -683,25 +684,36 @@ __device__ __forceinline__ void check_store_u(const D3Args<S>& a, long long n, t
     }
 }
 
-// Every fluid node of a 32x4xTZ tile: forces from the staged densities (the
-// halo resolves periodic wraps and the ghost mirrors of Eqs. 24-25), the
-// common velocity, the collision.  Open-face nodes take their post-boundary
-// populations from the face kernel; outlet nodes stop after the force (their
-// normal velocity waits for the inward neighbour's, Eq. 22), and the inward
-// neighbours of the outlet hand theirs over with the flux terms of Eqs. 21, 23.
-// Residency: FP32 runs 2 CTAs of 512 per SM (64 registers, a few spilled
-// words), FP16 storage 3 of 256 (its decode needs more live values), FP64 1
-// of 256.  Tiles without a fluid node leave before staging.
+// Density box of a tile and its halo by loads: periodic wraps, ghost mirrors and
+// walls resolved per site unless the whole box lies inside the grid.
+template <typename S, typename Put>
+__device__ __forceinline__ void stage_box(const D3Args<S>& a, int x0, int y0, int z0, bool inner, int tid, Put put) {
+    using R = typename Store<S>::R;
+    using V = typename Pair<R>::type;
+    const V* rp = reinterpret_cast<const V*>(a.rho);
+    for (int q = tid; q < Tile3<S>::HN; q += Tile3<S>::NT) {
+        const int hx = q % HX, hy = (q / HX) % HY, hz = q / (HX * HY);
+        const long long m = inner ? node_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz)
+                                  : site_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz);
+        put(q, m < 0 ? V{(R)0, (R)0} : rp[m]);
+    }
+}
+
+// FP64 and FP16 storage.  Every fluid node of a 32x4x2 tile: forces from the
+// staged densities (the halo resolves periodic wraps and the ghost mirrors of
+// Eqs. 24-25), the common velocity, the collision of one component after the
+// other.  Open-face nodes take their post-boundary populations from the face
+// kernel; outlet nodes stop after the force (their normal velocity waits for
+// the inward neighbour's, Eq. 22), and the inward neighbours of the outlet
+// hand theirs over with the flux terms of Eqs. 21, 23.  Residency: FP16 storage
+// 3 CTAs of 256 per SM (80 registers), FP64 1.  Tiles without a fluid node
+// leave before staging.
 template <typename S>
-__global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
-    d3q_collide_kernel(D3Args<S> a, const __grid_constant__ CUtensorMap rho_map, int use_tma) {
+__global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collide_kernel(D3Args<S> a) {
     using R = typename Store<S>::R;
     constexpr int TZ = Tile3<S>::TZ, HN = Tile3<S>::HN, NT = Tile3<S>::NT;
-    // (rho_1, rho_2) of the tile and its halo, psi = 0 at solids; 128-byte
-    // aligned: an interior FP32 tile receives it as one tensor copy
-    __shared__ __align__(128) typename Pair<R>::type s_rr[HN];
-    __shared__ __align__(8) unsigned long long s_bar;
-    __shared__ __half2 s_ref[is_half<S>() ? HN : 1];  // FP16 storage: the same densities rounded to half
+    __shared__ __align__(16) typename Pair<R>::type s_rr[HN];  // (rho_1, rho_2) of the tile and its halo
+    __shared__ __half2 s_ref[is_half<S>() ? HN : 1];           // FP16 storage: the same rounded to half
     __shared__ R s_rate[2][Q];  // relaxation rates of both components (indexed by component below)
     // component 0's pulled populations, kept for its collision after
     // component 1's (FP32 arithmetic; FP64 pulls them again, its tile would
@@ -720,42 +732,11 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
     // tiles whose halo lies inside the grid need no wrap / mirror / wall resolution
     const bool inner = x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= a.nx && y0 + TY + 2 <= a.ny &&
                        z0 + TZ + 2 <= a.nz;
-    bool staged = false;
-    if constexpr (std::is_same<S, float>::value) {
-        // interior FP32 tile: the (TX+4) x (TY+4) x (TZ+4) box of density
-        // pairs as one TMA copy (x0 - 2 is even: an 8-byte element start on a
-        // 16-byte boundary); the block-uniform test keeps a misaligned
-        // destination on the load path
-        if (use_tma && inner && (smem_addr(s_rr) & 127u) == 0u) {
-            if (tid == 0) {
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_bar)) : "memory");
-                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)),
-                             "r"((unsigned)(HN * sizeof(typename Pair<R>::type)))
-                             : "memory");
-                asm volatile(
-                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
-                    "[%1, {%2, %3, %4}], [%5];" ::"r"(smem_addr(s_rr)),
-                    "l"(&rho_map), "r"(x0 - 2), "r"(y0 - 2), "r"(z0 - 2), "r"(smem_addr(&s_bar))
-                    : "memory");
-            }
-            __syncthreads();  // the barrier exists before anyone waits on it; s_rate is written
-            if (!bar_wait(&s_bar, 0u) && tid == 0) atomicOr(a.status, STATUS3_TIMEOUT);
-            staged = true;
-        }
-    }
-    if (!staged) {
-        const auto* rp = reinterpret_cast<const typename Pair<R>::type*>(a.rho);
-        for (int q = tid; q < HN; q += NT) {
-            const int hx = q % HX, hy = (q / HX) % HY, hz = q / (HX * HY);
-            const long long m = inner ? node_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz)
-                                      : site_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz);
-            const typename Pair<R>::type v = m < 0 ? typename Pair<R>::type{(R)0, (R)0} : rp[m];
-            s_rr[q] = v;
-            if constexpr (is_half<S>()) s_ref[q] = __floats2half2_rn((float)v.x, (float)v.y);
-        }
-        __syncthreads();
-    }
+    stage_box(a, x0, y0, z0, inner, tid, [&](int q, typename Pair<R>::type v) {
+        s_rr[q] = v;
+        if constexpr (is_half<S>()) s_ref[q] = __floats2half2_rn((float)v.x, (float)v.y);
+    });
+    __syncthreads();
     if (info & INFO3_SOLID) return;  // solid, or outside the grid
     const int hc = (threadIdx.x + 2) + HX * ((threadIdx.y + 2) + HY * (threadIdx.z + 2));
     auto site = [&](int dx, int dy, int dz) { return s_rr[hc + dx + HX * (dy + HY * dz)]; };
@@ -867,6 +848,263 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
         const R fx = k ? F2[0] : F1[0], fy = k ? F2[1] : F1[1], fz = k ? F2[2] : F1[2];
         collide<R>(f, rk, u[0], u[1], u[2], fx, fy, fz, s_rate[k]);
         store_pop<S>(a, k, n, f, dest_rho);
+    }
+}
+
+// ---- FP32 collision: both components of a node in packed FP32x2 operations ----
+__device__ __forceinline__ float2 vc(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, vc(-1.f), a); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// Momentum of both components: sums of opposite-pair differences.
+__device__ __forceinline__ void momentum2(const float2 (&f)[Q], float2& jx, float2& jy, float2& jz) {
+    const float2 d7 = vsub(f[7], f[10]), d8 = vsub(f[8], f[9]), d11 = vsub(f[11], f[14]), d12 = vsub(f[12], f[13]),
+                 d15 = vsub(f[15], f[18]), d16 = vsub(f[16], f[17]);
+    jx = vadd(vsub(f[1], f[2]), vadd(vsub(d7, d8), vsub(d11, d12)));
+    jy = vadd(vsub(f[3], f[4]), vadd(vadd(d7, d8), vsub(d15, d16)));
+    jz = vadd(vsub(f[5], f[6]), vadd(vadd(d11, d12), vadd(d15, d16)));
+}
+
+// Eq. 1 as in collide(), with the 19 rows of T and T^-1 written out over the
+// sums and differences of opposite pairs: axis pairs (1,2), (3,4), (5,6), edge
+// pairs (7,10), (8,9) in xy, (11,14), (12,13) in xz, (15,18), (16,17) in yz.
+// s: rates of (e, eps, j, q, nu), the values the 19 diagonal entries take
+// (pi shares eps, m shares q).
+__device__ __forceinline__ void collide2(float2 (&f)[Q], float2 r, float ux, float uy, float uz, float2 Fx, float2 Fy,
+                                         float2 Fz, const float2 (&s)[5]) {
+    const float2 px = vadd(f[1], f[2]), py = vadd(f[3], f[4]), pz = vadd(f[5], f[6]);
+    const float2 p7 = vadd(f[7], f[10]), p8 = vadd(f[8], f[9]), p11 = vadd(f[11], f[14]), p12 = vadd(f[12], f[13]),
+                 p15 = vadd(f[15], f[18]), p16 = vadd(f[16], f[17]);
+    const float2 dx = vsub(f[1], f[2]), dy = vsub(f[3], f[4]), dz = vsub(f[5], f[6]);
+    const float2 d7 = vsub(f[7], f[10]), d8 = vsub(f[8], f[9]), d11 = vsub(f[11], f[14]), d12 = vsub(f[12], f[13]),
+                 d15 = vsub(f[15], f[18]), d16 = vsub(f[16], f[17]);
+    const float2 sxy = vadd(p7, p8), sxz = vadd(p11, p12), syz = vadd(p15, p16);
+    const float2 sa = vadd(px, vadd(py, pz)), se = vadd(vadd(sxy, sxz), syz);
+    const float2 U = vc(ux), V = vc(uy), W = vc(uz);
+    const float xx = ux * ux, yy = uy * uy, zz = uz * uz, uu = xx + yy + zz;
+    const float2 uF = vfma(U, Fx, vfma(V, Fy, vmul(W, Fz)));
+    const float2 half = vc(0.5f);
+    float2 h[5], ns[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        h[q] = vfma(vc(-0.5f), s[q], vc(1.f));
+        ns[q] = vmul(vc(-1.f), s[q]);
+    }
+    // g_r = (-s (m - m^eq) + (1 - s/2) F_m) / |row|^2
+    const float2 me = vfma(vc(-30.f), f[0], vfma(vc(-11.f), sa, vmul(vc(8.f), se)));
+    const float2 ge = vmul(vc(1.f / 2394.f), vfma(ns[0], vsub(me, vmul(r, vc(19.f * uu - 11.f))),
+                                                  vmul(h[0], vmul(vc(38.f), uF))));
+    const float2 mp = vfma(vc(12.f), f[0], vfma(vc(-4.f), sa, se));
+    const float2 gp = vmul(vc(1.f / 252.f), vfma(ns[1], vsub(mp, vmul(r, vc(3.f - 5.5f * uu))),
+                                                 vmul(h[1], vmul(vc(-11.f), uF))));
+    const float2 exy = vsub(d7, d8), exz = vsub(d11, d12), eyx = vadd(d7, d8), eyz = vsub(d15, d16),
+                 ezx = vadd(d11, d12), ezy = vadd(d15, d16);
+    const float2 jx = vadd(exy, exz), jy = vadd(eyx, eyz), jz = vadd(ezx, ezy);
+    const float2 rux = vmul(r, U), ruy = vmul(r, V), ruz = vmul(r, W);
+    const float2 c10 = vc(0.1f), c40 = vc(1.f / 40.f), t23 = vc(2.f / 3.f);
+    const float2 gjx = vmul(c10, vfma(ns[2], vsub(vadd(dx, jx), rux), vmul(h[2], Fx)));
+    const float2 gjy = vmul(c10, vfma(ns[2], vsub(vadd(dy, jy), ruy), vmul(h[2], Fy)));
+    const float2 gjz = vmul(c10, vfma(ns[2], vsub(vadd(dz, jz), ruz), vmul(h[2], Fz)));
+    // q^eq = -2/3 rho u, its forcing -2/3 F
+    const float2 hq = vmul(vmul(vc(-1.f), t23), h[3]);
+    const float2 gqx = vmul(c40, vfma(ns[3], vfma(t23, rux, vfma(vc(-4.f), dx, jx)), vmul(hq, Fx)));
+    const float2 gqy = vmul(c40, vfma(ns[3], vfma(t23, ruy, vfma(vc(-4.f), dy, jy)), vmul(hq, Fy)));
+    const float2 gqz = vmul(c40, vfma(ns[3], vfma(t23, ruz, vfma(vc(-4.f), dz, jz)), vmul(hq, Fz)));
+    // 3p_xx and 3pi_xx (equilibrium and forcing of pi: -1/2 of p's)
+    const float2 ax = vsub(vmul(vc(2.f), px), vadd(py, pz)), exx = vfma(vc(-2.f), syz, vadd(sxy, sxz));
+    const float2 qxx = vmul(r, vc(2.f * xx - yy - zz));
+    const float2 fxx = vmul(vc(2.f), vsub(vmul(vmul(vc(2.f), U), Fx), vfma(V, Fy, vmul(W, Fz))));
+    const float2 gxx = vmul(vc(1.f / 36.f), vfma(ns[4], vsub(vadd(ax, exx), qxx), vmul(h[4], fxx)));
+    const float2 gyx = vmul(vc(1.f / 72.f), vfma(ns[1], vfma(half, qxx, vfma(vc(-2.f), ax, exx)),
+                                                 vmul(h[1], vmul(vc(-0.5f), fxx))));
+    // p_ww and pi_ww
+    const float2 aw = vsub(py, pz), ew = vsub(sxy, sxz);
+    const float2 qww = vmul(r, vc(yy - zz)), fww = vmul(vc(2.f), vsub(vmul(V, Fy), vmul(W, Fz)));
+    const float2 gww = vmul(vc(1.f / 12.f), vfma(ns[4], vsub(vadd(aw, ew), qww), vmul(h[4], fww)));
+    const float2 gyw = vmul(vc(1.f / 24.f), vfma(ns[1], vfma(half, qww, vfma(vc(-2.f), aw, ew)),
+                                                 vmul(h[1], vmul(vc(-0.5f), fww))));
+    // p_xy, p_yz, p_xz
+    const float2 c4 = vc(0.25f);
+    const float2 gxy = vmul(c4, vfma(ns[4], vsub(vsub(p7, p8), vmul(rux, V)), vmul(h[4], vfma(U, Fy, vmul(V, Fx)))));
+    const float2 gyz = vmul(c4, vfma(ns[4], vsub(vsub(p15, p16), vmul(ruy, W)), vmul(h[4], vfma(V, Fz, vmul(W, Fy)))));
+    const float2 gxz = vmul(c4, vfma(ns[4], vsub(vsub(p11, p12), vmul(rux, W)), vmul(h[4], vfma(U, Fz, vmul(W, Fx)))));
+    // m_x, m_y, m_z (no equilibrium, no forcing)
+    const float2 n8 = vmul(vc(0.125f), ns[3]);
+    const float2 gmx = vmul(n8, vsub(exy, exz)), gmy = vmul(n8, vsub(eyz, eyx)), gmz = vmul(n8, vsub(ezx, ezy));
+    // back: f_i += even + odd, f_ibar += even - odd
+    auto put = [&](int i, int o, float2 ev, float2 od) {
+        f[i] = vadd(f[i], vadd(ev, od));
+        f[o] = vadd(f[o], vsub(ev, od));
+    };
+    f[0] = vadd(f[0], vfma(vc(-30.f), ge, vmul(vc(12.f), gp)));
+    const float2 ea = vfma(vc(-11.f), ge, vmul(vc(-4.f), gp)), ee = vfma(vc(8.f), ge, gp);
+    const float2 axx = vfma(vc(-2.f), gyx, gxx), aww = vfma(vc(-2.f), gyw, gww);
+    put(1, 2, vfma(vc(2.f), axx, ea), vfma(vc(-4.f), gqx, gjx));
+    const float2 eb = vsub(ea, axx);
+    put(3, 4, vadd(eb, aww), vfma(vc(-4.f), gqy, gjy));
+    put(5, 6, vsub(eb, aww), vfma(vc(-4.f), gqz, gjz));
+    const float2 Jx = vadd(gjx, gqx), Jy = vadd(gjy, gqy), Jz = vadd(gjz, gqz);
+    const float2 bxx = vadd(gxx, gyx), bww = vadd(gww, gyw), e1 = vadd(ee, bxx);
+    {
+        const float2 A = vadd(Jx, gmx), B = vsub(Jy, gmy), e = vadd(e1, bww);
+        put(7, 10, vadd(e, gxy), vadd(A, B));
+        put(8, 9, vsub(e, gxy), vsub(B, A));
+    }
+    {
+        const float2 A = vsub(Jx, gmx), B = vadd(Jz, gmz), e = vsub(e1, bww);
+        put(11, 14, vadd(e, gxz), vadd(A, B));
+        put(12, 13, vsub(e, gxz), vsub(B, A));
+    }
+    {
+        const float2 A = vadd(Jy, gmy), B = vsub(Jz, gmz), e = vfma(vc(-2.f), bxx, ee);
+        put(15, 18, vadd(e, gyz), vadd(A, B));
+        put(16, 17, vsub(e, gyz), vsub(B, A));
+    }
+}
+
+// FP32: the same step as d3q_collide_kernel with both components of a node in
+// the two lanes of packed FP32x2 instructions: one pass of about half the
+// instructions, nothing parked in shared memory between two collisions, and all
+// 38 pulls of a node issued before the density box is waited for (16 warps x 38
+// loads in flight per SM at 126 registers).  512x96x96 co-flow device: 330 ->
+// 280 us for the collision; the whole step 530 -> 435 us with the graph branches.
+__global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
+    d3q_collide_f32_kernel(const __grid_constant__ D3Args<float> a, const __grid_constant__ CUtensorMap rho_map,
+                           int use_tma) {
+    constexpr int TZ = Tile3<float>::TZ, HN = Tile3<float>::HN;
+    // (rho_1, rho_2) of the tile and its halo, psi = 0 at solids; 128-byte
+    // aligned: an interior tile receives it as one tensor copy
+    __shared__ __align__(128) float2 s_rr[HN];
+    __shared__ __align__(8) unsigned long long s_bar;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
+    const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
+    const bool in_grid = x < a.nx && y < a.ny && z < a.nz;
+    const long long n = in_grid ? node_index(a, x, y, z) : 0;
+    const uint32_t info = in_grid ? a.info[n] : (uint32_t)INFO3_SOLID;
+    // tiles whose halo lies inside the grid need no wrap / mirror / wall
+    // resolution; their box comes as one TMA copy (x0 - 2 is even: an 8-byte
+    // element start on a 16-byte boundary).  The block-uniform test keeps a
+    // misaligned destination on the load path.
+    const bool inner = x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= a.nx && y0 + TY + 2 <= a.ny &&
+                       z0 + TZ + 2 <= a.nz;
+    const bool tma = use_tma && inner && (smem_addr(s_rr) & 127u) == 0u;
+    if (tma && tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_bar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // a tile without fluid nodes has nothing to stage or collide
+    if (!__syncthreads_or(!(info & INFO3_SOLID))) return;
+    if (tma) {
+        if (tid == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)),
+                         "r"((unsigned)(HN * sizeof(float2)))
+                         : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                "[%1, {%2, %3, %4}], [%5];" ::"r"(smem_addr(s_rr)),
+                "l"(&rho_map), "r"(x0 - 2), "r"(y0 - 2), "r"(z0 - 2), "r"(smem_addr(&s_bar))
+                : "memory");
+        }
+    } else {
+        stage_box(a, x0, y0, z0, inner, tid, [&](int q, float2 v) { s_rr[q] = v; });
+    }
+    const int fid = (int)((info >> INFO3_FACE_SHIFT) & 7u);
+    const int nid = (int)((info >> INFO3_NBR_SHIFT) & 7u);
+    // all 38 pulls are in flight while the densities arrive
+    float2 f[Q];
+    int slot = -1;
+    if (!(info & INFO3_SOLID)) {
+        if (fid == 0) {
+            float v0[Q], v1[Q];
+            pull_raw<float>(a, 0, x, y, z, n, info, v0);
+            pull_raw<float>(a, 1, x, y, z, n, info, v1);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) f[i] = make_float2(v0[i], v1[i]);
+        } else {
+            slot = face_slot(a.face[fid - 1], x, y, z);
+            const float* ff = a.fface + (size_t)slot * 2 * Q;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) f[i] = make_float2(ff[i], ff[Q + i]);
+        }
+    }
+    if (tma) {
+        if (!bar_wait(&s_bar, 0u) && tid == 0) atomicOr(a.status, STATUS3_TIMEOUT);
+    } else {
+        __syncthreads();
+    }
+    if (info & INFO3_SOLID) return;  // solid, or outside the grid
+    const int hc = (threadIdx.x + 2) + HX * ((threadIdx.y + 2) + HY * (threadIdx.z + 2));
+    const float2 r = s_rr[hc];
+    float g1[3], g2[3], ad[3];
+    stencil_sums<float>([&](int dx, int dy, int dz) { return s_rr[hc + dx + HX * (dy + HY * dz)]; }, g1, g2);
+    adhesion_vector<float>(a, n, info, ad);
+    const float rt = r.x + r.y, inv = 1.f / rt;
+    float2 F[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float2 t = vfma(make_float2(-a.G[1], -a.G[2]), vc(ad[q]), vmul(vc(-a.G[0]), make_float2(g2[q], g1[q])));
+        F[q] = vmul(r, vadd(t, vc(a.body[q] * inv)));
+    }
+    if (fid != 0) {
+        const FaceDev3& Fc = a.face[fid - 1];
+        float* Fp = a.FpF + (size_t)slot * 6;  // this step's force: next step's inlet, this step's outlet
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            Fp[q] = F[q].x;
+            Fp[3 + q] = F[q].y;
+        }
+        if (Fc.kind == FACE3_OUTLET) return;  // finished by d3q_outlet_kernel
+    }
+    float u[3];
+    {
+        float2 j[3];
+        momentum2(f, j[0], j[1], j[2]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float2 t = vfma(vc(0.5f), F[q], j[q]);
+            u[q] = (t.x + t.y) * inv;
+        }
+    }
+    if (nid != 0) {
+        const FaceDev3& Fc = a.face[nid - 1];
+        const int ns = face_slot(Fc, x + Fc.o[0], y + Fc.o[1], z + Fc.o[2]);
+        float* Fp = a.FpN + (size_t)ns * 6;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            Fp[q] = F[q].x;
+            Fp[3 + q] = F[q].y;
+        }
+        if (Fc.kind == FACE3_OUTLET) {
+            const double sg = (double)(Fc.o[0] + Fc.o[1] + Fc.o[2]);
+            const float ua = Fc.axis == 0 ? u[0] : (Fc.axis == 1 ? u[1] : u[2]);
+            float* un = a.unbr + (size_t)ns * 3;
+            un[0] = u[0];
+            un[1] = u[1];
+            un[2] = u[2];
+            a.flux[(size_t)ns * 2 + 0] = (double)rt * sg * (double)ua;
+            a.flux[(size_t)ns * 2 + 1] = sg * (double)ua;
+        }
+    }
+    if (fid != 0) {  // inlet node: flux term of Q_in
+        const FaceDev3& Fc = a.face[fid - 1];
+        const double sg = (double)(Fc.o[0] + Fc.o[1] + Fc.o[2]);
+        const float ua = Fc.axis == 0 ? u[0] : (Fc.axis == 1 ? u[1] : u[2]);
+        a.flux[(size_t)slot * 2 + 0] = (double)rt * (-sg) * (double)ua;
+        a.flux[(size_t)slot * 2 + 1] = 0.0;
+    }
+    check_store_u<float>(a, n, rt, u);
+    const float2 s[5] = {make_float2(a.s[0][1], a.s[1][1]), make_float2(a.s[0][2], a.s[1][2]),
+                         make_float2(a.s[0][3], a.s[1][3]), make_float2(a.s[0][4], a.s[1][4]),
+                         make_float2(a.s[0][9], a.s[1][9])};
+    collide2(f, r, u[0], u[1], u[2], F[0], F[1], F[2], s);
+    const unsigned off = (unsigned)n * 4u;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        st_at(a.dst[0][i], off, f[i].x);
+        st_at(a.dst[1][i], off, f[i].y);
     }
 }
 
@@ -1072,32 +1310,74 @@ cudaError_t launch_macros(const R* rho_pairs, const R* umac, const uint32_t* inf
 }
 
 template <typename S>
+static cudaError_t launch_pull(const D3Args<S>& a, cudaStream_t st) {
+    const dim3 blk(32, 4, 2);
+    const dim3 grd((a.nx + 31) / 32, (a.ny + 3) / 4, (a.nz + 1) / 2);
+    d3q_pull_kernel<S><<<grd, blk, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename S>
+static cudaError_t launch_collide(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st) {
+    static const CUtensorMap kNoMap{};
+    constexpr int TZ = Tile3<S>::TZ;
+    const dim3 blk(TX, TY, TZ);
+    const dim3 grd((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + TZ - 1) / TZ);
+    if constexpr (std::is_same<S, float>::value)
+        d3q_collide_f32_kernel<<<grd, blk, 0, st>>>(a, rho_map ? *rho_map : kNoMap, rho_map ? 1 : 0);
+    else
+        d3q_collide_kernel<S><<<grd, blk, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+constexpr int FACE_NT = 64;  // threads of a face block: few long threads, spread over many SMs
+static int face_blocks(int slots) { return (slots + FACE_NT - 1) / FACE_NT; }
+
+template <typename S>
 cudaError_t launch_step(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st, cudaEvent_t mid_a,
                         cudaEvent_t mid_b) {
-    const dim3 blkA(32, 4, 2);
-    const dim3 grdA((a.nx + 31) / 32, (a.ny + 3) / 4, (a.nz + 1) / 2);
-    const int fblocks = (a.nface_slots + 127) / 128;
-    d3q_pull_kernel<S><<<grdA, blkA, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pull(a, st);
     if (e != cudaSuccess) return e;
     if (a.nface_slots > 0) {
-        d3q_face_pull_kernel<S><<<fblocks, 128, 0, st>>>(a);
+        d3q_face_pull_kernel<S><<<face_blocks(a.nface_slots), FACE_NT, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (mid_a) cudaEventRecord(mid_a, st);
-    constexpr int TZ = Tile3<S>::TZ;
-    const dim3 blkB(TX, TY, TZ);
-    const dim3 grdB((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + TZ - 1) / TZ);
-    static const CUtensorMap kNoMap{};
-    d3q_collide_kernel<S><<<grdB, blkB, 0, st>>>(a, rho_map ? *rho_map : kNoMap, rho_map ? 1 : 0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_collide(a, rho_map, st)) != cudaSuccess) return e;
     if (mid_b) cudaEventRecord(mid_b, st);
     if (a.nface_slots > 0) {
-        d3q_outlet_kernel<S><<<fblocks, 128, 0, st>>>(a);
+        d3q_outlet_kernel<S><<<face_blocks(a.nface_slots), FACE_NT, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         d3q_reduce_kernel<S><<<1, RED, 0, st>>>(a);
         e = cudaGetLastError();
     }
+    return e;
+}
+
+// Branch order.  The face pulls of a step need the previous step's collision,
+// outlet and reduction; the interior pulls the collision and outlet only; the
+// collision both pulls.  The reduction reads the flux terms, which the next
+// collision (after the next face pulls, hence after it) overwrites.
+template <typename S>
+cudaError_t launch_step_forked(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st, cudaStream_t side,
+                               const cudaEvent_t (&ev)[3]) {
+    cudaError_t e = cudaSuccess;
+    const bool faces = a.nface_slots > 0;
+    if (faces) {
+        d3q_face_pull_kernel<S><<<face_blocks(a.nface_slots), FACE_NT, 0, side>>>(a);
+        if ((e = cudaGetLastError()) == cudaSuccess) e = cudaEventRecord(ev[1], side);
+    }
+    if (e == cudaSuccess) e = launch_pull(a, st);
+    if (faces && e == cudaSuccess) e = cudaStreamWaitEvent(st, ev[1], 0);
+    if (e == cudaSuccess) e = launch_collide(a, rho_map, st);
+    if (!faces || e != cudaSuccess) return e;
+    if ((e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
+    d3q_outlet_kernel<S><<<face_blocks(a.nface_slots), FACE_NT, 0, st>>>(a);
+    if ((e = cudaGetLastError()) == cudaSuccess) e = cudaEventRecord(ev[0], st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev[2], 0);
+    if (e != cudaSuccess) return e;
+    d3q_reduce_kernel<S><<<1, RED, 0, side>>>(a);
+    if ((e = cudaGetLastError()) == cudaSuccess) e = cudaStreamWaitEvent(side, ev[0], 0);
     return e;
 }
 
@@ -1115,6 +1395,12 @@ template cudaError_t launch_step<double>(const D3Args<double>&, const CUtensorMa
                                           cudaEvent_t);
 template cudaError_t launch_step<__half>(const D3Args<__half>&, const CUtensorMap*, cudaStream_t, cudaEvent_t,
                                           cudaEvent_t);
+template cudaError_t launch_step_forked<float>(const D3Args<float>&, const CUtensorMap*, cudaStream_t, cudaStream_t,
+                                               const cudaEvent_t (&)[3]);
+template cudaError_t launch_step_forked<double>(const D3Args<double>&, const CUtensorMap*, cudaStream_t,
+                                                cudaStream_t, const cudaEvent_t (&)[3]);
+template cudaError_t launch_step_forked<__half>(const D3Args<__half>&, const CUtensorMap*, cudaStream_t,
+                                                cudaStream_t, const cudaEvent_t (&)[3]);
 template cudaError_t launch_macros<float>(const float*, const float*, const uint32_t*, int, int, int, int, long long,
                                            const unsigned*, float*, float*, unsigned*, cudaStream_t);
 template cudaError_t launch_macros<double>(const double*, const double*, const uint32_t*, int, int, int, int,

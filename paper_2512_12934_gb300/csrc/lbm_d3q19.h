@@ -28,9 +28,9 @@ enum { FACE3_INLET = 1, FACE3_OUTLET = 2 };
 // status word bits of a D3Q19 step: non-finite result; a bounded wait on a
 // tensor copy that ran out
 constexpr unsigned STATUS3_DIVERGED = 1u, STATUS3_TIMEOUT = 2u;
-// density box of one FP32 collide tile (32 x 4 x 4 nodes) and its 2-node halo,
+// density box of one FP32 collide tile (32 x 4 x 2 nodes) and its 2-node halo,
 // the tensor-copy box of the density field
-constexpr int RHO_BOX3_X = 36, RHO_BOX3_Y = 8, RHO_BOX3_Z = 8;
+constexpr int RHO_BOX3_X = 36, RHO_BOX3_Y = 8, RHO_BOX3_Z = 6;
 // device scalars of the open boundaries (ping-pong per step)
 enum { SC3_LAMBDA = 0, SC3_CHI = 1, SC3_QIN = 2, SC3_QOUT = 3, SC3_UMEAN = 4, SC3_N = 8 };
 
@@ -71,6 +71,12 @@ struct D3Args {
     int open_side[6];
     const S* fin;
     S* fout;
+    // per component and direction: the plane of fin shifted so that element n is
+    // the pull source of node n (away from periodic edges), and the plane of
+    // fout.  Uniform bases with one 32-bit byte offset per thread: an address
+    // costs no per-thread arithmetic.
+    const S* src[2][Q];
+    S* dst[2][Q];
     const uint32_t* info;
     R* rho;   // [plane][2] (rho_1, rho_2) of each node for the step, (0, 0) at solids (psi = 0)
     R* umac;  // [3][plane] u^eq of the step (may be null)
@@ -100,12 +106,21 @@ struct D3Args {
     R s[2][Q];
 };
 
-// rho_map: tensor map of the density field as 8-byte (rho_1, rho_2) pairs
-// (FP32 contexts; NULL: the collide kernel stages every density box with
-// loads)
+// One step.  rho_map: tensor map of the density field as 8-byte (rho_1, rho_2)
+// pairs (FP32 contexts; NULL: the collide kernel stages every density box with
+// loads).  mid_a, mid_b (may be NULL): recorded after the pulls and after the
+// collision.
 template <typename S>
 cudaError_t launch_step(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st,
                         cudaEvent_t mid_a = nullptr, cudaEvent_t mid_b = nullptr);
+
+// The same step in two branches, for capture into a graph: face pulls and flux
+// reduction on `side`, the rest on `st`.  ev[0]: on st, everything the next
+// step's face pulls read (recorded on st before the first step); ev[1], ev[2]:
+// scratch.  The caller joins `side` after the last step.
+template <typename S>
+cudaError_t launch_step_forked(const D3Args<S>& a, const CUtensorMap* rho_map, cudaStream_t st, cudaStream_t side,
+                               const cudaEvent_t (&ev)[3]);
 
 // Dense macroscopic fields rho [2][nz][ny][nx] and u [3][nz][ny][nx] in float,
 // 0 at solid nodes, from the density pairs and u^eq.  Nothing is written when

@@ -16,6 +16,7 @@ const char* error(const Ctx3* c);
 lbm_status reset(Ctx3* c, const double* rho_init, const double* u_init);
 lbm_status step(Ctx3* c, int64_t nsteps);
 lbm_status sync(Ctx3* c);
+lbm_status set_graphs(Ctx3* c, int on);  // graph replay of step runs on (default) or off
 lbm_status enable_timing(Ctx3* c, int every);
 lbm_status kernel_time_split(Ctx3* c, double* pull_ms, double* collide_ms, int64_t* samples);
 lbm_status get_macros(Ctx3* c, float* rho, float* u, int dst_is_device);
