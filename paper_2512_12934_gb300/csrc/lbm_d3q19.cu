@@ -29,6 +29,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -126,7 +127,7 @@ struct Tile3 {
     static constexpr int HZ = TZ + 4;
     static constexpr int HN = HX * HY * HZ;
     static constexpr int NT = TX * TY * TZ;
-    static constexpr int MIN_BLOCKS = sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 2 : 3);
+    static constexpr int MIN_BLOCKS = sizeof(S) == 8 ? 1 : 3;
 };
 static_assert(HX == RHO_BOX3_X && HY == RHO_BOX3_Y && Tile3<float>::HZ == RHO_BOX3_Z,
               "the density tensor-copy box must be the FP32 collide tile plus its halo");
@@ -185,60 +186,64 @@ __device__ __forceinline__ void st_at(S* base, unsigned off, S v) {
     *reinterpret_cast<S*>(reinterpret_cast<char*>(base) + off) = v;
 }
 
-// One stored population at a uniform base plus the thread's byte offset.
-template <typename S>
-__device__ __forceinline__ S ld_at(const S* base, unsigned off) {
-    return __ldg(reinterpret_cast<const S*>(reinterpret_cast<const char*>(base) + off));
+// The pull sources of components [K0, K1) of node n = (x, y, z) (Eq. 2, Eq. B1,
+// Eq. B2) as addresses: use(k, i, p).  Most nodes have no blocked direction and
+// no wrap: the shifted planes.  The others select each source (its neighbour
+// with periodic wraps, or the opposite direction of the node itself) without a
+// branch, so that their loads are in flight together too: a branch per
+// direction made every load wait for the one before it.  The offsets are
+// 32-bit: n * 8 bytes stays below 2^32 for every grid that fits the device.
+template <int K0, int K1, typename S, typename Use>
+__device__ __forceinline__ void pull_sources(const D3Args<S>& a, int x, int y, int z, long long n, uint32_t info,
+                                             Use use) {
+    auto at = [](const S* base, unsigned m) {
+        return reinterpret_cast<const S*>(reinterpret_cast<const char*>(base) + m * (unsigned)sizeof(S));
+    };
+    if ((info & (0x7FFFFu | INFO3_WRAP)) == 0u) {
+        static_for<K0, K1>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            static_for<0, Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                use(k, i, at(a.src[k][i], (unsigned)n));
+            });
+        });
+        return;
+    }
+    // index distances to the (wrapped) neighbours; that of a blocked source is not used
+    const int sz = a.ny * a.pitch;
+    const int dxm = wrap(x - 1, a.nx) - x, dxp = wrap(x + 1, a.nx) - x;
+    const int dym = (wrap(y - 1, a.ny) - y) * a.pitch, dyp = (wrap(y + 1, a.ny) - y) * a.pitch;
+    const int dzm = (wrap(z - 1, a.nz) - z) * sz, dzp = (wrap(z + 1, a.nz) - z) * sz;
+    static_for<0, Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        const bool bb = (info & (1u << i)) != 0;
+        const int d = (ex_(i) == 1 ? dxm : (ex_(i) == -1 ? dxp : 0)) + (ey_(i) == 1 ? dym : (ey_(i) == -1 ? dyp : 0)) +
+                      (ez_(i) == 1 ? dzm : (ez_(i) == -1 ? dzp : 0));
+        const unsigned m = (unsigned)n + (unsigned)(bb ? 0 : d);
+        static_for<K0, K1>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            use(k, i, at(a.fin + (bb ? k * Q + opp_(i) : k * Q + i) * a.plane, m));
+        });
+    });
 }
 
-// Raw pull of the 19 populations of component k at node n = (x, y, z) (Eq. 2,
-// Eq. B1, Eq. B2).  Most nodes have no blocked direction and no wrap: straight
-// loads from the shifted planes.  The others select each source first, so
-// that their 19 loads are in flight together too (a branch per direction made
-// every load wait for the one before it).  The offsets are 32-bit: n * 8 bytes
-// stays below 2^32 for every grid that fits the device.
-template <typename S>
-__device__ __forceinline__ void pull_raw(const D3Args<S>& a, int k, int x, int y, int z, long long n, uint32_t info,
+// Raw pull of component K at node n.
+template <int K, typename S>
+__device__ __forceinline__ void pull_raw(const D3Args<S>& a, int x, int y, int z, long long n, uint32_t info,
                                          S (&v)[Q]) {
-    const unsigned off = (unsigned)n * (unsigned)sizeof(S);
-    if ((info & (0x7FFFFu | INFO3_WRAP)) == 0u) {
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            v[i] = ld_at(a.src[k][i], off);
-        });
-    } else if (!(info & INFO3_WRAP)) {
-        const S* own = a.fin + (size_t)k * Q * a.plane;
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            const S* p = (info & (1u << i)) ? own + (size_t)opp_(i) * a.plane : a.src[k][i];
-            v[i] = ld_at(p, off);
-        });
-    } else {
-        const S* own = a.fin + (size_t)k * Q * a.plane;
-        const int xm = wrap(x - 1, a.nx), xp = wrap(x + 1, a.nx), ym = wrap(y - 1, a.ny), yp = wrap(y + 1, a.ny),
-                  zm = wrap(z - 1, a.nz), zp = wrap(z + 1, a.nz);
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            const int xs = ex_(i) == 1 ? xm : (ex_(i) == -1 ? xp : x);
-            const int ys = ey_(i) == 1 ? ym : (ey_(i) == -1 ? yp : y);
-            const int zs = ez_(i) == 1 ? zm : (ez_(i) == -1 ? zp : z);
-            const bool bb = (info & (1u << i)) != 0;
-            const long long m = bb ? n : node_index(a, xs, ys, zs);
-            v[i] = __ldg(own + (size_t)(bb ? opp_(i) : i) * a.plane + m);
-        });
-    }
+    pull_sources<K, K + 1>(a, x, y, z, n, info, [&](int, int i, const S* p) { v[i] = __ldg(p); });
 }
 
 // Pull of component k as real values.
-template <typename S, typename R>
-__device__ __forceinline__ void pull(const D3Args<S>& a, int k, int x, int y, int z, uint32_t info, R (&f)[Q]) {
+template <int k, typename S, typename R>
+__device__ __forceinline__ void pull(const D3Args<S>& a, int x, int y, int z, uint32_t info, R (&f)[Q]) {
     const long long n = node_index(a, x, y, z);
     // FP16 storage: every value this node pulls was encoded against its
     // reference density (the writer used the same half-rounded density)
     R ref = 0;
     if constexpr (is_half<S>()) ref = __half2float(a.rref_in[(size_t)k * a.plane + n]);
     S v[Q];
-    pull_raw<S>(a, k, x, y, z, n, info, v);
+    pull_raw<k>(a, x, y, z, n, info, v);
     static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         f[i] = (R)ld_pop(v[i]);
@@ -386,8 +391,8 @@ __device__ void face_reconstruct(const D3Args<S>& a, int fid, int x, int y, int 
     const uint32_t info2 = a.info[node_index(a, x2, y2, z2)];
     if (F.kind == FACE3_INLET) {
         R f2[2][Q];
-        pull<S, R>(a, 0, x2, y2, z2, info2, f2[0]);
-        pull<S, R>(a, 1, x2, y2, z2, info2, f2[1]);
+        pull<0, S, R>(a, x2, y2, z2, info2, f2[0]);
+        pull<1, S, R>(a, x2, y2, z2, info2, f2[1]);
         const R* Fp2 = a.FpN + (size_t)slot * 6;
         const R* Fp1 = a.FpF + (size_t)slot * 6;
         R r2[2], jx = 0, jy = 0, jz = 0;
@@ -430,8 +435,8 @@ __device__ void face_reconstruct(const D3Args<S>& a, int fid, int x, int y, int 
     } else {
         // convective outlet (Eq. 20) with lambda of the previous step
         R fN1[2][Q];
-        pull<S, R>(a, 0, x2, y2, z2, info2, fN1[0]);
-        pull<S, R>(a, 1, x2, y2, z2, info2, fN1[1]);
+        pull<0, S, R>(a, x2, y2, z2, info2, fN1[0]);
+        pull<1, S, R>(a, x2, y2, z2, info2, fN1[1]);
         const R lam = (R)a.scal_in[SC3_LAMBDA];
         R* fo = a.fo + (size_t)slot * 2 * Q;
         #pragma unroll
@@ -453,40 +458,35 @@ __device__ void face_reconstruct(const D3Args<S>& a, int fid, int x, int y, int 
         for (int i = 0; i < Q; ++i) ff[k * Q + i] = f[k][i];
 }
 
+// One thread per node and component: the 19 loads of a thread fit 40 registers,
+// so 48 warps an SM keep them in flight (both components in one thread, 24
+// warps at 80 registers: 116 us on 512x96x96, this form 103; FP16 storage on
+// 250x50x50: 18 us).
 template <typename S>
-__global__ void __launch_bounds__(256, 3) d3q_pull_kernel(D3Args<S> a) {
+__global__ void __launch_bounds__(256, sizeof(S) == 8 ? 3 : 6) d3q_pull_kernel(const __grid_constant__ D3Args<S> a, int zblock) {
     using R = typename Store<S>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z * blockDim.z + threadIdx.z;
-    if (x >= a.nx || y >= a.ny || z >= a.nz) return;
+    const int x = blockIdx.x * 32 + threadIdx.x;
+    const int y = blockIdx.y * 4 + threadIdx.y;
+    const int z = zblock + blockIdx.z, k = threadIdx.z;
+    if (x >= a.nx || y >= a.ny) return;
     const long long n = node_index(a, x, y, z);
     const uint32_t info = a.info[n];
-    if (info & INFO3_SOLID) {  // psi = 0 at solid sites of the force stencil
-        reinterpret_cast<typename Pair<R>::type*>(a.rho)[n] = typename Pair<R>::type{(R)0, (R)0};
-        return;
-    }
     if ((info >> INFO3_FACE_SHIFT) & 7u) return;  // open-face nodes: d3q_face_pull_kernel
-    R r[2];
-    if constexpr (is_half<S>()) {
-        // sum w_i = 1: rho_k = rho_ref + the sum of the stored deviations
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            S v[Q];
-            pull_raw<S>(a, k, x, y, z, n, info, v);
+    R r = 0;                                      // psi = 0 at solid sites of the force stencil
+    if (!(info & INFO3_SOLID)) {
+        S v[Q];
+        if (k == 0) pull_raw<0>(a, x, y, z, n, info, v);
+        else pull_raw<1>(a, x, y, z, n, info, v);
+        if constexpr (is_half<S>()) {
+            // sum w_i = 1: rho_k = rho_ref + the sum of the stored deviations
             float acc = 0.0f;
             static_for<0, Q>([&](auto I) { acc += __half2float(v[decltype(I)::value]); });
-            r[k] = __half2float(a.rref_in[(size_t)k * a.plane + n]) + acc;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            R f[Q];
-            pull<S, R>(a, k, x, y, z, info, f);
-            r[k] = sum19(f);
+            r = __half2float(a.rref_in[(size_t)k * a.plane + n]) + acc;
+        } else {
+            r = sum19(v);
         }
     }
-    reinterpret_cast<typename Pair<R>::type*>(a.rho)[n] = typename Pair<R>::type{r[0], r[1]};
+    a.rho[2 * n + k] = r;
 }
 
 // Face slot -> face index and node coordinates; false for solid positions.
@@ -513,8 +513,8 @@ __global__ void __launch_bounds__(128) d3q_face_pull_kernel(D3Args<S> a) {
     const long long n = node_index(a, c[0], c[1], c[2]);
     const uint32_t info = a.info[n];
     R f[2][Q];
-    pull<S, R>(a, 0, c[0], c[1], c[2], info, f[0]);
-    pull<S, R>(a, 1, c[0], c[1], c[2], info, f[1]);
+    pull<0, S, R>(a, c[0], c[1], c[2], info, f[0]);
+    pull<1, S, R>(a, c[0], c[1], c[2], info, f[1]);
     face_reconstruct<S>(a, fid, c[0], c[1], c[2], info, f);
     reinterpret_cast<typename Pair<R>::type*>(a.rho)[n] = typename Pair<R>::type{sum19(f[0]), sum19(f[1])};
 }
@@ -617,6 +617,23 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
     }
 }
 
+__device__ __forceinline__ void bar_init(unsigned long long* bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// One tensor copy of the density box that starts at (x, y, z), `bytes` long,
+// completing on phase 0 of `bar`.
+__device__ __forceinline__ void copy_box(const CUtensorMap* map, void* dst, unsigned bytes, int x, int y, int z,
+                                         unsigned long long* bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(smem_addr(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
+        : "memory");
+}
+
 template <typename S>
 __device__ __forceinline__ void adhesion_vector(const D3Args<S>& a, long long n, uint32_t info,
                                                 typename Store<S>::R (&ad)[3]) {
@@ -634,11 +651,19 @@ template <typename R>
 __device__ __forceinline__ void forces(const R* G, R r1, R r2, const R (&g1)[3], const R (&g2)[3], const R (&ad)[3],
                                        const R* body, R (&F1)[3], R (&F2)[3]) {
     // G = {G12, Gw1, Gw2}
-    const R rt = r1 + r2;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        F1[q] = -G[0] * r1 * g2[q] - G[1] * r1 * ad[q] + body[q] * r1 / rt;
-        F2[q] = -G[0] * r2 * g1[q] - G[2] * r2 * ad[q] + body[q] * r2 / rt;
+        F1[q] = -G[0] * r1 * g2[q] - G[1] * r1 * ad[q];
+        F2[q] = -G[0] * r2 * g1[q] - G[2] * r2 * ad[q];
+    }
+    // six divisions that most runs (no body force) do without
+    if (body[0] != (R)0 || body[1] != (R)0 || body[2] != (R)0) {
+        const R rt = r1 + r2;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            F1[q] += body[q] * r1 / rt;
+            F2[q] += body[q] * r2 / rt;
+        }
     }
 }
 
@@ -709,43 +734,76 @@ __device__ __forceinline__ void stage_box(const D3Args<S>& a, int x0, int y0, in
 // 3 CTAs of 256 per SM (80 registers), FP64 1.  Tiles without a fluid node
 // leave before staging.
 template <typename S>
-__global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collide_kernel(D3Args<S> a) {
+__global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
+    d3q_collide_kernel(const __grid_constant__ D3Args<S> a, const __grid_constant__ CUtensorMap rho_map, int use_tma,
+                       int zblock) {
     using R = typename Store<S>::R;
     constexpr int TZ = Tile3<S>::TZ, HN = Tile3<S>::HN, NT = Tile3<S>::NT;
-    __shared__ __align__(16) typename Pair<R>::type s_rr[HN];  // (rho_1, rho_2) of the tile and its halo
-    __shared__ __half2 s_ref[is_half<S>() ? HN : 1];           // FP16 storage: the same rounded to half
+    __shared__ __align__(128) typename Pair<R>::type s_rr[HN];  // (rho_1, rho_2) of the tile and its halo
+    __shared__ __align__(8) unsigned long long s_bar;
+    __shared__ __half2 s_ref[is_half<S>() ? HN : 1];            // FP16 storage: the same rounded to half
     __shared__ R s_rate[2][Q];  // relaxation rates of both components (indexed by component below)
     // component 0's pulled populations, kept for its collision after
     // component 1's (FP32 arithmetic; FP64 pulls them again, its tile would
     // exceed the static shared-memory limit)
     constexpr bool STASH = sizeof(R) == 4;
     __shared__ R s_f0[STASH ? Q : 1][STASH ? NT : 1];
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (zblock + blockIdx.z) * TZ;
     const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
     const bool in_grid = x < a.nx && y < a.ny && z < a.nz;
     const long long n = in_grid ? node_index(a, x, y, z) : 0;
     const uint32_t info = in_grid ? a.info[n] : (uint32_t)INFO3_SOLID;
+    // tiles whose halo lies inside the grid need no wrap / mirror / wall
+    // resolution; with FP16 storage their box is one TMA copy (see the FP32 kernel)
+    const bool inner = x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= a.nx && y0 + TY + 2 <= a.ny &&
+                       z0 + TZ + 2 <= a.nz;
+    const bool tma = is_half<S>() && use_tma && inner && (smem_addr(s_rr) & 127u) == 0u;
+    if (tma && tid == 0) bar_init(&s_bar);
     // a tile without fluid nodes has nothing to stage or collide
     if (!__syncthreads_or(!(info & INFO3_SOLID))) return;
     if (tid < 2 * Q) s_rate[tid / Q][tid % Q] = a.s[tid / Q][tid % Q];
-    // tiles whose halo lies inside the grid need no wrap / mirror / wall resolution
-    const bool inner = x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= a.nx && y0 + TY + 2 <= a.ny &&
-                       z0 + TZ + 2 <= a.nz;
-    stage_box(a, x0, y0, z0, inner, tid, [&](int q, typename Pair<R>::type v) {
-        s_rr[q] = v;
-        if constexpr (is_half<S>()) s_ref[q] = __floats2half2_rn((float)v.x, (float)v.y);
-    });
-    __syncthreads();
+    if (tma) {
+        if (tid == 0) copy_box(&rho_map, s_rr, HN * 8u, x0 - 2, y0 - 2, z0 - 2, &s_bar);
+    } else {
+        stage_box(a, x0, y0, z0, inner, tid, [&](int q, typename Pair<R>::type v) { s_rr[q] = v; });
+    }
+    const int fid = (int)((info >> INFO3_FACE_SHIFT) & 7u);
+    const int nid = (int)((info >> INFO3_NBR_SHIFT) & 7u);
+    // FP16 storage: both components' pulls are in flight while the densities arrive
+    S v0[Q], v1[Q];
+    float ref0 = 0.f, ref1 = 0.f;
+    if (is_half<S>() && fid == 0 && !(info & INFO3_SOLID)) {
+        pull_raw<0>(a, x, y, z, n, info, v0);
+        pull_raw<1>(a, x, y, z, n, info, v1);
+        ref0 = __half2float(a.rref_in[n]);
+        ref1 = __half2float(a.rref_in[a.plane + n]);
+    }
+    if (tma) {
+        if (!bar_wait(&s_bar, 0u) && tid == 0) atomicOr(a.status, STATUS3_TIMEOUT);
+    } else {
+        __syncthreads();
+    }
+    if constexpr (is_half<S>()) {
+        for (int q = tid; q < HN; q += NT) s_ref[q] = __floats2half2_rn((float)s_rr[q].x, (float)s_rr[q].y);
+        __syncthreads();
+    } else if (tma) {
+        __syncthreads();
+    }
     if (info & INFO3_SOLID) return;  // solid, or outside the grid
     const int hc = (threadIdx.x + 2) + HX * ((threadIdx.y + 2) + HY * (threadIdx.z + 2));
     auto site = [&](int dx, int dy, int dz) { return s_rr[hc + dx + HX * (dy + HY * dz)]; };
-    const int fid = (int)((info >> INFO3_FACE_SHIFT) & 7u);
-    const int nid = (int)((info >> INFO3_NBR_SHIFT) & 7u);
     R f[Q];
     R j[3] = {0, 0, 0};
     int slot = -1;
-    if (fid == 0) pull<S, R>(a, 0, x, y, z, info, f);  // loads overlap the stencil below
+    auto decode = [&](const S (&v)[Q], float ref) {
+        static_for<0, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            f[i] = (R)ld_pop(v[i]);
+            if constexpr (is_half<S>()) f[i] += ((R)w36_(i) / (R)36) * ref;
+        });
+    };
+    if (!is_half<S>() && fid == 0) pull<0, S, R>(a, x, y, z, info, f);  // loads overlap the stencil below
     R g1[3], g2[3], ad[3];
     stencil_sums<R>(site, g1, g2);
     adhesion_vector<S>(a, n, info, ad);
@@ -754,13 +812,15 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collid
     forces<R>(a.G, r1, r2, g1, g2, ad, a.body, F1, F2);
     const R rt = r1 + r2;
     if (fid == 0) {
+        if constexpr (is_half<S>()) decode(v0, ref0);
         add_j(f, j);
         if constexpr (STASH)
             static_for<0, Q>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 s_f0[i][tid] = f[i];
             });
-        pull<S, R>(a, 1, x, y, z, info, f);
+        if constexpr (is_half<S>()) decode(v1, ref1);
+        else pull<1, S, R>(a, x, y, z, info, f);
         add_j(f, j);
     } else {
         const FaceDev3& Fc = a.face[fid - 1];
@@ -819,6 +879,13 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collid
         const __half2 r = s_ref[h];
         return k ? __high2float(r) : __low2float(r);
     };
+    // no blocked direction (most nodes): constant offsets, no selects
+    const bool open = (info & 0x7FFFFu) == 0u;
+    auto dest_rho_open = [&](auto I, int k) -> R {
+        constexpr int i = decltype(I)::value;
+        const __half2 r = s_ref[hc + ex_(i) + HX * (ey_(i) + HY * ez_(i))];
+        return k ? __high2float(r) : __low2float(r);
+    };
     if constexpr (is_half<S>()) {
         a.rref_out[n] = __float2half_rn(r1);
         a.rref_out[a.plane + n] = __float2half_rn(r2);
@@ -835,7 +902,7 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collid
                         constexpr int i = decltype(I)::value;
                         f[i] = s_f0[i][tid];
                     });
-                else pull<S, R>(a, 0, x, y, z, info, f);
+                else pull<0, S, R>(a, x, y, z, info, f);
             } else {
                 const R* ff = a.fface + (size_t)slot * 2 * Q;
                 static_for<0, Q>([&](auto I) {
@@ -847,7 +914,8 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS) d3q_collid
         const R rk = k ? r2 : r1;
         const R fx = k ? F2[0] : F1[0], fy = k ? F2[1] : F1[1], fz = k ? F2[2] : F1[2];
         collide<R>(f, rk, u[0], u[1], u[2], fx, fy, fz, s_rate[k]);
-        store_pop<S>(a, k, n, f, dest_rho);
+        if (is_half<S>() && open) store_pop<S>(a, k, n, f, dest_rho_open);
+        else store_pop<S>(a, k, n, f, dest_rho);
     }
 }
 
@@ -858,31 +926,68 @@ __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// Momentum of both components: sums of opposite-pair differences.
-__device__ __forceinline__ void momentum2(const float2 (&f)[Q], float2& jx, float2& jy, float2& jz) {
-    const float2 d7 = vsub(f[7], f[10]), d8 = vsub(f[8], f[9]), d11 = vsub(f[11], f[14]), d12 = vsub(f[12], f[13]),
-                 d15 = vsub(f[15], f[18]), d16 = vsub(f[16], f[17]);
-    jx = vadd(vsub(f[1], f[2]), vadd(vsub(d7, d8), vsub(d11, d12)));
-    jy = vadd(vsub(f[3], f[4]), vadd(vadd(d7, d8), vsub(d15, d16)));
-    jz = vadd(vsub(f[5], f[6]), vadd(vadd(d11, d12), vadd(d15, d16)));
+__device__ __forceinline__ float2 ld_shared2(unsigned addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cp_async4(unsigned dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 
-// Eq. 1 as in collide(), with the 19 rows of T and T^-1 written out over the
+// The 18 moments of both components that the collision needs besides the
+// density, from the populations get(i), with the rows of T written out over the
 // sums and differences of opposite pairs: axis pairs (1,2), (3,4), (5,6), edge
 // pairs (7,10), (8,9) in xy, (11,14), (12,13) in xz, (15,18), (16,17) in yz.
-// s: rates of (e, eps, j, q, nu), the values the 19 diagonal entries take
-// (pi shares eps, m shares q).
-__device__ __forceinline__ void collide2(float2 (&f)[Q], float2 r, float ux, float uy, float uz, float2 Fx, float2 Fy,
-                                         float2 Fz, const float2 (&s)[5]) {
-    const float2 px = vadd(f[1], f[2]), py = vadd(f[3], f[4]), pz = vadd(f[5], f[6]);
-    const float2 p7 = vadd(f[7], f[10]), p8 = vadd(f[8], f[9]), p11 = vadd(f[11], f[14]), p12 = vadd(f[12], f[13]),
-                 p15 = vadd(f[15], f[18]), p16 = vadd(f[16], f[17]);
-    const float2 dx = vsub(f[1], f[2]), dy = vsub(f[3], f[4]), dz = vsub(f[5], f[6]);
-    const float2 d7 = vsub(f[7], f[10]), d8 = vsub(f[8], f[9]), d11 = vsub(f[11], f[14]), d12 = vsub(f[12], f[13]),
-                 d15 = vsub(f[15], f[18]), d16 = vsub(f[16], f[17]);
+struct Moments2 {
+    float2 e, eps, j[3], q[3], xx, pixx, ww, piww, xy, yz, xz, m[3];
+};
+template <typename Get>
+__device__ __forceinline__ void moments2(Get get, Moments2& M) {
+    const float2 f0 = get(0), f1 = get(1), f2 = get(2), f3 = get(3), f4 = get(4), f5 = get(5), f6 = get(6);
+    const float2 px = vadd(f1, f2), py = vadd(f3, f4), pz = vadd(f5, f6);
+    const float2 dx = vsub(f1, f2), dy = vsub(f3, f4), dz = vsub(f5, f6);
+    const float2 f7 = get(7), f10 = get(10), f8 = get(8), f9 = get(9);
+    const float2 p7 = vadd(f7, f10), p8 = vadd(f8, f9), d7 = vsub(f7, f10), d8 = vsub(f8, f9);
+    const float2 f11 = get(11), f14 = get(14), f12 = get(12), f13 = get(13);
+    const float2 p11 = vadd(f11, f14), p12 = vadd(f12, f13), d11 = vsub(f11, f14), d12 = vsub(f12, f13);
+    const float2 f15 = get(15), f18 = get(18), f16 = get(16), f17 = get(17);
+    const float2 p15 = vadd(f15, f18), p16 = vadd(f16, f17), d15 = vsub(f15, f18), d16 = vsub(f16, f17);
     const float2 sxy = vadd(p7, p8), sxz = vadd(p11, p12), syz = vadd(p15, p16);
     const float2 sa = vadd(px, vadd(py, pz)), se = vadd(vadd(sxy, sxz), syz);
+    M.e = vfma(vc(-30.f), f0, vfma(vc(-11.f), sa, vmul(vc(8.f), se)));
+    M.eps = vfma(vc(12.f), f0, vfma(vc(-4.f), sa, se));
+    const float2 exy = vsub(d7, d8), exz = vsub(d11, d12), eyx = vadd(d7, d8), eyz = vsub(d15, d16),
+                 ezx = vadd(d11, d12), ezy = vadd(d15, d16);
+    const float2 jx = vadd(exy, exz), jy = vadd(eyx, eyz), jz = vadd(ezx, ezy);
+    M.j[0] = vadd(dx, jx);
+    M.j[1] = vadd(dy, jy);
+    M.j[2] = vadd(dz, jz);
+    M.q[0] = vfma(vc(-4.f), dx, jx);
+    M.q[1] = vfma(vc(-4.f), dy, jy);
+    M.q[2] = vfma(vc(-4.f), dz, jz);
+    const float2 ax = vsub(vmul(vc(2.f), px), vadd(py, pz)), exx = vfma(vc(-2.f), syz, vadd(sxy, sxz));
+    M.xx = vadd(ax, exx);
+    M.pixx = vfma(vc(-2.f), ax, exx);
+    const float2 aw = vsub(py, pz), ew = vsub(sxy, sxz);
+    M.ww = vadd(aw, ew);
+    M.piww = vfma(vc(-2.f), aw, ew);
+    M.xy = vsub(p7, p8);
+    M.yz = vsub(p15, p16);
+    M.xz = vsub(p11, p12);
+    M.m[0] = vsub(exy, exz);
+    M.m[1] = vsub(eyz, eyx);
+    M.m[2] = vsub(ezx, ezy);
+}
+
+// Eq. 1 as in collide(), from the moments; put(i, value to add) per direction.
+// s: rates of (e, eps, j, q, nu), the values the 19 diagonal entries take (pi
+// shares eps, m shares q).
+template <typename Put>
+__device__ __forceinline__ void collide2(const Moments2& M, float2 r, float ux, float uy, float uz,
+                                         const float2 (&F)[3], const float2 (&s)[5], Put put) {
     const float2 U = vc(ux), V = vc(uy), W = vc(uz);
+    const float2 Fx = F[0], Fy = F[1], Fz = F[2];
     const float xx = ux * ux, yy = uy * uy, zz = uz * uz, uu = xx + yy + zz;
     const float2 uF = vfma(U, Fx, vfma(V, Fy, vmul(W, Fz)));
     const float2 half = vc(0.5f);
@@ -893,93 +998,90 @@ __device__ __forceinline__ void collide2(float2 (&f)[Q], float2 r, float ux, flo
         ns[q] = vmul(vc(-1.f), s[q]);
     }
     // g_r = (-s (m - m^eq) + (1 - s/2) F_m) / |row|^2
-    const float2 me = vfma(vc(-30.f), f[0], vfma(vc(-11.f), sa, vmul(vc(8.f), se)));
-    const float2 ge = vmul(vc(1.f / 2394.f), vfma(ns[0], vsub(me, vmul(r, vc(19.f * uu - 11.f))),
+    const float2 ge = vmul(vc(1.f / 2394.f), vfma(ns[0], vsub(M.e, vmul(r, vc(19.f * uu - 11.f))),
                                                   vmul(h[0], vmul(vc(38.f), uF))));
-    const float2 mp = vfma(vc(12.f), f[0], vfma(vc(-4.f), sa, se));
-    const float2 gp = vmul(vc(1.f / 252.f), vfma(ns[1], vsub(mp, vmul(r, vc(3.f - 5.5f * uu))),
+    const float2 gp = vmul(vc(1.f / 252.f), vfma(ns[1], vsub(M.eps, vmul(r, vc(3.f - 5.5f * uu))),
                                                  vmul(h[1], vmul(vc(-11.f), uF))));
-    const float2 exy = vsub(d7, d8), exz = vsub(d11, d12), eyx = vadd(d7, d8), eyz = vsub(d15, d16),
-                 ezx = vadd(d11, d12), ezy = vadd(d15, d16);
-    const float2 jx = vadd(exy, exz), jy = vadd(eyx, eyz), jz = vadd(ezx, ezy);
     const float2 rux = vmul(r, U), ruy = vmul(r, V), ruz = vmul(r, W);
     const float2 c10 = vc(0.1f), c40 = vc(1.f / 40.f), t23 = vc(2.f / 3.f);
-    const float2 gjx = vmul(c10, vfma(ns[2], vsub(vadd(dx, jx), rux), vmul(h[2], Fx)));
-    const float2 gjy = vmul(c10, vfma(ns[2], vsub(vadd(dy, jy), ruy), vmul(h[2], Fy)));
-    const float2 gjz = vmul(c10, vfma(ns[2], vsub(vadd(dz, jz), ruz), vmul(h[2], Fz)));
+    const float2 gjx = vmul(c10, vfma(ns[2], vsub(M.j[0], rux), vmul(h[2], Fx)));
+    const float2 gjy = vmul(c10, vfma(ns[2], vsub(M.j[1], ruy), vmul(h[2], Fy)));
+    const float2 gjz = vmul(c10, vfma(ns[2], vsub(M.j[2], ruz), vmul(h[2], Fz)));
     // q^eq = -2/3 rho u, its forcing -2/3 F
     const float2 hq = vmul(vmul(vc(-1.f), t23), h[3]);
-    const float2 gqx = vmul(c40, vfma(ns[3], vfma(t23, rux, vfma(vc(-4.f), dx, jx)), vmul(hq, Fx)));
-    const float2 gqy = vmul(c40, vfma(ns[3], vfma(t23, ruy, vfma(vc(-4.f), dy, jy)), vmul(hq, Fy)));
-    const float2 gqz = vmul(c40, vfma(ns[3], vfma(t23, ruz, vfma(vc(-4.f), dz, jz)), vmul(hq, Fz)));
+    const float2 gqx = vmul(c40, vfma(ns[3], vfma(t23, rux, M.q[0]), vmul(hq, Fx)));
+    const float2 gqy = vmul(c40, vfma(ns[3], vfma(t23, ruy, M.q[1]), vmul(hq, Fy)));
+    const float2 gqz = vmul(c40, vfma(ns[3], vfma(t23, ruz, M.q[2]), vmul(hq, Fz)));
     // 3p_xx and 3pi_xx (equilibrium and forcing of pi: -1/2 of p's)
-    const float2 ax = vsub(vmul(vc(2.f), px), vadd(py, pz)), exx = vfma(vc(-2.f), syz, vadd(sxy, sxz));
     const float2 qxx = vmul(r, vc(2.f * xx - yy - zz));
     const float2 fxx = vmul(vc(2.f), vsub(vmul(vmul(vc(2.f), U), Fx), vfma(V, Fy, vmul(W, Fz))));
-    const float2 gxx = vmul(vc(1.f / 36.f), vfma(ns[4], vsub(vadd(ax, exx), qxx), vmul(h[4], fxx)));
-    const float2 gyx = vmul(vc(1.f / 72.f), vfma(ns[1], vfma(half, qxx, vfma(vc(-2.f), ax, exx)),
-                                                 vmul(h[1], vmul(vc(-0.5f), fxx))));
+    const float2 gxx = vmul(vc(1.f / 36.f), vfma(ns[4], vsub(M.xx, qxx), vmul(h[4], fxx)));
+    const float2 gyx = vmul(vc(1.f / 72.f), vfma(ns[1], vfma(half, qxx, M.pixx), vmul(h[1], vmul(vc(-0.5f), fxx))));
     // p_ww and pi_ww
-    const float2 aw = vsub(py, pz), ew = vsub(sxy, sxz);
     const float2 qww = vmul(r, vc(yy - zz)), fww = vmul(vc(2.f), vsub(vmul(V, Fy), vmul(W, Fz)));
-    const float2 gww = vmul(vc(1.f / 12.f), vfma(ns[4], vsub(vadd(aw, ew), qww), vmul(h[4], fww)));
-    const float2 gyw = vmul(vc(1.f / 24.f), vfma(ns[1], vfma(half, qww, vfma(vc(-2.f), aw, ew)),
-                                                 vmul(h[1], vmul(vc(-0.5f), fww))));
+    const float2 gww = vmul(vc(1.f / 12.f), vfma(ns[4], vsub(M.ww, qww), vmul(h[4], fww)));
+    const float2 gyw = vmul(vc(1.f / 24.f), vfma(ns[1], vfma(half, qww, M.piww), vmul(h[1], vmul(vc(-0.5f), fww))));
     // p_xy, p_yz, p_xz
     const float2 c4 = vc(0.25f);
-    const float2 gxy = vmul(c4, vfma(ns[4], vsub(vsub(p7, p8), vmul(rux, V)), vmul(h[4], vfma(U, Fy, vmul(V, Fx)))));
-    const float2 gyz = vmul(c4, vfma(ns[4], vsub(vsub(p15, p16), vmul(ruy, W)), vmul(h[4], vfma(V, Fz, vmul(W, Fy)))));
-    const float2 gxz = vmul(c4, vfma(ns[4], vsub(vsub(p11, p12), vmul(rux, W)), vmul(h[4], vfma(U, Fz, vmul(W, Fx)))));
+    const float2 gxy = vmul(c4, vfma(ns[4], vsub(M.xy, vmul(rux, V)), vmul(h[4], vfma(U, Fy, vmul(V, Fx)))));
+    const float2 gyz = vmul(c4, vfma(ns[4], vsub(M.yz, vmul(ruy, W)), vmul(h[4], vfma(V, Fz, vmul(W, Fy)))));
+    const float2 gxz = vmul(c4, vfma(ns[4], vsub(M.xz, vmul(rux, W)), vmul(h[4], vfma(U, Fz, vmul(W, Fx)))));
     // m_x, m_y, m_z (no equilibrium, no forcing)
     const float2 n8 = vmul(vc(0.125f), ns[3]);
-    const float2 gmx = vmul(n8, vsub(exy, exz)), gmy = vmul(n8, vsub(eyz, eyx)), gmz = vmul(n8, vsub(ezx, ezy));
+    const float2 gmx = vmul(n8, M.m[0]), gmy = vmul(n8, M.m[1]), gmz = vmul(n8, M.m[2]);
     // back: f_i += even + odd, f_ibar += even - odd
-    auto put = [&](int i, int o, float2 ev, float2 od) {
-        f[i] = vadd(f[i], vadd(ev, od));
-        f[o] = vadd(f[o], vsub(ev, od));
+    auto both = [&](int i, int o, float2 ev, float2 od) {
+        put(i, vadd(ev, od));
+        put(o, vsub(ev, od));
     };
-    f[0] = vadd(f[0], vfma(vc(-30.f), ge, vmul(vc(12.f), gp)));
+    put(0, vfma(vc(-30.f), ge, vmul(vc(12.f), gp)));
     const float2 ea = vfma(vc(-11.f), ge, vmul(vc(-4.f), gp)), ee = vfma(vc(8.f), ge, gp);
     const float2 axx = vfma(vc(-2.f), gyx, gxx), aww = vfma(vc(-2.f), gyw, gww);
-    put(1, 2, vfma(vc(2.f), axx, ea), vfma(vc(-4.f), gqx, gjx));
+    both(1, 2, vfma(vc(2.f), axx, ea), vfma(vc(-4.f), gqx, gjx));
     const float2 eb = vsub(ea, axx);
-    put(3, 4, vadd(eb, aww), vfma(vc(-4.f), gqy, gjy));
-    put(5, 6, vsub(eb, aww), vfma(vc(-4.f), gqz, gjz));
+    both(3, 4, vadd(eb, aww), vfma(vc(-4.f), gqy, gjy));
+    both(5, 6, vsub(eb, aww), vfma(vc(-4.f), gqz, gjz));
     const float2 Jx = vadd(gjx, gqx), Jy = vadd(gjy, gqy), Jz = vadd(gjz, gqz);
     const float2 bxx = vadd(gxx, gyx), bww = vadd(gww, gyw), e1 = vadd(ee, bxx);
     {
         const float2 A = vadd(Jx, gmx), B = vsub(Jy, gmy), e = vadd(e1, bww);
-        put(7, 10, vadd(e, gxy), vadd(A, B));
-        put(8, 9, vsub(e, gxy), vsub(B, A));
+        both(7, 10, vadd(e, gxy), vadd(A, B));
+        both(8, 9, vsub(e, gxy), vsub(B, A));
     }
     {
         const float2 A = vsub(Jx, gmx), B = vadd(Jz, gmz), e = vsub(e1, bww);
-        put(11, 14, vadd(e, gxz), vadd(A, B));
-        put(12, 13, vsub(e, gxz), vsub(B, A));
+        both(11, 14, vadd(e, gxz), vadd(A, B));
+        both(12, 13, vsub(e, gxz), vsub(B, A));
     }
     {
         const float2 A = vadd(Jy, gmy), B = vsub(Jz, gmz), e = vfma(vc(-2.f), bxx, ee);
-        put(15, 18, vadd(e, gyz), vadd(A, B));
-        put(16, 17, vsub(e, gyz), vsub(B, A));
+        both(15, 18, vadd(e, gyz), vadd(A, B));
+        both(16, 17, vsub(e, gyz), vsub(B, A));
     }
 }
 
 // FP32: the same step as d3q_collide_kernel with both components of a node in
-// the two lanes of packed FP32x2 instructions: one pass of about half the
-// instructions, nothing parked in shared memory between two collisions, and all
-// 38 pulls of a node issued before the density box is waited for (16 warps x 38
-// loads in flight per SM at 126 registers).  512x96x96 co-flow device: 330 ->
-// 280 us for the collision; the whole step 530 -> 435 us with the graph branches.
+// the two lanes of packed FP32x2 instructions (half the instructions).  All 38
+// pulls of a node go straight to shared memory (cp.async) before the density
+// box is waited for, and are read from there twice, for the moments and for the
+// result: 80 registers and three CTAs of 256 per SM instead of two at 126 with
+// the populations in registers (265 against 277 us on the 512x96x96 co-flow
+// device; one component after the other, 64 registers: 330).  The rest is load
+// latency and shared-memory throughput (l1tex 58 %, DRAM 51 %); the step went
+// from 530 to 408 us.
 __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
     d3q_collide_f32_kernel(const __grid_constant__ D3Args<float> a, const __grid_constant__ CUtensorMap rho_map,
-                           int use_tma) {
-    constexpr int TZ = Tile3<float>::TZ, HN = Tile3<float>::HN;
+                           int use_tma, int zblock) {
+    constexpr int TZ = Tile3<float>::TZ, HN = Tile3<float>::HN, NT = Tile3<float>::NT;
     // (rho_1, rho_2) of the tile and its halo, psi = 0 at solids; 128-byte
-    // aligned: an interior tile receives it as one tensor copy
-    __shared__ __align__(128) float2 s_rr[HN];
+    // aligned: an interior tile receives it as one tensor copy.  Behind it the
+    // pulled populations [Q][NT] as component pairs.
+    extern __shared__ __align__(128) unsigned char s_dyn[];
+    float2* s_rr = reinterpret_cast<float2*>(s_dyn);
     __shared__ __align__(8) unsigned long long s_bar;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (zblock + blockIdx.z) * TZ;
     const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
+    const unsigned s_f = smem_addr(s_rr + HN) + 8u * (unsigned)tid;
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
     const bool in_grid = x < a.nx && y < a.ny && z < a.nz;
     const long long n = in_grid ? node_index(a, x, y, z) : 0;
@@ -991,43 +1093,29 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
     const bool inner = x0 >= 2 && y0 >= 2 && z0 >= 2 && x0 + TX + 2 <= a.nx && y0 + TY + 2 <= a.ny &&
                        z0 + TZ + 2 <= a.nz;
     const bool tma = use_tma && inner && (smem_addr(s_rr) & 127u) == 0u;
-    if (tma && tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_bar)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (tma && tid == 0) bar_init(&s_bar);
     // a tile without fluid nodes has nothing to stage or collide
     if (!__syncthreads_or(!(info & INFO3_SOLID))) return;
     if (tma) {
-        if (tid == 0) {
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)),
-                         "r"((unsigned)(HN * sizeof(float2)))
-                         : "memory");
-            asm volatile(
-                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
-                "[%1, {%2, %3, %4}], [%5];" ::"r"(smem_addr(s_rr)),
-                "l"(&rho_map), "r"(x0 - 2), "r"(y0 - 2), "r"(z0 - 2), "r"(smem_addr(&s_bar))
-                : "memory");
-        }
+        if (tid == 0) copy_box(&rho_map, s_rr, HN * 8u, x0 - 2, y0 - 2, z0 - 2, &s_bar);
     } else {
         stage_box(a, x0, y0, z0, inner, tid, [&](int q, float2 v) { s_rr[q] = v; });
     }
     const int fid = (int)((info >> INFO3_FACE_SHIFT) & 7u);
     const int nid = (int)((info >> INFO3_NBR_SHIFT) & 7u);
-    // all 38 pulls are in flight while the densities arrive
-    float2 f[Q];
+    // all 38 pulls go to shared memory while the densities arrive
     int slot = -1;
     if (!(info & INFO3_SOLID)) {
         if (fid == 0) {
-            float v0[Q], v1[Q];
-            pull_raw<float>(a, 0, x, y, z, n, info, v0);
-            pull_raw<float>(a, 1, x, y, z, n, info, v1);
-#pragma unroll
-            for (int i = 0; i < Q; ++i) f[i] = make_float2(v0[i], v1[i]);
+            pull_sources<0, 2>(a, x, y, z, n, info,
+                                [&](int k, int i, const float* p) { cp_async4(s_f + 8u * NT * i + 4u * k, p); });
         } else {
             slot = face_slot(a.face[fid - 1], x, y, z);
             const float* ff = a.fface + (size_t)slot * 2 * Q;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) f[i] = make_float2(ff[i], ff[Q + i]);
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < Q; ++i) cp_async4(s_f + 8u * NT * i + 4u * k, ff + k * Q + i);
         }
     }
     if (tma) {
@@ -1058,15 +1146,15 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
         }
         if (Fc.kind == FACE3_OUTLET) return;  // finished by d3q_outlet_kernel
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    auto pop = [&](int i) { return ld_shared2(s_f + 8u * NT * i); };
+    Moments2 M;
+    moments2(pop, M);
     float u[3];
-    {
-        float2 j[3];
-        momentum2(f, j[0], j[1], j[2]);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const float2 t = vfma(vc(0.5f), F[q], j[q]);
-            u[q] = (t.x + t.y) * inv;
-        }
+    for (int q = 0; q < 3; ++q) {
+        const float2 t = vfma(vc(0.5f), F[q], M.j[q]);
+        u[q] = (t.x + t.y) * inv;
     }
     if (nid != 0) {
         const FaceDev3& Fc = a.face[nid - 1];
@@ -1099,13 +1187,12 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
     const float2 s[5] = {make_float2(a.s[0][1], a.s[1][1]), make_float2(a.s[0][2], a.s[1][2]),
                          make_float2(a.s[0][3], a.s[1][3]), make_float2(a.s[0][4], a.s[1][4]),
                          make_float2(a.s[0][9], a.s[1][9])};
-    collide2(f, r, u[0], u[1], u[2], F[0], F[1], F[2], s);
     const unsigned off = (unsigned)n * 4u;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        st_at(a.dst[0][i], off, f[i].x);
-        st_at(a.dst[1][i], off, f[i].y);
-    }
+    collide2(M, r, u[0], u[1], u[2], F, s, [&](int i, float2 d) {
+        const float2 v = vadd(pop(i), d);
+        st_at(a.dst[0][i], off, v.x);
+        st_at(a.dst[1][i], off, v.y);
+    });
 }
 
 // One thread per outlet slot: the outlet node's velocity with the normal
@@ -1309,12 +1396,23 @@ cudaError_t launch_macros(const R* rho_pairs, const R* umac, const uint32_t* inf
     return cudaGetLastError();
 }
 
+constexpr int GRID_Z = 65535;  // largest z extent of a launch grid: longer grids take several launches
+
 template <typename S>
 static cudaError_t launch_pull(const D3Args<S>& a, cudaStream_t st) {
     const dim3 blk(32, 4, 2);
-    const dim3 grd((a.nx + 31) / 32, (a.ny + 3) / 4, (a.nz + 1) / 2);
-    d3q_pull_kernel<S><<<grd, blk, 0, st>>>(a);
+    for (int z = 0; z < a.nz; z += GRID_Z) {
+        const dim3 grd((a.nx + 31) / 32, (a.ny + 3) / 4, std::min(GRID_Z, a.nz - z));
+        d3q_pull_kernel<S><<<grd, blk, 0, st>>>(a, z);
+    }
     return cudaGetLastError();
+}
+
+constexpr size_t COLLIDE_F32_SMEM = (size_t)(Tile3<float>::HN + Q * Tile3<float>::NT) * sizeof(float2);
+
+cudaError_t prepare_kernels() {
+    return cudaFuncSetAttribute(d3q_collide_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)COLLIDE_F32_SMEM);
 }
 
 template <typename S>
@@ -1322,11 +1420,14 @@ static cudaError_t launch_collide(const D3Args<S>& a, const CUtensorMap* rho_map
     static const CUtensorMap kNoMap{};
     constexpr int TZ = Tile3<S>::TZ;
     const dim3 blk(TX, TY, TZ);
-    const dim3 grd((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + TZ - 1) / TZ);
-    if constexpr (std::is_same<S, float>::value)
-        d3q_collide_f32_kernel<<<grd, blk, 0, st>>>(a, rho_map ? *rho_map : kNoMap, rho_map ? 1 : 0);
-    else
-        d3q_collide_kernel<S><<<grd, blk, 0, st>>>(a);
+    const int nzb = (a.nz + TZ - 1) / TZ;
+    for (int z = 0; z < nzb; z += GRID_Z) {
+        const dim3 grd((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, std::min(GRID_Z, nzb - z));
+        if constexpr (std::is_same<S, float>::value)
+            d3q_collide_f32_kernel<<<grd, blk, COLLIDE_F32_SMEM, st>>>(a, rho_map ? *rho_map : kNoMap, rho_map ? 1 : 0, z);
+        else
+            d3q_collide_kernel<S><<<grd, blk, 0, st>>>(a, rho_map ? *rho_map : kNoMap, rho_map ? 1 : 0, z);
+    }
     return cudaGetLastError();
 }
 

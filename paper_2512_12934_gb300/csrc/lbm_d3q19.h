@@ -28,7 +28,7 @@ enum { FACE3_INLET = 1, FACE3_OUTLET = 2 };
 // status word bits of a D3Q19 step: non-finite result; a bounded wait on a
 // tensor copy that ran out
 constexpr unsigned STATUS3_DIVERGED = 1u, STATUS3_TIMEOUT = 2u;
-// density box of one FP32 collide tile (32 x 4 x 2 nodes) and its 2-node halo,
+// density box of one collide tile (32 x 4 x 2 nodes) and its 2-node halo,
 // the tensor-copy box of the density field
 constexpr int RHO_BOX3_X = 36, RHO_BOX3_Y = 8, RHO_BOX3_Z = 6;
 // device scalars of the open boundaries (ping-pong per step)
@@ -106,8 +106,11 @@ struct D3Args {
     R s[2][Q];
 };
 
+// Kernel attributes on the current device (once per context, before any launch).
+cudaError_t prepare_kernels();
+
 // One step.  rho_map: tensor map of the density field as 8-byte (rho_1, rho_2)
-// pairs (FP32 contexts; NULL: the collide kernel stages every density box with
+// pairs (FP32 arithmetic; NULL: the collide kernel stages every density box with
 // loads).  mid_a, mid_b (may be NULL): recorded after the pulls and after the
 // collision.
 template <typename S>

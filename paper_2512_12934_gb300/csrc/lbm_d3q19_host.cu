@@ -93,8 +93,8 @@ struct Ctx3 {
     double* scal[2] = {nullptr, nullptr};
     unsigned int* status = nullptr;
     unsigned int* hstatus = nullptr;  // pinned: the status word of the last macroscopic read
-    // FP32: tensor map of the density field as 8-byte (rho_1, rho_2) pairs,
-    // box (36, 8, 8) = one collide tile and its halo
+    // FP32 arithmetic: tensor map of the density field as 8-byte (rho_1, rho_2) pairs,
+    // box (36, 8, 6) = one collide tile and its halo
     CUtensorMap rho_map{};
     int have_rho_map = 0;
     double* mass_partial = nullptr;
@@ -348,7 +348,7 @@ lbm_status upload_state(Ctx3* c, const double* rho_init, const double* u_init) {
     return LBM_OK;
 }
 
-// FP32 contexts: tensor map of the density field ([plane] pairs of floats as
+// FP32 arithmetic: tensor map of the density field ([plane] pairs of floats as
 // 8-byte elements over x, y, z) for the collide kernel's one-copy staging of
 // interior tiles.  Without the driver entry point the kernel stages with
 // loads instead (same values).
@@ -357,7 +357,7 @@ void make_rho_map(Ctx3* c) {
                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
     c->have_rho_map = 0;
-    if (c->precision != LBM_FP32) return;
+    if (c->precision == LBM_FP64) return;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q{};
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
@@ -621,7 +621,7 @@ lbm_status create(const lbm_grid* g, const lbm_params* p, const lbm_open_bc* bcs
             }
 
     // device allocations
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = prepare_kernels();
     auto alloc = [&](void** ptr, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(ptr, std::max<size_t>(bytes, 16));
     };
