@@ -341,8 +341,8 @@ typedef struct lbm_batch lbm_batch;
  * batch work is enqueued on (NULL = legacy default stream). */
 lbm_status lbm_batch_create(lbm_ctx* const* members, int n, void* cuda_stream, lbm_batch** out);
 
-/* Enqueue nsteps steps of every member (runs of 32 steps replay captured
- * CUDA graphs); members' macroscopic fields are written by the last one. */
+/* Enqueue nsteps steps of every member (runs of 32, 8 and 2 steps replay
+ * captured CUDA graphs); members' macroscopic fields are written by the last one. */
 lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps);
 
 /* Wait for the batch stream; LBM_ERR_DIVERGED if any member diverged,
@@ -371,7 +371,7 @@ lbm_status lbm_batch_set_graph_mode(lbm_batch* b, int use_graphs);
 /* How a batch step call runs on the GPU.
  *  LBM_SCHEDULE_GRAPHS (default): per time step, one launch for the fast
  *    tile list and one for the general list, replayed from captured CUDA
- *    graphs in runs of 32 steps.
+ *    graphs in runs of 32, 8 and 2 steps.
  *  LBM_SCHEDULE_PERSISTENT (FP32 storage only): one cooperative launch per
  *    run of up to 1024 steps.  Its CTAs (as many as fit on the GPU at once,
  *    at most one per tile) walk the concatenated tile descriptors of all

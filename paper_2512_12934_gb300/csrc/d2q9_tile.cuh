@@ -1154,12 +1154,12 @@ __device__ __forceinline__ void adhesion_sum(SOL sol, R& ax, R& ay) {
 
 // Eq. 1 for one component of one node in moment space (T of Eq. 3, S of
 // Eq. 4), delta form: post-collision moment increments -s (m - m_eq) +
-// (1 - s/2) F_m with the analytic equilibrium and forcing moments, then the
+// h F_m (h = 1 - s/2) with the analytic equilibrium and forcing moments, then the
 // back-transform T^-1 = T^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4,
 // 1/4) added to the populations.  uu3 = 3 |u|^2.
 template <typename R>
-__device__ __forceinline__ void collide_scalar(const R* s, R r, R fx, R fy, R ux, R uy, R uu3, const R (&g)[9],
-                                               R (&o)[9]) {
+__device__ __forceinline__ void collide_scalar(const R* s, const R* h, R r, R fx, R fy, R ux, R uy, R uu3,
+                                               const R (&g)[9], R (&o)[9]) {
     const R d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d86 = g[8] - g[6];
     const R a13 = g[1] + g[3], a24 = g[2] + g[4], a57 = g[5] + g[7], a68 = g[6] + g[8];
     const R sa = a13 + a24, sd = a57 + a68;
@@ -1169,14 +1169,14 @@ __device__ __forceinline__ void collide_scalar(const R* s, R r, R fx, R fy, R ux
     const R mjy = d24 + (d57 - d86), mqy = (d57 - d86) - R(2) * d24;
     const R mxx = a13 - a24, mxy = a57 - a68;
     const R uF = ux * fx + uy * fy;
-    const R de = -s[1] * (me - r * (uu3 - R(2))) + (R(1) - R(0.5) * s[1]) * (R(6) * uF);
-    const R dp = -s[2] * (mp - r * (R(1) - uu3)) + (R(1) - R(0.5) * s[2]) * (R(-6) * uF);
-    const R djx = -s[3] * (mjx - r * ux) + (R(1) - R(0.5) * s[3]) * fx;
-    const R dqx = -s[4] * (mqx + r * ux) - (R(1) - R(0.5) * s[4]) * fx;
-    const R djy = -s[5] * (mjy - r * uy) + (R(1) - R(0.5) * s[5]) * fy;
-    const R dqy = -s[6] * (mqy + r * uy) - (R(1) - R(0.5) * s[6]) * fy;
-    const R dxx = -s[7] * (mxx - r * (ux * ux - uy * uy)) + (R(1) - R(0.5) * s[7]) * (R(2) * (ux * fx - uy * fy));
-    const R dxy = -s[8] * (mxy - r * ux * uy) + (R(1) - R(0.5) * s[8]) * (ux * fy + uy * fx);
+    const R de = -s[1] * (me - r * (uu3 - R(2))) + h[1] * (R(6) * uF);
+    const R dp = -s[2] * (mp - r * (R(1) - uu3)) + h[2] * (R(-6) * uF);
+    const R djx = -s[3] * (mjx - r * ux) + h[3] * fx;
+    const R dqx = -s[4] * (mqx + r * ux) - h[4] * fx;
+    const R djy = -s[5] * (mjy - r * uy) + h[5] * fy;
+    const R dqy = -s[6] * (mqy + r * uy) - h[6] * fy;
+    const R dxx = -s[7] * (mxx - r * (ux * ux - uy * uy)) + h[7] * (R(2) * (ux * fx - uy * fy));
+    const R dxy = -s[8] * (mxy - r * ux * uy) + h[8] * (ux * fy + uy * fx);
     const R ce = de * R(1.0 / 36.0), cp = dp * R(1.0 / 36.0);
     const R cjx = djx * R(1.0 / 6.0), cqx = dqx * R(1.0 / 12.0);
     const R cjy = djy * R(1.0 / 6.0), cqy = dqy * R(1.0 / 12.0);
@@ -1193,6 +1193,51 @@ __device__ __forceinline__ void collide_scalar(const R* s, R r, R fx, R fy, R ux
     o[6] = g[6] + (dg - px + py - cxy);
     o[7] = g[7] + (dg - px - py + cxy);
     o[8] = g[8] + (dg + px - py - cxy);
+}
+
+// The same in FP64, which GB300 executes at two operations per clock and SM: the
+// FP64 pipe bounds FP64 steps (84 % busy), so the operations are what counts.
+// With T^-1's normalisation and the forcing constants folded into the
+// coefficients (FoldedRates) and shared sums in the back-transform a component
+// takes 84 FP64 operations instead of about 108.
+__device__ __forceinline__ void collide_folded(const double* A, const double* B, double r, double fx, double fy,
+                                               double ux, double uy, double uu3, const double (&g)[9],
+                                               double (&o)[9]) {
+    const double d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d86 = g[8] - g[6];
+    const double a13 = g[1] + g[3], a24 = g[2] + g[4], a57 = g[5] + g[7], a68 = g[6] + g[8];
+    const double sa = a13 + a24, sd = a57 + a68, dp = d57 + d86, dm = d57 - d86;
+    const double me = (2.0 * sd - sa) - 4.0 * g[0], mp = (sd - 2.0 * sa) + 4.0 * g[0];
+    const double rx = r * ux, ry = r * uy;
+    const double uF = ux * fx + uy * fy;
+    const double ce = A[1] * (me - r * (uu3 - 2.0)) + B[1] * uF;
+    const double cp = A[2] * (mp - r * (1.0 - uu3)) + B[2] * uF;
+    const double cjx = A[3] * ((d13 + dp) - rx) + B[3] * fx, cqx = A[4] * ((dp - 2.0 * d13) + rx) + B[4] * fx;
+    const double cjy = A[5] * ((d24 + dm) - ry) + B[5] * fy, cqy = A[6] * ((dm - 2.0 * d24) + ry) + B[6] * fy;
+    const double cxx = A[7] * ((a13 - a24) - r * (ux * ux - uy * uy)) + B[7] * (ux * fx - uy * fy);
+    const double cxy = A[8] * ((a57 - a68) - r * (ux * uy)) + B[8] * (ux * fy + uy * fx);
+    const double ea = -ce - 2.0 * cp, dg = 2.0 * ce + cp;
+    const double bx = cjx - 2.0 * cqx, by = cjy - 2.0 * cqy;
+    const double px = cjx + cqx, py = cjy + cqy;
+    const double ex = ea + cxx, ey = ea - cxx, ep = dg + cxy, em = dg - cxy, sp = px + py, sm = px - py;
+    o[0] = g[0] + 4.0 * (cp - ce);
+    o[1] = g[1] + (ex + bx);
+    o[2] = g[2] + (ey + by);
+    o[3] = g[3] + (ex - bx);
+    o[4] = g[4] + (ey - by);
+    o[5] = g[5] + (ep + sp);
+    o[6] = g[6] + (em - sm);
+    o[7] = g[7] + (ep - sp);
+    o[8] = g[8] + (em + sm);
+}
+
+// Collision of component k in the step's arithmetic.
+template <typename S, typename R>
+__device__ __forceinline__ void collide_one(const D2Args<S, R>& a, int k, R r, R fx, R fy, R ux, R uy, R uu3,
+                                            const R (&g)[9], R (&o)[9]) {
+    if constexpr (std::is_same<R, double>::value)
+        collide_folded(a.fold.a[k], a.fold.b[k], r, fx, fy, ux, uy, uu3, g, o);
+    else
+        collide_scalar<R>(a.s[k], a.h[k], r, fx, fy, ux, uy, uu3, g, o);
 }
 
 // One tile of one step.  bxy = bx | by << 16; bflags = BLOCK_* flags; strips
@@ -1232,18 +1277,30 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
         // ---- Eq. 10: 24-point 8th-order gradient of the other component ----
         R g0x, g0y, g1x, g1y;
         psi_gradient<R>([&](int dy, int dx) { return sm.rr[ty + 2 + dy][tx + 2 + dx]; }, g0x, g0y, g1x, g1y);
-        // ---- Eq. 11: adhesion, only in tiles that see a solid site ----
-        R ax = R(0), ay = R(0);
-        if (bflags & BLOCK_SOLID)
-            adhesion_sum<R>([&](int dy, int dx) { return sm.sol[ty + 2 + dy][tx + 2 + dx]; }, ax, ay);
         const R rt = rho0 + rho1;
         const R inv_rt = R(1) / rt;
-        R gw0, gw1;
-        adhesion_coeffs(a, rho0, rho1, gw0, gw1);
-        Fx0 = -a.G12 * rho0 * g1x - gw0 * rho0 * ax + a.body[0] * rho0 * inv_rt;
-        Fy0 = -a.G12 * rho0 * g1y - gw0 * rho0 * ay + a.body[1] * rho0 * inv_rt;
-        Fx1 = -a.G12 * rho1 * g0x - gw1 * rho1 * ax + a.body[0] * rho1 * inv_rt;
-        Fy1 = -a.G12 * rho1 * g0y - gw1 * rho1 * ay + a.body[1] * rho1 * inv_rt;
+        // ---- Eq. 11: adhesion, only in tiles that see a solid site (elsewhere
+        // its terms are exact zeros; Eq. 12's coefficients cost two divisions)
+        if (bflags & BLOCK_SOLID) {
+            R ax = R(0), ay = R(0), gw0, gw1;
+            adhesion_sum<R>([&](int dy, int dx) { return sm.sol[ty + 2 + dy][tx + 2 + dx]; }, ax, ay);
+            adhesion_coeffs(a, rho0, rho1, gw0, gw1);
+            Fx0 = -a.G12 * rho0 * g1x - gw0 * rho0 * ax;
+            Fy0 = -a.G12 * rho0 * g1y - gw0 * rho0 * ay;
+            Fx1 = -a.G12 * rho1 * g0x - gw1 * rho1 * ax;
+            Fy1 = -a.G12 * rho1 * g0y - gw1 * rho1 * ay;
+        } else {
+            Fx0 = -a.G12 * rho0 * g1x;
+            Fy0 = -a.G12 * rho0 * g1y;
+            Fx1 = -a.G12 * rho1 * g0x;
+            Fy1 = -a.G12 * rho1 * g0y;
+        }
+        if (a.body_on) {
+            Fx0 += a.body[0] * rho0 * inv_rt;
+            Fy0 += a.body[1] * rho0 * inv_rt;
+            Fx1 += a.body[0] * rho1 * inv_rt;
+            Fy1 += a.body[1] * rho1 * inv_rt;
+        }
         // ---- Eqs. 7, 8: common velocity ----
         const R jx = (jx_of(f[0]) + R(0.5) * Fx0) + (jx_of(f[1]) + R(0.5) * Fx1);
         const R jy = (jy_of(f[0]) + R(0.5) * Fy0) + (jy_of(f[1]) + R(0.5) * Fy1);
@@ -1357,11 +1414,10 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
             const R uu3 = R(3) * (ux * ux + uy * uy);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const R* s = a.s[k];
                 const R r = k == 0 ? rho0 : rho1;
                 const R fx = k == 0 ? Fx0 : Fx1, fy = k == 0 ? Fy0 : Fy1;
                 R o[9];
-                collide_scalar<R>(s, r, fx, fy, ux, uy, uu3, f[k], o);
+                collide_one(a, k, r, fx, fy, ux, uy, uu3, f[k], o);
                 if constexpr (is_half_<S>()) {
                     // encode with the reference density of the node that pulls each value
                     const R own = half_round(r);

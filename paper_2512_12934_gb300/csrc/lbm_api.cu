@@ -47,6 +47,32 @@ void side_normal(int side, int* ox, int* oy) {
 
 }  // namespace
 
+// Step runs are replayed from captured graphs of 32, 8 and 2 steps (even sizes
+// leave the ping-pong parity unchanged), one per starting parity.  The short
+// ones serve the rest of a call: a step launched on its own runs its two tile
+// lists one after the other (49 steps of 640x320 FP64: 17 of them at 200 us
+// instead of 171).
+constexpr int kGraphSizes = 3;
+constexpr int kGraphSteps[kGraphSizes] = {32, 8, 2};
+struct StepGraphs {
+    cudaGraphExec_t exec[kGraphSizes][2] = {};
+    int early[kGraphSizes][2] = {};  // the graph launches its steps early
+    void drop() {
+        for (int q = 0; q < kGraphSizes; ++q)
+            for (int p = 0; p < 2; ++p) {
+                if (exec[q][p]) cudaGraphExecDestroy(exec[q][p]);
+                exec[q][p] = nullptr;
+                early[q][p] = 0;
+            }
+    }
+    bool early_in_use() const {
+        for (int q = 0; q < kGraphSizes; ++q)
+            for (int p = 0; p < 2; ++p)
+                if (exec[q][p] && early[q][p]) return true;
+        return false;
+    }
+};
+
 struct lbm_ctx {
     lbm3::Ctx3* d3 = nullptr;  // non-null: a D3Q19 context (lbm_d3q19_host.cu owns it)
     lbm_grid grid{};
@@ -96,13 +122,12 @@ struct lbm_ctx {
     int64_t step = 0;
     int64_t launches = 0;
     double s[2][9]{};
-    // CUDA-graph replay of step runs: one executable graph per starting parity
+    // CUDA-graph replay of step runs
     int use_graphs = 1;
     cudaStream_t cap_stream = nullptr;
     cudaStream_t side_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    int gexec_early[2] = {0, 0};  // the graph of that parity launches its steps early
+    StepGraphs graphs;
     // sampled per-launch timing
     std::vector<int> h_faceid, h_nbrid;  // per node (unpitched): face id + 1, inward-neighbour face id + 1
     std::vector<uint8_t> host_solid;   // pitched copy of the solid mask
@@ -143,8 +168,6 @@ lbm_status cuda_fail(lbm_ctx* c, cudaError_t e, const char* where) {
         cudaError_t e_ = (call);                                         \
         if (e_ != cudaSuccess) return cuda_fail(c, e_, #call);           \
     } while (0)
-
-constexpr int kGraphSteps = 32;  // even: a replay leaves the ping-pong parity unchanged
 
 // Early-launch step graphs (LBM_SCHEDULE_GRAPHS_EARLY): every edge between
 // two kernel nodes of a captured step graph becomes a programmatic edge that
@@ -206,8 +229,7 @@ constexpr int kMaxSamples = 4096;
 void free_ctx(lbm_ctx* c) {
     if (!c) return;
     if (c->solo) lbm_batch_destroy(c->solo);
-    for (int p = 0; p < 2; ++p)
-        if (c->gexec[p]) cudaGraphExecDestroy(c->gexec[p]);
+    c->graphs.drop();
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->side_stream) cudaStreamDestroy(c->side_stream);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -273,9 +295,19 @@ D2Args<S, R> make_args_par(lbm_ctx* c, int in, bool write_macros) {
     a.Gw[0] = (R)c->params.Gw[0];
     a.Gw[1] = (R)c->params.Gw[1];
     for (int k = 0; k < 2; ++k)
-        for (int r = 0; r < 9; ++r) a.s[k][r] = (R)c->s[k][r];
+        for (int r = 0; r < 9; ++r) {
+            a.s[k][r] = (R)c->s[k][r];
+            a.h[k][r] = R(1) - R(0.5) * a.s[k][r];
+            if constexpr (std::is_same<R, double>::value) {
+                static const double inv[9] = {0, 1.0 / 36, 1.0 / 36, 1.0 / 6, 1.0 / 12, 1.0 / 6, 1.0 / 12, 0.25, 0.25};
+                static const double cf[9] = {0, 6, -6, 1, -1, 1, -1, 2, 1};
+                a.fold.a[k][r] = -a.s[k][r] * inv[r];
+                a.fold.b[k][r] = a.h[k][r] * cf[r] * inv[r];
+            }
+        }
     a.body[0] = (R)c->params.body_force[0];
     a.body[1] = (R)c->params.body_force[1];
+    a.body_on = a.body[0] != R(0) || a.body[1] != R(0);
     return a;
 }
 
@@ -332,10 +364,10 @@ lbm_status launch_one(lbm_ctx* c, bool macros, cudaStream_t st, cudaEvent_t mid 
     return LBM_OK;
 }
 
-// Capture kGraphSteps consecutive steps that start at ping-pong parity `par`.
+// Capture kGraphSteps[size] consecutive steps that start at ping-pong parity `par`.
 template <typename S, typename R>
-lbm_status ensure_graph(lbm_ctx* c, int par) {
-    if (c->gexec[par]) return LBM_OK;
+lbm_status ensure_graph(lbm_ctx* c, int size, int par) {
+    if (c->graphs.exec[size][par]) return LBM_OK;
     if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     if (!c->side_stream) CK(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
     if (!c->ev_fork) CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
@@ -345,7 +377,7 @@ lbm_status ensure_graph(lbm_ctx* c, int par) {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < kGraphSteps && e == cudaSuccess; ++i) {
+    for (int i = 0; i < kGraphSteps[size] && e == cudaSuccess; ++i) {
         e = launch_lists<S, R>(c, false, c->cap_stream, c->side_stream);
         c->cur = 1 - c->cur;
     }
@@ -353,10 +385,11 @@ lbm_status ensure_graph(lbm_ctx* c, int par) {
     c->cur = saved;
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess)
-        e = instantiate_step_graph(g, c->schedule == LBM_SCHEDULE_GRAPHS_EARLY, &c->gexec[par], &c->gexec_early[par]);
+        e = instantiate_step_graph(g, c->schedule == LBM_SCHEDULE_GRAPHS_EARLY, &c->graphs.exec[size][par],
+                                   &c->graphs.early[size][par]);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        c->gexec[par] = nullptr;
+        c->graphs.exec[size][par] = nullptr;
         return cuda_fail(c, e, "step graph capture");
     }
     return LBM_OK;
@@ -365,19 +398,20 @@ lbm_status ensure_graph(lbm_ctx* c, int par) {
 // cnt steps without macro output: graph replays, then single launches.
 template <typename S, typename R>
 lbm_status run_plain(lbm_ctx* c, int64_t cnt) {
-    while (c->use_graphs && cnt >= kGraphSteps) {
-        if (ensure_graph<S, R>(c, c->cur) != LBM_OK) {
-            c->use_graphs = 0;  // capture unavailable: keep launching the same kernel directly
-            cudaGetLastError();
-            break;
+    const int per = (c->nfast > 0) + (c->ngeneral > 0) + (c->nmarch > 0) + (c->chi_same_step ? 1 : 0);
+    for (int size = 0; size < kGraphSizes; ++size)
+        while (c->use_graphs && cnt >= kGraphSteps[size]) {
+            if (ensure_graph<S, R>(c, size, c->cur) != LBM_OK) {
+                c->use_graphs = 0;  // capture unavailable: keep launching the same kernel directly
+                cudaGetLastError();
+                break;
+            }
+            cudaError_t e = cudaGraphLaunch(c->graphs.exec[size][c->cur], c->stream);
+            if (e != cudaSuccess) return cuda_fail(c, e, "step graph launch");
+            c->step += kGraphSteps[size];
+            c->launches += (int64_t)kGraphSteps[size] * per;
+            cnt -= kGraphSteps[size];
         }
-        cudaError_t e = cudaGraphLaunch(c->gexec[c->cur], c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "step graph launch");
-        c->step += kGraphSteps;
-        c->launches += (int64_t)kGraphSteps *
-                       ((c->nfast > 0) + (c->ngeneral > 0) + (c->nmarch > 0) + (c->chi_same_step ? 1 : 0));
-        cnt -= kGraphSteps;
-    }
     for (; cnt > 0; --cnt) {
         lbm_status st = launch_one<S, R>(c, false, c->stream);
         if (st != LBM_OK) return st;
@@ -771,7 +805,7 @@ lbm_status build_tiles(lbm_ctx* c, int v, bool sync_first) {
                 }
             uint8_t fl = 0;
             if (edge) fl |= BLOCK_EDGE;
-            if (near_solid || closed_edge || gen) fl |= BLOCK_SOLID;
+            if (near_solid || closed_edge) fl |= BLOCK_SOLID;
             const int packed = (int)bx | ((int)by << 16);
             int64_t own_fluid = 0;
             for (int yy = std::max(0, y0); yy < std::min(ny, y0 + c->ty); ++yy)
@@ -888,11 +922,7 @@ lbm_status build_tiles(lbm_ctx* c, int v, bool sync_first) {
     c->block_slot = nullptr;
     c->block_strips = nullptr;
     c->partials[0] = c->partials[1] = nullptr;
-    for (int p = 0; p < 2; ++p)
-        if (c->gexec[p]) {
-            cudaGraphExecDestroy(c->gexec[p]);
-            c->gexec[p] = nullptr;
-        }
+    c->graphs.drop();
     CK(cudaMalloc((void**)&c->blocks, blist.size() * sizeof(int) + 4));
     CK(cudaMalloc((void**)&c->block_flags, bflags.size() + 4));
     CK(cudaMalloc((void**)&c->block_slot, slot_all.size() * sizeof(int) + 4));
@@ -1003,8 +1033,7 @@ struct lbm_batch {
     int use_graphs = 1;
     cudaStream_t cap_stream = nullptr, side_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    int gexec_early[2] = {0, 0};
+    StepGraphs graphs;
     int64_t launches = 0;
     // persistent schedule: one cooperative launch per run of up to
     // kPersistSteps steps, grid barriers with bounded waits between steps
@@ -1041,11 +1070,7 @@ void free_batch_lists(lbm_batch* b) {
     b->strips = nullptr;
     b->member = nullptr;
     for (int i = 0; i < 4; ++i) b->args[i] = nullptr;
-    for (int p2 = 0; p2 < 2; ++p2)
-        if (b->gexec[p2]) {
-            cudaGraphExecDestroy(b->gexec[p2]);
-            b->gexec[p2] = nullptr;
-        }
+    b->graphs.drop();
 }
 
 // Concatenate the members' tile lists (fast tiles first, then general tiles)
@@ -1198,8 +1223,8 @@ lbm_status batch_run_persistent(lbm_batch* b, int64_t n) {
 }
 
 template <typename S, typename R>
-lbm_status batch_graph(lbm_batch* b, int par) {
-    if (b->gexec[par]) return LBM_OK;
+lbm_status batch_graph(lbm_batch* b, int size, int par) {
+    if (b->graphs.exec[size][par]) return LBM_OK;
     if (!b->cap_stream) BCK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
     if (!b->side_stream) BCK(cudaStreamCreateWithFlags(&b->side_stream, cudaStreamNonBlocking));
     if (!b->ev_fork) BCK(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
@@ -1209,7 +1234,7 @@ lbm_status batch_graph(lbm_batch* b, int par) {
     cudaGraph_t g = nullptr;
     BCK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < kGraphSteps && e == cudaSuccess; ++i) {
+    for (int i = 0; i < kGraphSteps[size] && e == cudaSuccess; ++i) {
         e = batch_launch<S, R>(b, false, b->cap_stream, b->side_stream);
         b->bpar ^= 1;
     }
@@ -1217,10 +1242,11 @@ lbm_status batch_graph(lbm_batch* b, int par) {
     b->bpar = saved;
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess)
-        e = instantiate_step_graph(g, b->schedule == LBM_SCHEDULE_GRAPHS_EARLY, &b->gexec[par], &b->gexec_early[par]);
+        e = instantiate_step_graph(g, b->schedule == LBM_SCHEDULE_GRAPHS_EARLY, &b->graphs.exec[size][par],
+                                   &b->graphs.early[size][par]);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        b->gexec[par] = nullptr;
+        b->graphs.exec[size][par] = nullptr;
         return bfail(b, LBM_ERR_CUDA, std::string("batch graph capture: ") + cudaGetErrorString(e));
     }
     return LBM_OK;
@@ -1240,15 +1266,17 @@ lbm_status batch_run(lbm_batch* b, int64_t n) {
     if (b->schedule == LBM_SCHEDULE_PERSISTENT) return batch_run_persistent<S, R>(b, n);
     int64_t rem = n;
     while (rem > 1) {
-        if (b->use_graphs && rem - 1 >= kGraphSteps) {
-            if (batch_graph<S, R>(b, b->bpar) != LBM_OK) {
+        int size = 0;
+        while (size < kGraphSizes && rem - 1 < kGraphSteps[size]) ++size;
+        if (b->use_graphs && size < kGraphSizes) {
+            if (batch_graph<S, R>(b, size, b->bpar) != LBM_OK) {
                 b->use_graphs = 0;
                 cudaGetLastError();
                 continue;
             }
-            BCK(cudaGraphLaunch(b->gexec[b->bpar], b->stream));
-            batch_advance(b, kGraphSteps);  // even: bpar unchanged
-            rem -= kGraphSteps;
+            BCK(cudaGraphLaunch(b->graphs.exec[size][b->bpar], b->stream));
+            batch_advance(b, kGraphSteps[size]);  // even: bpar unchanged
+            rem -= kGraphSteps[size];
             continue;
         }
         BCK((batch_launch<S, R>(b, false, b->stream, nullptr)));
@@ -1697,12 +1725,7 @@ lbm_status lbm_set_schedule(lbm_ctx* c, int schedule) {
         return fail(c, LBM_ERR_UNSUPPORTED, "the persistent schedule runs the lagged chi only");
     CK(cudaStreamSynchronize(c->stream));
     if ((schedule == LBM_SCHEDULE_GRAPHS_EARLY) != (c->schedule == LBM_SCHEDULE_GRAPHS_EARLY))
-        for (int p = 0; p < 2; ++p)  // graphs of the other form
-            if (c->gexec[p]) {
-                cudaGraphExecDestroy(c->gexec[p]);
-                c->gexec[p] = nullptr;
-                c->gexec_early[p] = 0;
-            }
+        c->graphs.drop();  // graphs of the other form
     c->schedule = schedule;
     return LBM_OK;
 }
@@ -1710,7 +1733,7 @@ lbm_status lbm_set_schedule(lbm_ctx* c, int schedule) {
 lbm_status lbm_get_schedule(lbm_ctx* c, int* schedule, int* early_in_use) {
     if (!c || !schedule || !early_in_use) return fail(c, LBM_ERR_INVALID_ARG, "NULL argument");
     *schedule = c->d3 ? LBM_SCHEDULE_GRAPHS : c->schedule;
-    *early_in_use = c->d3 ? 0 : ((c->gexec[0] && c->gexec_early[0]) || (c->gexec[1] && c->gexec_early[1]));
+    *early_in_use = c->d3 ? 0 : (c->graphs.early_in_use() ? 1 : 0);
     return LBM_OK;
 }
 
@@ -1725,11 +1748,7 @@ lbm_status lbm_set_wall_velocity(lbm_ctx* c, int side, double ux) {
         return fail(c, LBM_ERR_UNSUPPORTED, "moving walls are built for FP32 and FP64 storage");
     CK(cudaStreamSynchronize(c->stream));
     c->wall_ux[side == LBM_YMIN ? 0 : 1] = ux;
-    for (int p = 0; p < 2; ++p)  // captured steps carry the old arguments
-        if (c->gexec[p]) {
-            cudaGraphExecDestroy(c->gexec[p]);
-            c->gexec[p] = nullptr;
-        }
+    c->graphs.drop();  // captured steps carry the old arguments
     return LBM_OK;
 }
 
@@ -1739,11 +1758,7 @@ lbm_status lbm_set_wetting(lbm_ctx* c, double delta) {
     if (!std::isfinite(delta) || delta > 1.0) return fail(c, LBM_ERR_INVALID_ARG, "delta must be in (0, 1], or <= 0 to switch off");
     CK(cudaStreamSynchronize(c->stream));
     c->wet_delta = delta > 0.0 ? delta : 0.0;
-    for (int p = 0; p < 2; ++p)  // captured steps carry the old arguments
-        if (c->gexec[p]) {
-            cudaGraphExecDestroy(c->gexec[p]);
-            c->gexec[p] = nullptr;
-        }
+    c->graphs.drop();  // captured steps carry the old arguments
     return LBM_OK;
 }
 
@@ -1762,11 +1777,7 @@ lbm_status lbm_set_chi_timing(lbm_ctx* c, int same_step) {
         CK(cudaMemset(c->oc_state, 0, bytes));
     }
     c->chi_same_step = on ? 1 : 0;
-    for (int p = 0; p < 2; ++p)  // captured steps carry the old launch sequence
-        if (c->gexec[p]) {
-            cudaGraphExecDestroy(c->gexec[p]);
-            c->gexec[p] = nullptr;
-        }
+    c->graphs.drop();  // captured steps carry the old launch sequence
     return LBM_OK;
 }
 
@@ -2119,12 +2130,7 @@ lbm_status lbm_batch_set_schedule(lbm_batch* b, int schedule) {
         return bfail(b, LBM_ERR_UNSUPPORTED, "the persistent schedule is built for FP32 storage only");
     if ((schedule == LBM_SCHEDULE_GRAPHS_EARLY) != (b->schedule == LBM_SCHEDULE_GRAPHS_EARLY)) {
         BCK(cudaStreamSynchronize(b->stream));
-        for (int p = 0; p < 2; ++p)
-            if (b->gexec[p]) {
-                cudaGraphExecDestroy(b->gexec[p]);
-                b->gexec[p] = nullptr;
-                b->gexec_early[p] = 0;
-            }
+        b->graphs.drop();
     }
     b->schedule = schedule;
     return LBM_OK;
@@ -2133,7 +2139,7 @@ lbm_status lbm_batch_set_schedule(lbm_batch* b, int schedule) {
 lbm_status lbm_batch_get_schedule(lbm_batch* b, int* schedule, int* early_in_use) {
     if (!b || !schedule || !early_in_use) return bfail(b, LBM_ERR_INVALID_ARG, "NULL argument");
     *schedule = b->schedule;
-    *early_in_use = (b->gexec[0] && b->gexec_early[0]) || (b->gexec[1] && b->gexec_early[1]);
+    *early_in_use = b->graphs.early_in_use() ? 1 : 0;
     return LBM_OK;
 }
 

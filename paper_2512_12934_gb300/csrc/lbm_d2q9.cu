@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) d2q9_outlet_chi_kernel(const __grid_const
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             R o[9];
-            collide_scalar<R>(a.s[k], k == 0 ? rho0 : rho1, q[20 + 2 * k], q[21 + 2 * k], ux, uy, uu3, f[k], o);
+            collide_one(a, k, k == 0 ? rho0 : rho1, q[20 + 2 * k], q[21 + 2 * k], ux, uy, uu3, f[k], o);
 #pragma unroll
             for (int i = 0; i < 9; ++i) Pop<S, R>::st(a.fout, (k * 9 + i) * a.plane + n, o[i], R(0));
         }

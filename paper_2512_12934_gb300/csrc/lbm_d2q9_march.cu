@@ -192,7 +192,7 @@ __device__ __forceinline__ void collide_node(const MarchSmem& sm, const D2Args<f
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             float o[9];
-            collide_scalar<float>(a.s[k], k == 0 ? rho0 : rho1, k == 0 ? Fx0 : Fx1, k == 0 ? Fy0 : Fy1, ux, uy, uu3,
+            collide_scalar<float>(a.s[k], a.h[k], k == 0 ? rho0 : rho1, k == 0 ? Fx0 : Fx1, k == 0 ? Fy0 : Fy1, ux, uy, uu3,
                                   f[k], o);
 #pragma unroll
             for (int i = 0; i < 9; ++i) a.fout[(k * 9 + i) * a.plane + n] = o[i];

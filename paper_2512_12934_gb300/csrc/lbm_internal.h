@@ -48,6 +48,16 @@ struct FaceDev {
     double sxx, syy;  // sum over the unknown set U of w_i e_ix^2 and w_i e_iy^2
 };
 
+// Relaxation coefficients of the FP64 collision with the normalisation of T^-1
+// and the constants of the forcing moments folded in (row r of component k:
+// a = -s/|row|^2, b = (1 - s/2) c/|row|^2 with c = 6, -6, 1, -1, 1, -1, 2, 1).
+template <typename R>
+struct FoldedRates {};
+template <>
+struct FoldedRates<double> {
+    double a[2][9], b[2][9];
+};
+
 // Kernel arguments of one D2Q9 step.  S is the population storage type,
 // R the arithmetic type.
 template <typename S, typename R>
@@ -99,7 +109,10 @@ struct D2Args {
     R G12;
     R Gw[2];
     R s[2][9];
+    R h[2][9];  // 1 - s/2
+    FoldedRates<R> fold;
     R body[2];
+    int body_on;  // the body force is not zero
 };
 
 // Batched step: tile list entries of many instances; member[] names the
