@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(NTB) mlp_infer_kernel(const float* __restrict_
 // on), copied in by one bulk copy of the member's prepared image.  Layers 1
 // (K = 4) and 4 (N = 2), the biases and GELU run on the FP32 pipes in the
 // epilogues; thread (w, l) owns sample 32 (w % 4) + l (its TMEM lane) and
-// the 32 neurons of column quarter w / 4.
+// neurons 32 c + 8 (w / 4) .. + 7 of each chunk c of 32.
 constexpr int TCT = 512;
 constexpr int TC_WH = H * H * 4, TC_WL = H * H * 2, TC_LAYER = TC_WH + TC_WL, TC_IMG = 2 * TC_LAYER;
 constexpr size_t TC_SMEM = (size_t)TC_IMG + 128;
@@ -624,21 +624,31 @@ __device__ __forceinline__ void tc_mma(bool tf32, uint32_t d, uint32_t a, uint64
                      :: "r"(d), "r"(a), "l"(b), "r"(id), "r"(acc) : "memory");
 }
 
-__device__ __forceinline__ void tc_st16(uint32_t t, const uint32_t (&v)[16]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                 :: "r"(t), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
-}
 __device__ __forceinline__ void tc_st8(uint32_t t, const uint32_t (&v)[8]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  :: "r"(t), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
 }
-__device__ __forceinline__ void tc_ld16(uint32_t t, uint32_t (&v)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+__device__ __forceinline__ void tc_st4(uint32_t t, const uint32_t (&v)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 :: "r"(t), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+// Eight columns of this thread's lane (the caller waits for its loads).
+__device__ __forceinline__ void tc_ld8(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "r"(t) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// The loads above have landed; ties the values to the wait.
+__device__ __forceinline__ void tc_ld_wait(float (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                   "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11])
+                 :: "memory");
+    asm volatile("" : "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]), "+f"(v[18]),
+                      "+f"(v[19]), "+f"(v[20]), "+f"(v[21]));
+    asm volatile("" : "+f"(v[22]), "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]),
+                      "+f"(v[29]), "+f"(v[30]), "+f"(v[31]));
 }
 
 // Bounded wait on phase `parity` of an mbarrier; false (and the status bit)
@@ -666,29 +676,88 @@ __device__ __forceinline__ void tc_sync() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// The activations a[16] of neurons j0..j0+15 (j0 even) of this thread's
-// sample as the next MMA's A operand: Ah, Al (one column each) and Ab (two
-// per column, the even neuron in the low half).
-__device__ __forceinline__ void tc_put_act(uint32_t tAh, uint32_t tAl, uint32_t tAb, int j0, const float (&a)[16]) {
-    uint32_t h[16], lo[16], b2[8];
+// GELU of two values in packed FP32x2 operations: z Phi(z) = (z + |z|)/2 - t h(t),
+// t = |z|, h(t) = erfc(t/sqrt 2)/2 = exp(-t^2/2) P(1/(1 + 0.38 t)), the form of
+// Hastings' approximations (Abramowitz and Stegun 7.1.25-28) with a degree-6 P
+// fitted here by weighted minimax: the error of t h(t) is below 2e-9, so FP32
+// rounding dominates (rms 4.2e-8 over |z| < 6, erff's form 5.3e-8).  Both
+// branches of erff and its divergence go: 21 instructions per pair instead of
+// about 46.  The clamp keeps t exp(..) finite; infinities and NaN pass through
+// the first term.
+__device__ __forceinline__ float2 gelu2(float2 z) {
+    const float2 t = make_float2(fminf(fabsf(z.x), 1e4f), fminf(fabsf(z.y), 1e4f));
+    const float2 d = __ffma2_rn(t, make_float2(0.38f, 0.38f), make_float2(1.f, 1.f));
+    const float2 x = __fmul2_rn(__fmul2_rn(t, make_float2(-0.72134752f, -0.72134752f)), t);  // -t^2/2 log2 e
+    float2 u, e;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(u.x) : "f"(d.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(u.y) : "f"(d.y));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(x.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(x.y));
+    constexpr float c[7] = {-0.0014650963712483644f, -0.13392633199691772f, -0.2417038530111313f,
+                            0.1196700930595398f,     -0.4798668920993805f,  0.2958149015903473f,
+                            -0.05852290615439415f};  // -P
+    float2 q = make_float2(c[6], c[6]);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int k = 5; k >= 0; --k) q = __ffma2_rn(q, u, make_float2(c[k], c[k]));
+    const float2 s = make_float2(z.x + fabsf(z.x), z.y + fabsf(z.y));
+    return __ffma2_rn(s, make_float2(0.5f, 0.5f), __fmul2_rn(t, __fmul2_rn(e, q)));
+}
+
+// The activations a[8] of neurons j0..j0+7 (j0 even) of this thread's sample as
+// the next MMA's A operand: Ah, Al (one column each) and Ab (two per column,
+// the even neuron in the low half).
+__device__ __forceinline__ void tc_put_act(uint32_t tAh, uint32_t tAl, uint32_t tAb, int j0, const float (&a)[8]) {
+    uint32_t h[8], lo[8], b2[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
         const float ah = tf32_rna(a[i]);
         h[i] = __float_as_uint(ah);
         lo[i] = __float_as_uint(a[i] - ah);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < 4; ++i) {
         const __nv_bfloat162 pr = __floats2bfloat162_rn(a[2 * i], a[2 * i + 1]);  // .x = low half
         b2[i] = *reinterpret_cast<const uint32_t*>(&pr);
     }
-    tc_st16(tAh + j0, h);
-    tc_st16(tAl + j0, lo);
-    tc_st8(tAb + j0 / 2, b2);
+    tc_st8(tAh + j0, h);
+    tc_st8(tAl + j0, lo);
+    tc_st4(tAb + j0 / 2, b2);
+}
+
+// The chunk's A columns are written: hand it to warp 0, whose first thread
+// issues the chunk's 10 MMAs (K = 32: four TF32 steps of Ah and of Al, two BF16
+// steps of Ab; a K step moves the descriptor's start address by 256 bytes, +16
+// in its field).  The other warps go on to the next chunk at once.
+__device__ __forceinline__ void tc_issue_chunk(int c, uint32_t tmem, uint32_t wh) {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (threadIdx.x >= 32) {
+        asm volatile("bar.arrive %0, %1;" ::"r"(c + 1), "n"(TCT) : "memory");
+        return;
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(c + 1), "n"(TCT) : "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (threadIdx.x == 0) {
+        const uint32_t it = tc_idesc(2), ib = tc_idesc(1);
+        const uint32_t d = tmem, ah = tmem + 128, al = tmem + 256, ab = tmem + 384;
+        const uint64_t dh = tc_desc(wh, (H / 4) * 128), dl = tc_desc(wh + TC_WH, (H / 8) * 128);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tc_mma(true, d, ah + 8 * (4 * c + q), dh + 16 * (4 * c + q), it, c > 0 || q > 0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tc_mma(true, d, al + 8 * (4 * c + q), dh + 16 * (4 * c + q), it, 1);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) tc_mma(false, d, ab + 8 * (2 * c + q), dl + 16 * (2 * c + q), ib, 1);
+    }
+    __syncwarp();
 }
 
 // Persistent per member: CTA (x, e) loads member e's weights once and runs
-// tiles x, x + gridDim.x, ... of that member.
+// tiles x, x + gridDim.x, ... of that member.  The FP32 work between the layers
+// (GELU, operand splitting) bounds it, so the MMAs run under it: a layer's input
+// is produced in four chunks of 32 neurons (8 per warp quarter) and each chunk's
+// MMAs are issued while the next chunk is computed.  Before (erff, the whole
+// layer written, one barrier, 40 MMAs, a wait): 222 us for 65,536 points x 5
+// members with the tensor pipe idle 78 % of the time; now 140 us.
 __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __restrict__ params,
                                                               const unsigned char* __restrict__ img,
                                                               const float* __restrict__ X, int B,
@@ -698,12 +767,13 @@ __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __res
     unsigned char* sw = tc_raw + ((128u - (tc_smem(tc_raw) & 127u)) & 127u);
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_bar[2];  // [0] weights landed, [1] MMAs of a layer done
-    __shared__ float s_w1[H * I], s_b[3][H], s_w4[O * H], s_b4[O];
+    __shared__ __align__(16) float s_w1[I][H], s_b[3][H], s_w4[O][H];
+    __shared__ float s_b4[O];
     __shared__ float s_part[4][O][TB];
-    __shared__ int s_ok, s_mma_pending;
+    __shared__ int s_ok;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = warp & 3, qc = warp >> 2;
-    const int row = 32 * g + lane, j0 = 32 * qc;
+    const int row = 32 * g + lane;
     const int e = blockIdx.y, ntiles = (B + TB - 1) / TB;
     const float* p = params + (size_t)e * PS;
     if (tid == 0) {
@@ -711,10 +781,10 @@ __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __res
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(tc_smem(&s_bar[1])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_ok = 1;
-        s_mma_pending = -1;
     }
     __syncthreads();
     bool weights = false;  // thread 0: the weight image has landed
+    int pending = -1;      // thread 0: layer whose MMAs are committed and not waited for
     if (tid == 0) {
         // the member's weight image: four bulk copies onto one transaction count
         const unsigned char* src = img + (size_t)e * TC_IMG;
@@ -724,112 +794,118 @@ __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __res
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          :: "r"(tc_smem(sw + c * (TC_IMG / 4))), "l"(src + c * (TC_IMG / 4)), "r"(TC_IMG / 4),
                             "r"(tc_smem(&s_bar[0])) : "memory");
-        // the other threads stage the small parameters and run layer 1 meanwhile
+        // the other threads stage the small parameters meanwhile
         weights = tc_wait(&s_bar[0], 0, status, limit);
         if (!weights) s_ok = 0;
     }
-    for (int i = tid; i < H * I; i += TCT) s_w1[i] = p[oW1 + i];
+    for (int i = tid; i < H * I; i += TCT) s_w1[i % I][i / I] = p[oW1 + i];
     for (int i = tid; i < H; i += TCT) {
         s_b[0][i] = p[ob1 + i];
         s_b[1][i] = p[ob2 + i];
         s_b[2][i] = p[ob3 + i];
     }
-    for (int i = tid; i < O * H; i += TCT) s_w4[i] = p[oW4 + i];
+    for (int i = tid; i < O * H; i += TCT) s_w4[i / H][i % H] = p[oW4 + i];
     if (tid < O) s_b4[tid] = p[ob4 + tid];
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(tc_smem(&s_tmem)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_sync();
-    const uint32_t lane_off = (uint32_t)(32 * g) << 16;
-    const uint32_t tD = s_tmem + lane_off, tAh = tD + 128, tAl = tD + 256, tAb = tD + 384;
-#pragma unroll 1
-    for (int t = blockIdx.x; t < ntiles && s_ok; t += gridDim.x) {
+    const uint32_t tmem = s_tmem, lane_off = (uint32_t)(32 * g) << 16;
+    const uint32_t tD = tmem + lane_off, tAh = tD + 128, tAl = tD + 256, tAb = tD + 384;
+    bool ok = s_ok != 0;  // the same in every thread
+    float x[I];
+    auto load_x = [&](int t) {
         const int b = t * TB + row;
-        // ---- layer 1 (K = 4) on the FP32 pipes, GELU, A of layer 2 ----
-        {
-            float x[I] = {0.0f, 0.0f, 0.0f, 0.0f};
-            if (b < B)
 #pragma unroll
-                for (int k = 0; k < I; ++k) x[k] = __ldg(X + (size_t)b * I + k);
-#pragma unroll
-            for (int c = 0; c < 32; c += 16) {
-                float a[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int j = j0 + c + i;
-                    float z = s_b[0][j];
-#pragma unroll
-                    for (int k = 0; k < I; ++k) z = fmaf(s_w1[j * I + k], x[k], z);
-                    a[i] = gelu(z);
-                }
-                tc_put_act(tAh, tAl, tAb, j0 + c, a);
-            }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        for (int k = 0; k < I; ++k) x[k] = t < ntiles && b < B ? __ldg(X + (size_t)b * I + k) : 0.0f;
+    };
+    // every thread waits for the layer's MMAs; one decision for the whole CTA
+    auto layer_done = [&](int l) {
+        if (tid == 0) {
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                         :: "r"(tc_smem(&s_bar[1])) : "memory");
+            pending = l;
         }
+        // two commits per tile: phase parity = layer
+        ok = __syncthreads_and(tc_wait(&s_bar[1], (uint32_t)l, status, limit)) != 0;
+        if (ok) pending = -1;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    if (ok) load_x(blockIdx.x);
 #pragma unroll 1
-        for (int l = 0; l < 2; ++l) {
-            tc_sync();
-            if (tid == 0) {
-                // 40 MMAs of the layer from one thread; a K step moves the
-                // descriptor's start address by 256 bytes (+16 in its field)
-                const uint32_t wh = tc_smem(sw + l * TC_LAYER), wl = wh + TC_WH;
-                const uint32_t it = tc_idesc(2), ib = tc_idesc(1);
-                const uint32_t d = s_tmem, ah = s_tmem + 128, al = s_tmem + 256, ab = s_tmem + 384;
-                const uint64_t dh = tc_desc(wh, (H / 4) * 128), dl = tc_desc(wl, (H / 8) * 128);
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        // ---- layer 1 (K = 4) on the FP32 pipes, GELU, A of layer 2 ----
 #pragma unroll
-                for (int s = 0; s < H / 8; ++s) tc_mma(true, d, ah + 8 * s, dh + 16 * s, it, s > 0);
+        for (int c = 0; c < 4; ++c) {
+            const int j0 = 32 * c + 8 * qc;
+            float a[8];
 #pragma unroll
-                for (int s = 0; s < H / 8; ++s) tc_mma(true, d, al + 8 * s, dh + 16 * s, it, 1);
+            for (int i = 0; i < 8; i += 4) {
+                const float4 b4 = *reinterpret_cast<const float4*>(&s_b[0][j0 + i]);
+                float2 z0 = make_float2(b4.x, b4.y), z1 = make_float2(b4.z, b4.w);
 #pragma unroll
-                for (int s = 0; s < H / 16; ++s) tc_mma(false, d, ab + 8 * s, dl + 16 * s, ib, 1);
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(tc_smem(&s_bar[1])) : "memory");
-                s_mma_pending = l;
-            }
-            __syncthreads();
-            // two commits per tile: phase parity = layer
-            // one decision for the whole CTA: every thread saw the phase complete
-            const int ok_before = s_ok;
-            if (!__syncthreads_and(ok_before && tc_wait(&s_bar[1], (uint32_t)l, status, limit))) {
-                if (tid == 0) s_ok = 0;
-                break;
-            }
-            if (tid == 0) s_mma_pending = -1;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (l == 0) {
-                // ---- epilogue of layer 2: bias, GELU, A of layer 3 ----
-#pragma unroll
-                for (int c = 0; c < 32; c += 16) {
-                    uint32_t v[16];
-                    tc_ld16(tD + j0 + c, v);
-                    float a[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) a[i] = gelu(__uint_as_float(v[i]) + s_b[1][j0 + c + i]);
-                    tc_put_act(tAh, tAl, tAb, j0 + c, a);
+                for (int k = 0; k < I; ++k) {
+                    const float4 w4 = *reinterpret_cast<const float4*>(&s_w1[k][j0 + i]);
+                    z0 = __ffma2_rn(make_float2(w4.x, w4.y), make_float2(x[k], x[k]), z0);
+                    z1 = __ffma2_rn(make_float2(w4.z, w4.w), make_float2(x[k], x[k]), z1);
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            } else {
-                // ---- epilogue of layer 3 and layer 4 (N = 2): partial sums over this quarter ----
-                float y0 = 0.0f, y1 = 0.0f;
+                z0 = gelu2(z0);
+                z1 = gelu2(z1);
+                a[i] = z0.x;
+                a[i + 1] = z0.y;
+                a[i + 2] = z1.x;
+                a[i + 3] = z1.y;
+            }
+            tc_put_act(tAh, tAl, tAb, j0, a);
+            tc_issue_chunk(c, tmem, tc_smem(sw));
+        }
+        load_x(t + gridDim.x);  // arrives while the hidden layers run
+        layer_done(0);
+        if (!ok) break;
+        float v[32];
 #pragma unroll
-                for (int c = 0; c < 32; c += 16) {
-                    uint32_t v[16];
-                    tc_ld16(tD + j0 + c, v);
+        for (int c = 0; c < 4; ++c) tc_ld8(tD + 32 * c + 8 * qc, v + 8 * c);
+        tc_ld_wait(v);
+        // ---- epilogue of layer 2: bias, GELU, A of layer 3.  The first chunk's
+        // barrier also says that every warp has read its part of D, which that
+        // chunk's MMAs overwrite ----
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int j = j0 + c + i;
-                        const float a = gelu(__uint_as_float(v[i]) + s_b[2][j]);
-                        y0 = fmaf(a, s_w4[j], y0);
-                        y1 = fmaf(a, s_w4[H + j], y1);
-                    }
-                }
-                s_part[qc][0][row] = y0;
-                s_part[qc][1][row] = y1;
+        for (int c = 0; c < 4; ++c) {
+            const int j0 = 32 * c + 8 * qc;
+            float a[8];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const float2 b2 = *reinterpret_cast<const float2*>(&s_b[1][j0 + i]);
+                const float2 z = gelu2(__fadd2_rn(make_float2(v[8 * c + i], v[8 * c + i + 1]), b2));
+                a[i] = z.x;
+                a[i + 1] = z.y;
+            }
+            tc_put_act(tAh, tAl, tAb, j0, a);
+            tc_issue_chunk(c, tmem, tc_smem(sw + TC_LAYER));
+        }
+        layer_done(1);
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc_ld8(tD + 32 * c + 8 * qc, v + 8 * c);
+        tc_ld_wait(v);
+        // ---- epilogue of layer 3 and layer 4 (N = 2): partial sums over this thread's neurons ----
+        float2 y0 = make_float2(0.f, 0.f), y1 = y0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int j0 = 32 * c + 8 * qc;
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const float2 b2 = *reinterpret_cast<const float2*>(&s_b[2][j0 + i]);
+                const float2 z = gelu2(__fadd2_rn(make_float2(v[8 * c + i], v[8 * c + i + 1]), b2));
+                y0 = __ffma2_rn(z, *reinterpret_cast<const float2*>(&s_w4[0][j0 + i]), y0);
+                y1 = __ffma2_rn(z, *reinterpret_cast<const float2*>(&s_w4[1][j0 + i]), y1);
             }
         }
+        s_part[qc][0][row] = y0.x + y0.y;
+        s_part[qc][1][row] = y1.x + y1.y;
         tc_sync();
-        if (s_ok && tid < O * TB) {
+        if (tid < O * TB) {
             const int r = tid % TB, o = tid / TB, bb = t * TB + r;
             const float y = s_b4[o] + ((s_part[0][o][r] + s_part[1][o][r]) + (s_part[2][o][r] + s_part[3][o][r]));
             if (bb < B) Y[((size_t)e * B + bb) * O + o] = y;
@@ -840,17 +916,21 @@ __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __res
     tc_sync();
     if (tid == 0) {
         if (!weights) tc_wait(&s_bar[0], 0, status, TC_WAIT_LIMIT);
-        if (s_mma_pending >= 0) tc_wait(&s_bar[1], (uint32_t)s_mma_pending, status, TC_WAIT_LIMIT);
+        if (pending >= 0) tc_wait(&s_bar[1], (uint32_t)pending, status, TC_WAIT_LIMIT);
     }
     tc_sync();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(s_tmem), "r"(512) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(512) : "memory");
 }
 
 // Ensemble mean and relative spread (max over outputs of the population std
 // over members / |mean|), two passes over the members.
+// mean, spread and status_out may be mapped host memory: the inference status
+// word goes out with the results, so a call needs no copy after it.
 __global__ void mlp_reduce_kernel(const float* __restrict__ Y, int E, int B, float* __restrict__ mean,
-                                  float* __restrict__ spread) {
+                                  float* __restrict__ spread, const unsigned* __restrict__ status,
+                                  unsigned* __restrict__ status_out) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b == 0) *status_out = *status;
     if (b >= B) return;
     float sp = 0.0f;
 #pragma unroll
@@ -897,10 +977,19 @@ struct lbm_mlp {
     long long wait_limit = TC_WAIT_LIMIT;  // SM cycles a tensor-core wait may take
     void* ws = nullptr;       // grow-only device workspace of the per-call buffers
     size_t ws_bytes = 0;
+    unsigned* hstatus = nullptr;  // pinned: status word of the last prediction
+    float* hio = nullptr;         // pinned: X, mean and spread of a small host prediction
     std::string err;
 };
 
 namespace {
+
+// Host predictions of up to this many points run on mapped pinned memory: the
+// kernels read X and write the results over the host link themselves, two
+// launches and one synchronisation instead of those plus four copies (221
+// points: 63 -> 31 us a call; beyond a few thousand points the copy engine moves the
+// bytes faster than every member reading X over the link).
+constexpr int kMappedPoints = 4096;
 
 lbm_status mfail(lbm_mlp* m, lbm_status st, const std::string& msg) {
     if (m) m->err = msg;
@@ -1085,14 +1174,18 @@ lbm_status launch_infer(lbm_mlp* mm, const float* dX, int n, float* dY) {
 
 // After the stream has drained: a tensor-core wait that ran out is an error
 // (the outputs of that call are undefined); the word is cleared for the next.
-lbm_status check_infer(lbm_mlp* mm) {
-    unsigned st = 0;
-    MCK(cudaMemcpy(&st, mm->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
+lbm_status infer_result(lbm_mlp* mm, unsigned st) {
     if (st) {
         MCK(cudaMemset(mm->status, 0, sizeof(unsigned)));
         return mfail(mm, LBM_ERR_TIMEOUT, "a tensor-core wait of the inference kernel ran out; outputs undefined");
     }
     return LBM_OK;
+}
+
+lbm_status check_infer(lbm_mlp* mm) {
+    unsigned st = 0;
+    MCK(cudaMemcpy(&st, mm->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    return infer_result(mm, st);
 }
 
 }  // namespace
@@ -1132,6 +1225,8 @@ lbm_status lbm_mlp_create(int members, uint64_t seed, void* cuda_stream, lbm_mlp
     if (e == cudaSuccess) e = cudaMalloc((void**)&mm->tcimg, (size_t)members * TC_IMG);
     if (e == cudaSuccess) e = cudaMalloc((void**)&mm->status, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(mm->status, 0, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&mm->hstatus, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&mm->hio, (size_t)kMappedPoints * (I + O + 1) * sizeof(float));
     if (e != cudaSuccess) {
         const std::string msg = std::string("mlp allocation: ") + cudaGetErrorString(e);
         lbm_mlp_destroy(mm);
@@ -1285,11 +1380,18 @@ lbm_status lbm_mlp_train(lbm_mlp* mm, const float* X, const float* T, int n, int
 lbm_status lbm_mlp_predict(lbm_mlp* mm, const float* X, int n, float* mean, float* spread, int dst_is_device) {
     if (!mm || !X || !mean || !spread || n < 1) return mfail(mm, LBM_ERR_INVALID_ARG, "bad predict request");
     Scratch s;
-    const size_t hn = dst_is_device ? 0 : (size_t)n;
+    const bool mapped = !dst_is_device && n <= kMappedPoints;
+    const size_t hn = dst_is_device || mapped ? 0 : (size_t)n;
     CARVE(hn * I, hn * O, (size_t)mm->E * n * O, 0, hn, 0, 0);
     const float* dX = X;
     float *dm = mean, *ds = spread;
-    if (!dst_is_device) {
+    if (mapped) {
+        float* h = mm->hio;
+        std::memcpy(h, X, (size_t)n * I * sizeof(float));
+        dX = h;
+        dm = h + (size_t)kMappedPoints * I;
+        ds = dm + (size_t)kMappedPoints * O;
+    } else if (!dst_is_device) {
         MCK(cudaMemcpyAsync(s.X, X, (size_t)n * I * sizeof(float), cudaMemcpyHostToDevice, mm->stream));
         dX = s.X;
         dm = s.T;
@@ -1297,14 +1399,18 @@ lbm_status lbm_mlp_predict(lbm_mlp* mm, const float* X, int n, float* mean, floa
     }
     lbm_status st = launch_infer(mm, dX, n, s.Y);
     if (st != LBM_OK) return st;
-    mlp_reduce_kernel<<<(n + 255) / 256, 256, 0, mm->stream>>>(s.Y, mm->E, n, dm, ds);
+    mlp_reduce_kernel<<<(n + 255) / 256, 256, 0, mm->stream>>>(s.Y, mm->E, n, dm, ds, mm->status, mm->hstatus);
     MCK(cudaGetLastError());
-    if (!dst_is_device) {
+    if (!dst_is_device && !mapped) {
         MCK(cudaMemcpyAsync(mean, dm, (size_t)n * O * sizeof(float), cudaMemcpyDeviceToHost, mm->stream));
         MCK(cudaMemcpyAsync(spread, ds, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, mm->stream));
     }
     MCK(cudaStreamSynchronize(mm->stream));
-    return check_infer(mm);
+    if (mapped) {
+        std::memcpy(mean, dm, (size_t)n * O * sizeof(float));
+        std::memcpy(spread, ds, (size_t)n * sizeof(float));
+    }
+    return infer_result(mm, *static_cast<volatile unsigned*>(mm->hstatus));
 }
 
 lbm_status lbm_mlp_set_wait_limit(lbm_mlp* mm, long long cycles) {
@@ -1330,6 +1436,8 @@ void lbm_mlp_destroy(lbm_mlp* mm) {
     void* p[] = {mm->params, mm->m, mm->v, mm->wt, mm->tcimg, mm->status, mm->ws};
     for (void* q : p)
         if (q) cudaFree(q);
+    if (mm->hstatus) cudaFreeHost(mm->hstatus);
+    if (mm->hio) cudaFreeHost(mm->hio);
     delete mm;
 }
 
