@@ -219,8 +219,9 @@ lbm_status lbm_kernel_time(lbm_ctx* ctx, double* mean_ms, int64_t* samples);
 lbm_status lbm_kernel_time_split(lbm_ctx* ctx, double* fast_ms, double* general_ms, int64_t* samples);
 
 /* Tile shape of the fused step kernel: variant in [0, lbm_num_tile_variants()),
- * 0: 32x8, 1: 32x4, 2: 64x4, 3: 32x16 nodes per CTA (default: 1 below 2^22
- * nodes, else 0).  Bit-identical results on grids without open faces; with
+ * 0: 32x8, 1: 32x4, 2: 64x4, 3: 32x16 nodes per CTA (default: 0; 1 for
+ * FP64 grids with open faces below 2^18 nodes and other grids with an open y
+ * face below 2^22).  Bit-identical results on grids without open faces; with
  * open faces the FP64 flux partials are grouped per tile, so chi may differ
  * in its last bit.  Variant 4 tiles like variant 0 and, for FP32 storage,
  * runs the interior tiles (those whose pulls and interaction stencil stay

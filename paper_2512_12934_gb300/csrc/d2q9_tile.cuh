@@ -147,23 +147,86 @@ __device__ __forceinline__ R feq_(int i, R rho, R ux, R uy) {
 // f*_i(x - e_i); a set bit i in `info` means that source is solid or outside
 // a closed edge, and halfway bounce-back (Eq. B1) takes f*_opp(i)(x).
 
-// Interior pull: every source lies inside the grid, no wrap needed.
+//
+// A pull is issued in two parts.  The loads take the plain neighbours (wrapped
+// on every axis, so always inside the grid) and need no descriptor: they go out
+// together with the descriptor's own load instead of one memory latency after
+// it, and cost no selects.  The few nodes with a blocked direction then replace
+// those values.  us per step, before -> now: 100x100 periodic 4.67 -> 3.70,
+// 512x512 10.6 -> 9.9, channels 1024x128 8.25 -> 7.9, 4096x2048 308 -> 292, 24
+// T-junctions in a batch 80.7 -> 77.0.
+
+// Loads of an interior node: every source lies inside the grid, no wrap needed.
 template <typename S, typename R>
-__device__ __forceinline__ void pull_interior(const D2Args<S, R>& a, int n, unsigned info, R (&f)[2][9]) {
-    R ref[2];
-    node_ref(a, n, ref);
+__device__ __forceinline__ void pull_load_interior(const D2Args<S, R>& a, int n, const R (&ref)[2], R (&f)[2][9]) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const bool bb = (info >> i) & 1u;
-        const int src = bb ? n : n - ex_(i) - ey_(i) * a.pitch;
-        const int dir = bb ? opp_(i) : i;
+    for (int i = 0; i < 9; ++i)
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + dir) * a.plane + src, w_<R>(i) * ref[k]);
+            f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + i) * a.plane + (n - ex_(i) - ey_(i) * a.pitch), w_<R>(i) * ref[k]);
+}
+
+// Loads of any node inside the grid.
+template <typename S, typename R>
+__device__ __forceinline__ void pull_load_wrap(const D2Args<S, R>& a, int x, int y, const R (&ref)[2], R (&f)[2][9]) {
+    const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
+    const int ym = (y == 0 ? a.ny - 1 : y - 1) * a.pitch, yp = (y == a.ny - 1 ? 0 : y + 1) * a.pitch;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int src = (ex_(i) > 0 ? xm : (ex_(i) < 0 ? xp : x)) + (ey_(i) > 0 ? ym : (ey_(i) < 0 ? yp : y * a.pitch));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + i) * a.plane + src, w_<R>(i) * ref[k]);
     }
 }
 
-// General pull: sources wrap on periodic axes.
+// Blocked directions (halfway bounce-back, Eq. B1) of node n.
+template <typename S, typename R>
+__device__ __forceinline__ void pull_fix(const D2Args<S, R>& a, int n, unsigned info, const R (&ref)[2],
+                                         R (&f)[2][9]) {
+    if ((info & 0x1FEu) == 0u) return;
+#pragma unroll
+    for (int i = 1; i < 9; ++i)
+        if ((info >> i) & 1u) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + opp_(i)) * a.plane + n, w_<R>(i) * ref[k]);
+        }
+}
+
+// Moving wall beyond a closed y edge (halfway bounce-back carrying the wall's
+// momentum): a population reflected there gains 2 w_i rho_k (e_i . u_w) / c_s^2,
+// rho_k the node's own density (the sum of its post-collision populations).
+// FP32 / FP64 storage.
+template <typename S, typename R>
+__device__ __forceinline__ void pull_wall(const D2Args<S, R>& a, int x, int y, unsigned info, R (&f)[2][9]) {
+    if constexpr (!is_half_<S>()) {
+        const int side = y == 0 ? 0 : (y == a.ny - 1 ? 1 : -1);
+        if (a.wall_on && !a.py && side >= 0 && a.wall_ux[side] != R(0)) {
+            const int n = y * a.pitch + x;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                R rk = R(0);
+#pragma unroll
+                for (int j = 0; j < 9; ++j) rk += Pop<S, R>::ld(a.fin, (k * 9 + j) * a.plane + n, R(0));
+#pragma unroll
+                for (int i = 0; i < 9; ++i)
+                    if (((info >> i) & 1u) && (side == 0 ? ey_(i) > 0 : ey_(i) < 0))
+                        f[k][i] += R(6) * w_<R>(i) * rk * (R(ex_(i)) * a.wall_ux[side]);
+            }
+        }
+    }
+}
+
+// The rest of a pull whose loads are out: blocked directions, moving walls.
+template <typename S, typename R>
+__device__ __forceinline__ void pull_finish(const D2Args<S, R>& a, int x, int y, unsigned info, const R (&ref)[2],
+                                            R (&f)[2][9]) {
+    pull_fix(a, y * a.pitch + x, info, ref, f);
+    pull_wall(a, x, y, info, f);
+}
+
+// Whole pull of a node whose descriptor is known (serially staged tiles): each
+// source is selected before its one load, which takes fewer registers.
 template <typename S, typename R>
 __device__ __forceinline__ void pull_wrap(const D2Args<S, R>& a, int x, int y, unsigned info, R (&f)[2][9]) {
     const int n = y * a.pitch + x;
@@ -186,25 +249,7 @@ __device__ __forceinline__ void pull_wrap(const D2Args<S, R>& a, int x, int y, u
         for (int k = 0; k < 2; ++k)
             f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + dir) * a.plane + src, w_<R>(i) * ref[k]);
     }
-    // Moving wall beyond a closed y edge (halfway bounce-back carrying the
-    // wall's momentum): a population reflected there gains
-    // 2 w_i rho_k (e_i . u_w) / c_s^2, rho_k the node's own density (the sum
-    // of its post-collision populations).  FP32 / FP64 storage.
-    if constexpr (!is_half_<S>()) {
-        const int side = y == 0 ? 0 : (y == a.ny - 1 ? 1 : -1);
-        if (a.wall_on && !a.py && side >= 0 && a.wall_ux[side] != R(0)) {
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                R rk = R(0);
-#pragma unroll
-                for (int j = 0; j < 9; ++j) rk += Pop<S, R>::ld(a.fin, (k * 9 + j) * a.plane + n, R(0));
-#pragma unroll
-                for (int i = 0; i < 9; ++i)
-                    if (((info >> i) & 1u) && (side == 0 ? ey_(i) > 0 : ey_(i) < 0))
-                        f[k][i] += R(6) * w_<R>(i) * rk * (R(ex_(i)) * a.wall_ux[side]);
-            }
-        }
-    }
+    pull_wall(a, x, y, info, f);
 }
 
 // rho_k = sum_i f_i (Eq. 8) in a fixed pairwise order.
@@ -364,18 +409,23 @@ __device__ __forceinline__ bool site_rho(const D2Args<S, R>& a, int gx, int gy, 
         r1 = rho_of(g[1]);
     } else if (MODE == 1) {
         if (resolve_closed(a, gx, gy)) return false;
-        const unsigned inf = a.info[gy * a.pitch + gx];
+        const int n = gy * a.pitch + gx;
+        const unsigned inf = a.info[n];
+        R ref[2], g[2][9];
+        node_ref(a, n, ref);
+        pull_load_wrap(a, gx, gy, ref, g);
         if (inf & INFO_SOLID) return false;
-        R g[2][9];
-        pull_wrap(a, gx, gy, inf, g);
+        pull_finish(a, gx, gy, inf, ref, g);
         r0 = rho_of(g[0]);
         r1 = rho_of(g[1]);
     } else {
         const int n = gy * a.pitch + gx;
         const unsigned inf = a.info[n];
+        R ref[2], g[2][9];
+        node_ref(a, n, ref);
+        pull_load_interior(a, n, ref, g);
         if (inf & INFO_SOLID) return false;
-        R g[2][9];
-        pull_interior(a, n, inf, g);
+        pull_fix(a, n, inf, ref, g);
         r0 = rho_of(g[0]);
         r1 = rho_of(g[1]);
     }
@@ -405,10 +455,22 @@ __device__ __forceinline__ typename RhoPair<R>::type rpair(R a, R b) {
 template <typename S, typename R, int TX, int TY>
 struct TileSmem {
     typename RhoPair<R>::type rr[TY + 4][TX + 4];
+    // FP16 storage: the same densities rounded to half, the references of the
+    // nodes that read this tile's populations (one rounding per site instead of
+    // one per direction)
+    typename RhoPair<R>::type hr[is_half_<S>() ? TY + 4 : 1][is_half_<S>() ? TX + 4 : 1];
     unsigned char sol[TY + 4][TX + 4];
     R un[TX > TY ? TX : TY];
     R lam, chi;  // outlet coefficients of this step (general tiles that see the outlet)
 };
+
+// Densities of one staged site.
+template <typename SM, typename R>
+__device__ __forceinline__ void put_rho(SM& sm, int ry, int rx, R r0, R r1) {
+    sm.rr[ry][rx] = rpair<R>(r0, r1);
+    if constexpr (sizeof(sm.hr) > sizeof(typename RhoPair<R>::type))
+        sm.hr[ry][rx] = rpair<R>(half_round(r0), half_round(r1));
+}
 
 // General tiles also keep up to two face strips: the face nodes of one grid
 // side along the tile's halo range, each reconstructed once per tile.
@@ -449,11 +511,14 @@ __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R,
             info = INFO_SOLID;
             fluid = false;
             if (inb) {
-                info = a.info[y * a.pitch + x];
+                const int n = y * a.pitch + x;
+                info = a.info[n];
+                R ref[2];
+                node_ref(a, n, ref);
+                pull_load_wrap(a, x, y, ref, f);
                 fluid = !(info & INFO_SOLID);
                 if (fluid) {
-                    if (MODE == 2) pull_general(a, x, y, info, R(0), f);
-                    else pull_wrap(a, x, y, info, f);
+                    pull_finish(a, x, y, info, ref, f);
                     r0 = rho_of(f[0]);
                     r1 = rho_of(f[1]);
                     sol = 0;
@@ -464,15 +529,18 @@ __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R,
         } else {
             const int n = y * a.pitch + x;
             info = a.info[n];
+            R ref[2];
+            node_ref(a, n, ref);
+            pull_load_interior(a, n, ref, f);
             fluid = !(info & INFO_SOLID);
             if (fluid) {
-                pull_interior(a, n, info, f);
+                pull_fix(a, n, info, ref, f);
                 r0 = rho_of(f[0]);
                 r1 = rho_of(f[1]);
                 sol = 0;
             }
         }
-        sm.rr[ty + 2][tx + 2] = rpair<R>(r0, r1);
+        put_rho(sm, ty + 2, tx + 2, r0, r1);
         sm.sol[ty + 2][tx + 2] = sol;
     };
     // halo ring: densities only
@@ -493,7 +561,7 @@ __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R,
         }
         R h0 = R(0), h1 = R(0);
         const bool ok = site_rho<S, R, MODE>(a, x0 - 2 + rx, y0 - 2 + ry, h0, h1);
-        sm.rr[ry][rx] = rpair<R>(h0, h1);
+        put_rho(sm, ry, rx, h0, h1);
         sm.sol[ry][rx] = ok ? 0 : 1;
     };
     // When one pass of the node threads covers the ring, its pulls are
@@ -668,6 +736,9 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         unsigned char sol = 1;
         if (x >= 0 && x < a.nx && y >= 0 && y < a.ny) {
             info = a.info[y * a.pitch + x];
+            R ref[2];
+            node_ref(a, y * a.pitch + x, ref);
+            pull_load_wrap(a, x, y, ref, f);
             fluid = !(info & INFO_SOLID);
             if (fluid) {
                 sol = 0;
@@ -678,7 +749,7 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                     own_idx = side <= 1 ? ty : tx;
                     if (own_strip < 0) pending = true;
                 } else {
-                    pull_general(a, x, y, info, R(0), f);
+                    pull_finish(a, x, y, info, ref, f);
                     r0 = rho_of(f[0]);
                     r1 = rho_of(f[1]);
                 }
@@ -690,7 +761,7 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         pend_y = y;
         pend_rx = tx + 2;
         pend_ry = ty + 2;
-        sm.rr[ty + 2][tx + 2] = rpair<R>(r0, r1);
+        put_rho(sm, ty + 2, tx + 2, r0, r1);
         sm.sol[ty + 2][tx + 2] = sol;
     } else if (tid < NT + RING) {
         // ---- halo ring: densities only ----
@@ -701,6 +772,9 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         unsigned char hs = 1;
         if (!resolve_site(a, gx, gy)) {
             const unsigned inf = a.info[gy * a.pitch + gx];
+            R ref[2], g[2][9];
+            node_ref(a, gy * a.pitch + gx, ref);
+            pull_load_wrap(a, gx, gy, ref, g);
             if (!(inf & INFO_SOLID)) {
                 hs = 0;
                 const int fid = (int)((inf >> INFO_FACE_SHIFT) & 7u);
@@ -722,14 +796,13 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                         pend_info = inf;
                     }
                 } else {
-                    R g[2][9];
-                    pull_general(a, gx, gy, inf, R(0), g);
+                    pull_finish(a, gx, gy, inf, ref, g);
                     h0 = rho_of(g[0]);
                     h1 = rho_of(g[1]);
                 }
             }
         }
-        sm.rr[ry][rx] = rpair<R>(h0, h1);
+        put_rho(sm, ry, rx, h0, h1);
         sm.sol[ry][rx] = hs;
     } else if (tid >= G::SB) {
         // ---- face strips (and lambda, chi) ----
@@ -744,28 +817,32 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         const int side = j == 0 ? side0 : side1;
         int sx = -1, sy = -1;
         unsigned inf = INFO_SOLID, inf2 = INFO_SOLID;
+        R g[2][9], gn[2][9], ref[2], ref2[2];
         if (has) {
             strip_node<TX, TY>(side, e, x0, y0, a.nx, a.ny, sx, sy);
             if (sx >= 0 && sx < a.nx && sy >= 0 && sy < a.ny) {
                 inf = a.info[sy * a.pitch + sx];
                 // the inward neighbour along this strip's normal, read with
                 // the node's own word (a corner node may belong to the face of
-                // the other side; it is re-read below then)
+                // the other side; it is re-read below then).  Both pulls are in
+                // flight before either word is needed and before lambda is
+                // folded; only the blend of Eqs. 13-20 waits for it
                 const int x2 = sx - side_ox(side), y2 = sy - side_oy(side);
-                if (x2 >= 0 && x2 < a.nx && y2 >= 0 && y2 < a.ny) inf2 = a.info[y2 * a.pitch + x2];
+                inf2 = a.info[y2 * a.pitch + x2];
+                node_ref(a, sy * a.pitch + sx, ref);
+                node_ref(a, y2 * a.pitch + x2, ref2);
+                pull_load_wrap(a, sx, sy, ref, g);
+                pull_load_wrap(a, x2, y2, ref2, gn);
             }
         }
-        // both pulls in flight before lambda is folded; only the blend of
-        // Eqs. 13-20 waits for it
         const bool face = !(inf & INFO_SOLID) && ((inf >> INFO_FACE_SHIFT) & 7u);
         const int fid = (int)((inf >> INFO_FACE_SHIFT) & 7u) - 1;
         const int fside = face ? a.face[fid].side : 0;
-        R g[2][9], gn[2][9];
         if (face) {
             const int x2 = sx - side_ox(fside), y2 = sy - side_oy(fside);
-            if (fside != side) inf2 = a.info[y2 * a.pitch + x2];
-            pull_wrap(a, sx, sy, inf, g);
-            pull_wrap(a, x2, y2, inf2, gn);
+            pull_finish(a, sx, sy, inf, ref, g);
+            if (fside != side) pull_wrap(a, x2, y2, a.info[y2 * a.pitch + x2], gn);
+            else pull_finish(a, x2, y2, inf2, ref2, gn);
         }
         R lam = R(0);
         if (lam_on) {
@@ -825,7 +902,7 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                 r1 = rho_of(g[1]);
                 sol = 0;
             }
-            sm.rr[pend_ry][pend_rx] = rpair<R>(r0, r1);
+            put_rho(sm, pend_ry, pend_rx, r0, r1);
             sm.sol[pend_ry][pend_rx] = sol;
         }
         __syncthreads();
@@ -836,10 +913,10 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         for (int k = 0; k < 2; ++k)
 #pragma unroll
             for (int i = 0; i < 9; ++i) f[k][i] = sm.fs_f[own_strip][own_idx][k * 9 + i];
-        sm.rr[ty + 2][tx + 2] = rpair<R>(rho_of(f[0]), rho_of(f[1]));
+        put_rho(sm, ty + 2, tx + 2, rho_of(f[0]), rho_of(f[1]));
     }
     if (def_j >= 0) {
-        sm.rr[def_ry][def_rx] = rpair<R>(sm.fs_rho[def_j][def_e][0], sm.fs_rho[def_j][def_e][1]);
+        put_rho(sm, def_ry, def_rx, sm.fs_rho[def_j][def_e][0], sm.fs_rho[def_j][def_e][1]);
     }
 }
 
@@ -929,7 +1006,7 @@ __device__ __forceinline__ void stage_tile_compact(const D2Args<S, R>& a, TileSm
     } else if (site_rho<S, R, 2>(a, x, y, r0, r1, lam)) {
         sol = 0;
     }
-    sm.rr[ty + 2][tx + 2] = rpair<R>(r0, r1);
+    put_rho(sm, ty + 2, tx + 2, r0, r1);
     sm.sol[ty + 2][tx + 2] = sol;
 
     // ---- halo ring ----
@@ -975,7 +1052,7 @@ __device__ __forceinline__ void stage_tile_compact(const D2Args<S, R>& a, TileSm
                 }
             }
         }
-        sm.rr[ry][rx] = rpair<R>(h0, h1);
+        put_rho(sm, ry, rx, h0, h1);
         sm.sol[ry][rx] = hs;
     }
     __syncthreads();
@@ -984,10 +1061,10 @@ __device__ __forceinline__ void stage_tile_compact(const D2Args<S, R>& a, TileSm
         for (int k = 0; k < 2; ++k)
 #pragma unroll
             for (int i = 0; i < 9; ++i) f[k][i] = sm.fs_f[own_strip][own_idx][k * 9 + i];
-        sm.rr[ty + 2][tx + 2] = rpair<R>(rho_of(f[0]), rho_of(f[1]));
+        put_rho(sm, ty + 2, tx + 2, rho_of(f[0]), rho_of(f[1]));
     }
     if (def_j >= 0) {
-        sm.rr[def_ry][def_rx] = rpair<R>(sm.fs_rho[def_j][def_e][0], sm.fs_rho[def_j][def_e][1]);
+        put_rho(sm, def_ry, def_rx, sm.fs_rho[def_j][def_e][0], sm.fs_rho[def_j][def_e][1]);
     }
 }
 
@@ -1401,7 +1478,7 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
 #pragma unroll
                     for (int i = 0; i < 9; ++i) {
                         const R dref = ((info >> opp_(i)) & 1u) ? own
-                                                               : half_round(k ? sm.rr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].y : sm.rr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].x);
+                                                               : (k ? sm.hr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].y : sm.hr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].x);
                         Pop<S, R>::st(a.fout, (k * 9 + i) * a.plane + n, o2[k][i], w_<R>(i) * dref);
                     }
                     static_cast<__half*>(a.rref_out)[k * a.plane + n] = __float2half_rn(float(r));
@@ -1424,7 +1501,7 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
 #pragma unroll
                     for (int i = 0; i < 9; ++i) {
                         const R dref = ((info >> opp_(i)) & 1u) ? own
-                                                               : half_round(k ? sm.rr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].y : sm.rr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].x);
+                                                               : (k ? sm.hr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].y : sm.hr[ty + 2 + ey_(i)][tx + 2 + ex_(i)].x);
                         Pop<S, R>::st(a.fout, (k * 9 + i) * a.plane + n, o[i], w_<R>(i) * dref);
                     }
                     static_cast<__half*>(a.rref_out)[k * a.plane + n] = __float2half_rn(float(r));
@@ -1488,9 +1565,10 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
 }
 
 // Register cap of a general tile, within the 64 K register file for every
-// variant.  FP32 keeps 80 (measured on GB300: a 64-register cap spilled
-// ~0.5 KB per thread and made the step 20 % slower, although it would leave
-// room for a fifth fast tile on the SM).
+// variant.  FP32 tiles with staging roles keep 96 (both strip pulls are in
+// flight at once; at 80 they spill 0.3 KB: 8.56 us per 1024x128 step with 32x8
+// tiles against 7.89), serially staged ones 80, which leaves three on an SM (96:
+// 292 -> 295 us per 4096x2048 step, 72.5 -> 75.9 for 24 T-junctions).
 template <int TX, int TY, bool ROLES>
 __host__ __device__ constexpr int gen_threads() {
     return ROLES ? GenRoles<TX, TY>::THREADS : TX * TY;
@@ -1504,7 +1582,7 @@ template <typename R, int TX, int TY, bool ROLES>
 __host__ __device__ constexpr int gen_maxreg() {
     constexpr int warps = (gen_threads<TX, TY, ROLES>() + 31) / 32;
     constexpr int fit = 16384 / (((warps + 3) / 4) * 32) / 8 * 8;
-    constexpr int want = sizeof(R) == 4 ? 80 : 128;
+    constexpr int want = sizeof(R) == 4 ? (ROLES ? 96 : 80) : 128;
     return want < fit ? want : fit;
 }
 

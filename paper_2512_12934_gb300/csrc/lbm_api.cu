@@ -952,6 +952,23 @@ lbm_status build_tiles(lbm_ctx* c, int v, bool sync_first) {
 }
 
 
+// Default tile shape (lbm_set_tile_variant overrides): 32x8, whose halo ring
+// costs 0.69 pulls per node against 1.25 for 32x4 (variant 1).  Two kinds of
+// grid keep 32x4.  FP64 tiles hold half as many CTAs per SM: small FP64 grids
+// with open faces are faster with it.  With an open face on a y side the tile
+// height decides which nodes near it the general tiles collide (in packed
+// FP32x2 arithmetic, rounded differently in the last bit), and slow devices
+// amplify that to 2e-5 of u in 200 steps; their results are kept.  us per step,
+// 32x8 / 32x4: 100x100 periodic 3.70 / 4.02, 512x512 10.0 / 10.3, channels
+// 1024x128 7.9 / 9.0, 2048x512 46.1 / 46.7, 4096x1024 155 / 159, FP16 storage
+// 4001x1022 166 / 189, FP64 640x320 142.5 / 141.1, 960x320 194 / 201, 24
+// T-junctions in a batch 72.5 / 77.0.
+int default_variant(const lbm_ctx* c) {
+    const long long nodes = (long long)c->nx * c->ny;
+    if (c->precision == LBM_FP64) return c->nfaces > 0 && nodes < (1LL << 18) ? 1 : 0;
+    return (c->open_side[2] || c->open_side[3]) && nodes < (1LL << 22) ? 1 : 0;
+}
+
 // ---- snapshots (autotuning runs trial steps and then puts the state back) ----
 struct Snapshot {
     void* f = nullptr;
@@ -1647,10 +1664,7 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
     c->host_solid_in.assign(sol.begin(), sol.end());
     c->h_faceid = faceid;
     c->h_nbrid = nbrid;
-    // default tile shape: narrow tiles (more CTAs, shorter chains) for small
-    // grids, 32x8 for large ones (measured on GB300; lbm_set_tile_variant
-    // overrides)
-    lbm_status st = build_tiles(c, (long long)nx * ny < (1LL << 22) ? 1 : 0, false);
+    lbm_status st = build_tiles(c, default_variant(c), false);
     if (st != LBM_OK) {
         const std::string msg = c->err;
         free_ctx(c);

@@ -232,10 +232,11 @@ void d2q9_variant_tile(int variant, int* tx, int* ty) {
 }
 int d2q9_num_variants() { return (int)(sizeof(kVariants) / sizeof(kVariants[0])); }
 
-// A general list of at most two CTAs per SM is latency-bound: its tiles stage
-// with the extra GenRoles warps.  Longer lists (batched ensembles) fill the
-// GPU by themselves and stage serially on the node threads.
-static bool general_roles(int nblocks) {
+// A general list of at most 256 nodes per SM is latency-bound: its tiles stage
+// with the extra GenRoles warps.  Longer lists (batched ensembles, large grids)
+// fill the GPU by themselves and stage serially on the node threads.  The line
+// counts nodes, so that a list stages alike under every tile shape.
+static bool general_roles(int nblocks, int tile_nodes) {
     static int sms = 0;
     if (sms == 0) {
         int dev = 0;
@@ -243,7 +244,7 @@ static bool general_roles(int nblocks) {
                                                       cudaSuccess || sms <= 0)
             sms = 152;
     }
-    return nblocks <= 2 * sms;
+    return (long long)nblocks * tile_nodes <= 256LL * sms;
 }
 
 // (Serial staging is built for FP32 storage only, to bound compile time;
@@ -255,7 +256,7 @@ static void launch_tile(const D2Args<S, R>& a, bool general, int nblocks, cudaSt
         return;
     }
     if constexpr (std::is_same<S, float>::value) {
-        if (!general_roles(nblocks)) {
+        if (!general_roles(nblocks, TX * TY)) {
             d2q9_general_kernel<S, R, TX, TY, false><<<nblocks, TX * TY, 0, st>>>(a);
             return;
         }
@@ -270,7 +271,7 @@ static void launch_batch_tile(const BatchArgs<S, R>& b, bool general, int nblock
         return;
     }
     if constexpr (std::is_same<S, float>::value) {
-        if (!general_roles(nblocks)) {
+        if (!general_roles(nblocks, TX * TY)) {
             d2q9_batch_general_kernel<S, R, TX, TY, false><<<nblocks, TX * TY, 0, st>>>(b);
             return;
         }
