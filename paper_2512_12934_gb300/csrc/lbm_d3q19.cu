@@ -715,13 +715,23 @@ template <typename S, typename Put>
 __device__ __forceinline__ void stage_box(const D3Args<S>& a, int x0, int y0, int z0, bool inner, int tid, Put put) {
     using R = typename Store<S>::R;
     using V = typename Pair<R>::type;
+    constexpr int HN = Tile3<S>::HN, NT = Tile3<S>::NT, PASSES = (HN + NT - 1) / NT;
     const V* rp = reinterpret_cast<const V*>(a.rho);
-    for (int q = tid; q < Tile3<S>::HN; q += Tile3<S>::NT) {
-        const int hx = q % HX, hy = (q / HX) % HY, hz = q / (HX * HY);
-        const long long m = inner ? node_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz)
-                                  : site_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz);
-        put(q, m < 0 ? V{(R)0, (R)0} : rp[m]);
+    V v[PASSES];
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {  // every pass's load in flight before the first store
+        const int q = p * NT + tid;
+        v[p] = V{(R)0, (R)0};
+        if (q < HN) {
+            const int hx = q % HX, hy = (q / HX) % HY, hz = q / (HX * HY);
+            const long long m = inner ? node_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz)
+                                      : site_index(a, x0 - 2 + hx, y0 - 2 + hy, z0 - 2 + hz);
+            if (m >= 0) v[p] = rp[m];
+        }
     }
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p)
+        if (p * NT + tid < HN) put(p * NT + tid, v[p]);
 }
 
 // FP64 and FP16 storage.  Every fluid node of a 32x4x2 tile: forces from the
