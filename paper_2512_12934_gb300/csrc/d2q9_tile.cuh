@@ -225,8 +225,24 @@ __device__ __forceinline__ void pull_finish(const D2Args<S, R>& a, int x, int y,
     pull_wall(a, x, y, info, f);
 }
 
-// Whole pull of a node whose descriptor is known (serially staged tiles): each
-// source is selected before its one load, which takes fewer registers.
+// Whole pulls of a node whose descriptor is known (serially staged general tiles
+// and tiles whose arguments lie in shared memory, i.e. batches, where the early
+// loads spilled at 64 registers: 32 small T-junctions 44.4 us per step with
+// these, 45.4 with early loads): each source is selected before its one load.
+template <typename S, typename R>
+__device__ __forceinline__ void pull_interior(const D2Args<S, R>& a, int n, unsigned info, R (&f)[2][9]) {
+    R ref[2];
+    node_ref(a, n, ref);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const bool bb = (info >> i) & 1u;
+        const int src = bb ? n : n - ex_(i) - ey_(i) * a.pitch;
+        const int dir = bb ? opp_(i) : i;
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            f[k][i] = Pop<S, R>::ld(a.fin, (k * 9 + dir) * a.plane + src, w_<R>(i) * ref[k]);
+    }
+}
 template <typename S, typename R>
 __device__ __forceinline__ void pull_wrap(const D2Args<S, R>& a, int x, int y, unsigned info, R (&f)[2][9]) {
     const int n = y * a.pitch + x;
@@ -397,7 +413,8 @@ __device__ __forceinline__ bool resolve_closed(const D2Args<S, R>& a, int& gx, i
 
 // Tile modes: 0 deep interior, 1 edge (wrap / closed edges), 2 general.
 // Density pair of a halo site (no populations kept).  Returns false if solid.
-template <typename S, typename R, int MODE>
+// EARLY: the pull's loads go out before the descriptor is known.
+template <typename S, typename R, int MODE, bool EARLY>
 __device__ __forceinline__ bool site_rho(const D2Args<S, R>& a, int gx, int gy, R& r0, R& r1, R lam = R(0)) {
     if (MODE == 2) {
         if (resolve_site(a, gx, gy)) return false;
@@ -412,20 +429,26 @@ __device__ __forceinline__ bool site_rho(const D2Args<S, R>& a, int gx, int gy, 
         const int n = gy * a.pitch + gx;
         const unsigned inf = a.info[n];
         R ref[2], g[2][9];
-        node_ref(a, n, ref);
-        pull_load_wrap(a, gx, gy, ref, g);
+        if constexpr (EARLY) {
+            node_ref(a, n, ref);
+            pull_load_wrap(a, gx, gy, ref, g);
+        }
         if (inf & INFO_SOLID) return false;
-        pull_finish(a, gx, gy, inf, ref, g);
+        if constexpr (EARLY) pull_finish(a, gx, gy, inf, ref, g);
+        else pull_wrap(a, gx, gy, inf, g);
         r0 = rho_of(g[0]);
         r1 = rho_of(g[1]);
     } else {
         const int n = gy * a.pitch + gx;
         const unsigned inf = a.info[n];
         R ref[2], g[2][9];
-        node_ref(a, n, ref);
-        pull_load_interior(a, n, ref, g);
+        if constexpr (EARLY) {
+            node_ref(a, n, ref);
+            pull_load_interior(a, n, ref, g);
+        }
         if (inf & INFO_SOLID) return false;
-        pull_fix(a, n, inf, ref, g);
+        if constexpr (EARLY) pull_fix(a, n, inf, ref, g);
+        else pull_interior(a, n, inf, g);
         r0 = rho_of(g[0]);
         r1 = rho_of(g[1]);
     }
@@ -498,7 +521,7 @@ struct TileSmemGen : TileSmem<S, R, TX, TY> {
 
 // Stage the tile's densities (own node + two-node halo) in shared memory;
 // the own node's post-stream populations stay in registers.
-template <typename S, typename R, int TX, int TY, int MODE>
+template <typename S, typename R, int TX, int TY, int MODE, bool EARLY>
 __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R, TX, TY>& sm, int x0, int y0,
                                            int tx, int ty, R (&f)[2][9], unsigned& info, bool& fluid) {
     constexpr int RX = TX + 4, RY = TY + 4, NT = TX * TY;
@@ -514,27 +537,33 @@ __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R,
                 const int n = y * a.pitch + x;
                 info = a.info[n];
                 R ref[2];
-                node_ref(a, n, ref);
-                pull_load_wrap(a, x, y, ref, f);
+                if constexpr (EARLY) {
+                    node_ref(a, n, ref);
+                    pull_load_wrap(a, x, y, ref, f);
+                }
                 fluid = !(info & INFO_SOLID);
                 if (fluid) {
-                    pull_finish(a, x, y, info, ref, f);
+                    if constexpr (EARLY) pull_finish(a, x, y, info, ref, f);
+                    else pull_wrap(a, x, y, info, f);
                     r0 = rho_of(f[0]);
                     r1 = rho_of(f[1]);
                     sol = 0;
                 }
-            } else if (site_rho<S, R, MODE>(a, x, y, r0, r1)) {
+            } else if (site_rho<S, R, MODE, EARLY>(a, x, y, r0, r1)) {
                 sol = 0;
             }
         } else {
             const int n = y * a.pitch + x;
             info = a.info[n];
             R ref[2];
-            node_ref(a, n, ref);
-            pull_load_interior(a, n, ref, f);
+            if constexpr (EARLY) {
+                node_ref(a, n, ref);
+                pull_load_interior(a, n, ref, f);
+            }
             fluid = !(info & INFO_SOLID);
             if (fluid) {
-                pull_fix(a, n, info, ref, f);
+                if constexpr (EARLY) pull_fix(a, n, info, ref, f);
+                else pull_interior(a, n, info, f);
                 r0 = rho_of(f[0]);
                 r1 = rho_of(f[1]);
                 sol = 0;
@@ -560,7 +589,7 @@ __device__ __forceinline__ void stage_tile(const D2Args<S, R>& a, TileSmem<S, R,
             rx = c < 2 ? c : TX + c;
         }
         R h0 = R(0), h1 = R(0);
-        const bool ok = site_rho<S, R, MODE>(a, x0 - 2 + rx, y0 - 2 + ry, h0, h1);
+        const bool ok = site_rho<S, R, MODE, EARLY>(a, x0 - 2 + rx, y0 - 2 + ry, h0, h1);
         put_rho(sm, ry, rx, h0, h1);
         sm.sol[ry][rx] = ok ? 0 : 1;
     };
@@ -892,7 +921,7 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                     r0 = rho_of(f[0]);
                     r1 = rho_of(f[1]);
                     sol = 0;
-                } else if (site_rho<S, R, 2>(a, pend_x, pend_y, r0, r1, lam)) {
+                } else if (site_rho<S, R, 2, false>(a, pend_x, pend_y, r0, r1, lam)) {
                     sol = 0;
                 }
             } else {
@@ -1003,7 +1032,7 @@ __device__ __forceinline__ void stage_tile_compact(const D2Args<S, R>& a, TileSm
             }
             sol = 0;
         }
-    } else if (site_rho<S, R, 2>(a, x, y, r0, r1, lam)) {
+    } else if (site_rho<S, R, 2, false>(a, x, y, r0, r1, lam)) {
         sol = 0;
     }
     put_rho(sm, ty + 2, tx + 2, r0, r1);
@@ -1318,8 +1347,9 @@ __device__ __forceinline__ void collide_one(const D2Args<S, R>& a, int k, R r, R
 }
 
 // One tile of one step.  bxy = bx | by << 16; bflags = BLOCK_* flags; strips
-// and slot are used by general tiles only.
-template <typename S, typename R, int TX, int TY, bool GEN, bool ROLES = true>
+// and slot are used by general tiles only.  EARLY: fast tiles load before their
+// descriptors (see the pulls above).
+template <typename S, typename R, int TX, int TY, bool GEN, bool ROLES = true, bool EARLY = true>
 __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsigned bflags, unsigned strips,
                                           int slot) {
     constexpr int NT = TX * TY, NW = NT / 32;
@@ -1339,8 +1369,8 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
         stage_tile_general<S, R, TX, TY>(a, smx, x0, y0, strips, bflags, f, info, fluid);
     else if constexpr (GEN)
         stage_tile_compact<S, R, TX, TY>(a, smx, x0, y0, tx, ty, strips, bflags, f, info, fluid);
-    else if (bflags & BLOCK_EDGE) stage_tile<S, R, TX, TY, 1>(a, sm, x0, y0, tx, ty, f, info, fluid);
-    else stage_tile<S, R, TX, TY, 0>(a, sm, x0, y0, tx, ty, f, info, fluid);
+    else if (bflags & BLOCK_EDGE) stage_tile<S, R, TX, TY, 1, EARLY>(a, sm, x0, y0, tx, ty, f, info, fluid);
+    else stage_tile<S, R, TX, TY, 0, EARLY>(a, sm, x0, y0, tx, ty, f, info, fluid);
     __syncthreads();
     // general tiles: the ring and strip warps are done once the tile is staged
     if (GEN && tid >= NT) return;

@@ -48,8 +48,12 @@ template <typename S, typename R, int TX, int TY, bool GEN, bool ROLES = true>
 __device__ __forceinline__ void batch_tile(const BatchArgs<S, R>& b) {
     __shared__ D2Args<S, R> sa;
     grid_dep_wait();
+    // the tile's list entry travels beside the member's arguments
     const int li = b.off + blockIdx.x;
-    const int m = b.member[li];
+    const int m = b.member[li], blk = b.blocks[li];
+    const unsigned fl = b.flags[li];
+    const unsigned strips = GEN ? b.strips[li] : 0u;
+    const int slot = GEN ? b.slot[li] : -1;
     {
         static_assert(sizeof(D2Args<S, R>) % 4 == 0, "argument block must be word-sized");
         const int* src = reinterpret_cast<const int*>(b.args + m);
@@ -57,7 +61,7 @@ __device__ __forceinline__ void batch_tile(const BatchArgs<S, R>& b) {
         for (int i = threadIdx.x; i < (int)(sizeof(D2Args<S, R>) / 4); i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
-    step_tile<S, R, TX, TY, GEN, ROLES>(sa, b.blocks[li], b.flags[li], b.strips[li], b.slot[li]);
+    step_tile<S, R, TX, TY, GEN, ROLES, false>(sa, blk, fl, strips, slot);
 }
 
 template <typename S, typename R, int TX, int TY>

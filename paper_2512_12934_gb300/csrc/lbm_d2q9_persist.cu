@@ -73,7 +73,7 @@ __global__ void __maxnreg__((gen_maxreg<R, TX, TY, false>()))
                 for (int i = threadIdx.x; i < (int)(sizeof(D2Args<S, R>) / 4); i += blockDim.x) dst[i] = src[i];
             }
             __syncthreads();
-            if (t < p.nfast) step_tile<S, R, TX, TY, false>(sa, p.blocks[t], p.flags[t], 0u, -1);
+            if (t < p.nfast) step_tile<S, R, TX, TY, false, true, false>(sa, p.blocks[t], p.flags[t], 0u, -1);
             else step_tile<S, R, TX, TY, true, false>(sa, p.blocks[t], p.flags[t], p.strips[t], p.slot[t]);
         }
         if (s + 1 < p.nsteps && !grid_barrier(p, (unsigned)(s + 1) * gridDim.x + (unsigned)p.bar_skew)) return;
