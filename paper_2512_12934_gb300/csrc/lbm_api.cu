@@ -267,6 +267,7 @@ D2Args<S, R> make_args_par(lbm_ctx* c, int in, bool write_macros) {
     a.block_slot = c->block_slot;
     a.block_strips = c->block_strips;
     a.list_off = 0;
+    a.reverse = in;
     a.nfaces = c->nfaces;
     for (int i = 0; i < c->nfaces; ++i) a.face[i] = c->faces[i];
     a.out_face = c->out_face;
@@ -1168,6 +1169,7 @@ cudaError_t batch_launch(lbm_batch* b, bool macros, cudaStream_t st, cudaStream_
     a.strips = b->strips;
     a.member = b->member;
     a.off = 0;
+    a.reverse = b->bpar;
     cudaError_t e = cudaSuccess;
     const bool fork = side && b->nfast > 0 && b->ngeneral > 0;
     if (fork) {

@@ -75,6 +75,7 @@ struct D2Args {
     const int* __restrict__ block_slot;       // per list entry: flux-reduction slot or -1
     const unsigned* __restrict__ block_strips;  // per list entry: (side0 + 1) | (side1 + 1) << 8, 0 = none
     int list_off;                             // first list entry of this launch
+    int reverse;                              // fast tiles run from the end of their list (every other step)
     int nfaces;
     FaceDev face[MAX_FACES];
     int out_face;           // index of the outlet face or -1
@@ -126,6 +127,7 @@ struct BatchArgs {
     const unsigned* strips;
     const int* member;
     int off;
+    int reverse;  // tiles from the end of the launch's list (every other step)
 };
 
 template <typename S, typename R>
