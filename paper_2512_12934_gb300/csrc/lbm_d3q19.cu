@@ -1160,7 +1160,10 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
             Fp[q] = F[q].x;
             Fp[3 + q] = F[q].y;
         }
-        if (Fc.kind == FACE3_OUTLET) return;  // finished by d3q_outlet_kernel
+        if (Fc.kind == FACE3_OUTLET) {  // finished by d3q_outlet_kernel
+            asm volatile("cp.async.wait_all;" ::: "memory");  // no copy outlives its thread
+            return;
+        }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     auto pop = [&](int i) { return ld_shared2(s_f + 8u * NT * i); };
