@@ -400,7 +400,8 @@ lbm_status ensure_graph(lbm_ctx* c, int size, int par) {
 template <typename S, typename R>
 lbm_status run_plain(lbm_ctx* c, int64_t cnt) {
     const int per = (c->nfast > 0) + (c->ngeneral > 0) + (c->nmarch > 0) + (c->chi_same_step ? 1 : 0);
-    for (int size = 0; size < kGraphSizes; ++size)
+    const bool replay = cnt >= kGraphSteps[kGraphSizes - 1] && !stream_capturing(c->stream);
+    for (int size = 0; size < kGraphSizes && replay; ++size)
         while (c->use_graphs && cnt >= kGraphSteps[size]) {
             if (ensure_graph<S, R>(c, size, c->cur) != LBM_OK) {
                 c->use_graphs = 0;  // capture unavailable: keep launching the same kernel directly
@@ -1284,10 +1285,11 @@ lbm_status batch_run(lbm_batch* b, int64_t n) {
         }
     if (b->schedule == LBM_SCHEDULE_PERSISTENT) return batch_run_persistent<S, R>(b, n);
     int64_t rem = n;
+    const bool replay = rem > kGraphSteps[kGraphSizes - 1] && !stream_capturing(b->stream);
     while (rem > 1) {
         int size = 0;
         while (size < kGraphSizes && rem - 1 < kGraphSteps[size]) ++size;
-        if (b->use_graphs && size < kGraphSizes) {
+        if (replay && b->use_graphs && size < kGraphSizes) {
             if (batch_graph<S, R>(b, size, b->bpar) != LBM_OK) {
                 b->use_graphs = 0;
                 cudaGetLastError();

@@ -768,11 +768,7 @@ lbm_status step(Ctx3* c, int64_t nsteps) {
     // the call's last step writes u^eq and runs on its own; sampled runs and
     // streams under capture take plain launches throughout
     while (c->use_graphs && c->time_every == 0 && nsteps - 1 - s >= kGraphSteps3) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            break;
-        }
+        if (lbm::stream_capturing(c->stream)) break;
         if (!ensure_graph3(c)) {
             c->use_graphs = 0;
             break;

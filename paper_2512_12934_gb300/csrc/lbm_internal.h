@@ -209,6 +209,16 @@ inline bool kernel_writable(const void* p) {
             at.type == cudaMemoryTypeHost);
 }
 
+// Whether work on st is being recorded into a stream capture (or that cannot be
+// told).  A graph launch cannot be recorded; plain launches can, so step runs
+// are launched step by step then.
+inline bool stream_capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Dense macroscopic fields rho [2][ny][nx], u [2][ny][nx] from macro [4][plane]
 // (0 at solid nodes); rho and u may be device or mapped host memory.  Nothing
 // is written when *status is set; *status_out (mapped host memory) receives it.
