@@ -334,8 +334,10 @@ lbm_status lbm_mass_noalloc(const void* f, int precision, int nx, int ny, int pi
  * existing contexts (the members, created with lbm_create, all of one
  * precision); the caller keeps owning them and may still read them between
  * batch steps (lbm_get_macros, lbm_get_diagnostics, ...).  Every member takes
- * the batch's tile variant.  A batch step advances every member by one time
- * step with exactly the arithmetic of lbm_step on that member alone. */
+ * the batch's tile variant: the one set or autotuned for a member (the first
+ * such member's), else 1 if that is any member's default, else 0.  A batch
+ * step advances every member by one time step with exactly the arithmetic of
+ * lbm_step on that member alone. */
 typedef struct lbm_batch lbm_batch;
 
 /* members: n >= 1 distinct contexts of one precision; cuda_stream: the stream

@@ -117,6 +117,7 @@ struct lbm_ctx {
     int open_side[4] = {0, 0, 0, 0};
     int nface_nodes = 0;
     int xoff = 0, yoff = 0, variant = 0, tx = 32, ty = 8;
+    bool variant_chosen = false;  // by the caller (set or autotuned); else default_variant's
     dim3 gdim;
     int cur = 0;
     int64_t step = 0;
@@ -971,6 +972,20 @@ int default_variant(const lbm_ctx* c) {
     return (c->open_side[2] || c->open_side[3]) && nodes < (1LL << 22) ? 1 : 0;
 }
 
+// Tile variant of a new batch, whatever the order of its members: the one that
+// the caller chose for a member (the first such), else 32x4 if that is any
+// member's default.  A member with the 32x4 default keeps its results (see
+// above); those of the others do not depend on the shape but for the last bit
+// of chi (the grouping of its FP64 partials).
+int batch_variant(const std::vector<lbm_ctx*>& members) {
+    int v = 0;
+    for (const lbm_ctx* c : members) {
+        if (c->variant_chosen) return d2q9_tile_kernel_variant(c->variant);
+        v = std::max(v, default_variant(c));
+    }
+    return v;
+}
+
 // ---- snapshots (autotuning runs trial steps and then puts the state back) ----
 struct Snapshot {
     void* f = nullptr;
@@ -1372,6 +1387,7 @@ lbm_status batch_autotune(lbm_batch* b, int steps, int* chosen, double* best_ms)
         if (st == LBM_OK) st = s2;
     }
     if (st != LBM_OK) return st;
+    for (lbm_ctx* c : b->m) c->variant_chosen = true;
     b->variant = best;
     st = batch_build_any(b);
     *chosen = best;
@@ -2002,7 +2018,9 @@ lbm_status lbm_kernel_time_split(lbm_ctx* c, double* fast_ms, double* general_ms
 lbm_status lbm_set_tile_variant(lbm_ctx* c, int variant) {
     if (!c) return fail(nullptr, LBM_ERR_INVALID_ARG, "ctx is NULL");
     if (c->d3) return fail(c, LBM_ERR_UNSUPPORTED, "not implemented for D3Q19 contexts");
-    return build_tiles(c, variant, true);
+    lbm_status st = build_tiles(c, variant, true);
+    if (st == LBM_OK) c->variant_chosen = true;
+    return st;
 }
 
 int lbm_num_tile_variants(void) { return d2q9_num_variants(); }
@@ -2048,7 +2066,7 @@ lbm_status lbm_batch_create(lbm_ctx* const* members, int n, void* cuda_stream, l
     b->m.assign(members, members + n);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     b->precision = members[0]->precision;
-    b->variant = members[0]->variant;
+    b->variant = batch_variant(b->m);
     lbm_status st = LBM_OK;
     for (lbm_ctx* c : b->m)
         if (st == LBM_OK && c->variant != b->variant) st = build_tiles(c, b->variant, true);
@@ -2097,6 +2115,7 @@ lbm_status lbm_batch_set_tile_variant(lbm_batch* b, int variant) {
     for (lbm_ctx* c : b->m) {
         lbm_status st = build_tiles(c, variant, true);
         if (st != LBM_OK) return bfail(b, st, c->err);
+        c->variant_chosen = true;
     }
     b->variant = variant;
     return batch_build_any(b);
