@@ -1595,10 +1595,15 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
 }
 
 // Register cap of a general tile, within the 64 K register file for every
-// variant.  FP32 tiles with staging roles keep 96 (both strip pulls are in
-// flight at once; at 80 they spill 0.3 KB: 8.56 us per 1024x128 step with 32x8
-// tiles against 7.89), serially staged ones 80, which leaves three on an SM (96:
-// 292 -> 295 us per 4096x2048 step, 72.5 -> 75.9 for 24 T-junctions).
+// variant.  FP32 tiles of more than 128 nodes with staging roles have an SM to
+// themselves at any cap and keep 96 (both strip pulls are in flight at once; at
+// 80 they spill 0.3 KB: 8.56 us per 1024x128 step with 32x8 tiles against 7.7).
+// Those of 32x4 nodes keep 80, at which two share an SM and more fast tiles fit
+// beside one.  us per step at 96 / 80: T-junction batches 8 x 24-38 wide 19.1 /
+// 16.7, 12 x 24-40 26.7 / 21.1, FP16 storage 24 x 24-72 96.4 / 82.5, one device
+// 100 wide 12.5 / 11.7.  A short list leaves the SMs to its tiles either way and
+// runs at 96 (launch_tile).  Serially staged tiles keep 80, which leaves three on
+// an SM (96: 292 -> 295 us per 4096x2048 step, 72.5 -> 75.9 for 24 T-junctions).
 template <int TX, int TY, bool ROLES>
 __host__ __device__ constexpr int gen_threads() {
     return ROLES ? GenRoles<TX, TY>::THREADS : TX * TY;
@@ -1612,9 +1617,12 @@ template <typename R, int TX, int TY, bool ROLES>
 __host__ __device__ constexpr int gen_maxreg() {
     constexpr int warps = (gen_threads<TX, TY, ROLES>() + 31) / 32;
     constexpr int fit = 16384 / (((warps + 3) / 4) * 32) / 8 * 8;
-    constexpr int want = sizeof(R) == 4 ? (ROLES ? 96 : 80) : 128;
+    constexpr int want = sizeof(R) == 4 ? (ROLES && TX * TY > 128 ? 96 : 80) : 128;
     return want < fit ? want : fit;
 }
+// Two 32x4 tiles with staging roles share an SM.
+static_assert(2 * ((GenRoles<32, 4>::THREADS / 32 + 3) / 4) * 32 * gen_maxreg<float, 32, 4, true>() <= 16384,
+              "a 32x4 general tile must leave half of the register file");
 
 }  // namespace
 }  // namespace lbm

@@ -338,15 +338,15 @@ cudaError_t launch_lists(lbm_ctx* c, bool macros, cudaStream_t st, cudaStream_t 
     // same-step chi: the outlet nodes are collided after the general tiles
     // (on their stream), once the step's flux partials exist
     const bool chi_same = a.oc_save != nullptr;
-    if (fork && e == cudaSuccess) e = launch_d2q9_step<S, R>(ag, c->variant, true, c->ngeneral, side);
+    if (fork && e == cudaSuccess) e = launch_d2q9_step<S, R>(ag, c->variant, true, c->ngeneral, c->nfast, side);
     if (fork && chi_same && e == cudaSuccess) e = launch_d2q9_outlet_chi<S, R>(a, side);
     if constexpr (std::is_same<S, float>::value && std::is_same<R, float>::value) {
         if (e == cudaSuccess && c->nmarch > 0)
             e = launch_d2q9_march(a, &c->tmap[c->cur], c->march_runs, c->march_flags, c->nmarch, st);
     }
-    if (e == cudaSuccess) e = launch_d2q9_step<S, R>(a, c->variant, false, c->nfast, st);
+    if (e == cudaSuccess) e = launch_d2q9_step<S, R>(a, c->variant, false, c->nfast, c->ngeneral, st);
     if (e == cudaSuccess && mid) e = cudaEventRecord(mid, st);
-    if (!fork && e == cudaSuccess) e = launch_d2q9_step<S, R>(ag, c->variant, true, c->ngeneral, st);
+    if (!fork && e == cudaSuccess) e = launch_d2q9_step<S, R>(ag, c->variant, true, c->ngeneral, c->nfast, st);
     if (!fork && chi_same && e == cudaSuccess) e = launch_d2q9_outlet_chi<S, R>(a, st);
     if (fork && e == cudaSuccess) {
         e = cudaEventRecord(c->ev_join, side);
@@ -1195,9 +1195,9 @@ cudaError_t batch_launch(lbm_batch* b, bool macros, cudaStream_t st, cudaStream_
     // general list first when forked (see launch_lists)
     BatchArgs<S, R> ag = a;
     ag.off = b->nfast;
-    if (fork && e == cudaSuccess) e = launch_d2q9_batch<S, R>(ag, b->variant, true, b->ngeneral, side);
-    if (e == cudaSuccess) e = launch_d2q9_batch<S, R>(a, b->variant, false, b->nfast, st);
-    if (!fork && e == cudaSuccess) e = launch_d2q9_batch<S, R>(ag, b->variant, true, b->ngeneral, st);
+    if (fork && e == cudaSuccess) e = launch_d2q9_batch<S, R>(ag, b->variant, true, b->ngeneral, b->nfast, side);
+    if (e == cudaSuccess) e = launch_d2q9_batch<S, R>(a, b->variant, false, b->nfast, b->ngeneral, st);
+    if (!fork && e == cudaSuccess) e = launch_d2q9_batch<S, R>(ag, b->variant, true, b->ngeneral, b->nfast, st);
     if (fork && e == cudaSuccess) {
         e = cudaEventRecord(b->ev_join, side);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->ev_join, 0);

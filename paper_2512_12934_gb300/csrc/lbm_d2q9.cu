@@ -38,8 +38,8 @@ __global__ void __launch_bounds__(TX * TY, (fast_min_blocks<R, TX, TY>())) d2q9_
     step_tile<S, R, TX, TY, false>(a, a.blocks[li], a.block_flags[li], 0u, -1);
 }
 
-template <typename S, typename R, int TX, int TY, bool ROLES>
-__global__ void __maxnreg__((gen_maxreg<R, TX, TY, ROLES>())) d2q9_general_kernel(const __grid_constant__ D2Args<S, R> a) {
+template <typename S, typename R, int TX, int TY, bool ROLES, int MAXREG = gen_maxreg<R, TX, TY, ROLES>()>
+__global__ void __maxnreg__(MAXREG) d2q9_general_kernel(const __grid_constant__ D2Args<S, R> a) {
     grid_dep_wait();
     const int li = a.list_off + blockIdx.x;
     step_tile<S, R, TX, TY, true, ROLES>(a, a.blocks[li], a.block_flags[li], a.block_strips[li], a.block_slot[li]);
@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(TX * TY, (fast_min_blocks<R, TX, TY>())) d2q9_
     batch_tile<S, R, TX, TY, false>(b);
 }
 
-template <typename S, typename R, int TX, int TY, bool ROLES>
-__global__ void __maxnreg__((gen_maxreg<R, TX, TY, ROLES>())) d2q9_batch_general_kernel(const __grid_constant__ BatchArgs<S, R> b) {
+template <typename S, typename R, int TX, int TY, bool ROLES, int MAXREG = gen_maxreg<R, TX, TY, ROLES>()>
+__global__ void __maxnreg__(MAXREG) d2q9_batch_general_kernel(const __grid_constant__ BatchArgs<S, R> b) {
     batch_tile<S, R, TX, TY, true, ROLES>(b);
 }
 
@@ -240,11 +240,7 @@ void d2q9_variant_tile(int variant, int* tx, int* ty) {
 }
 int d2q9_num_variants() { return (int)(sizeof(kVariants) / sizeof(kVariants[0])); }
 
-// A general list of at most 256 nodes per SM is latency-bound: its tiles stage
-// with the extra GenRoles warps.  Longer lists (batched ensembles, large grids)
-// fill the GPU by themselves and stage serially on the node threads.  The line
-// counts nodes, so that a list stages alike under every tile shape.
-static bool general_roles(int nblocks, int tile_nodes) {
+int device_sms() {
     static int sms = 0;
     if (sms == 0) {
         int dev = 0;
@@ -252,13 +248,32 @@ static bool general_roles(int nblocks, int tile_nodes) {
                                                       cudaSuccess || sms <= 0)
             sms = 152;
     }
-    return (long long)nblocks * tile_nodes <= 256LL * sms;
+    return sms;
+}
+
+// A general list of at most 256 nodes per SM is latency-bound: its tiles stage
+// with the extra GenRoles warps.  Longer lists (batched ensembles, large grids)
+// fill the GPU by themselves and stage serially on the node threads.  The line
+// counts nodes, so that a list stages alike under every tile shape.
+static bool general_roles(int nblocks, int tile_nodes) { return (long long)nblocks * tile_nodes <= 256LL * device_sms(); }
+
+// Whether 32x4 general tiles (384 threads) at 96 registers, one to an SM, find
+// room beside the fast tiles (128 threads at 64): a step whose two lists fit the
+// register files together then is one wave, its general tiles do not spill and
+// it is faster; beyond that a general tile keeps fast tiles off its SM.  The
+// line: lists of up to half the SMs, 4.5 fast tiles' registers each, that leave
+// room for the fast list at 8 to an SM.  us per step at 96 / 80, general + fast
+// tiles: 30 + 408 8.0 / 8.4, 42 + 885 8.8 / 10.2, 58 + 924 10.6 / 10.6, 64 + 960
+// 10.2 / 8.6, 58 + 1730 12.4 / 11.6; batches 72 + 276 8.9 / 9.6, 58 + 536 9.6 /
+// 11.1, 78 + 748 13.2 / 12.0, 106 + 572 13.3 / 12.0.
+static bool room_for_large_tiles(int general, int fast) {
+    return 2 * general <= device_sms() && 9 * general + 2 * fast <= 16 * device_sms();
 }
 
 // (Serial staging is built for FP32 storage only, to bound compile time;
 // the other precisions always stage with GenRoles.)
 template <typename S, typename R, int TX, int TY>
-static void launch_tile(const D2Args<S, R>& a, bool general, int nblocks, cudaStream_t st) {
+static void launch_tile(const D2Args<S, R>& a, bool general, int nblocks, int beside, cudaStream_t st) {
     if (!general) {
         d2q9_step_kernel<S, R, TX, TY, false><<<nblocks, TX * TY, 0, st>>>(a);
         return;
@@ -268,12 +283,17 @@ static void launch_tile(const D2Args<S, R>& a, bool general, int nblocks, cudaSt
             d2q9_general_kernel<S, R, TX, TY, false><<<nblocks, TX * TY, 0, st>>>(a);
             return;
         }
+        if constexpr (TX * TY == 128)
+            if (room_for_large_tiles(nblocks, beside)) {
+                d2q9_general_kernel<S, R, TX, TY, true, 96><<<nblocks, GenRoles<TX, TY>::THREADS, 0, st>>>(a);
+                return;
+            }
     }
     d2q9_general_kernel<S, R, TX, TY, true><<<nblocks, GenRoles<TX, TY>::THREADS, 0, st>>>(a);
 }
 
 template <typename S, typename R, int TX, int TY>
-static void launch_batch_tile(const BatchArgs<S, R>& b, bool general, int nblocks, cudaStream_t st) {
+static void launch_batch_tile(const BatchArgs<S, R>& b, bool general, int nblocks, int beside, cudaStream_t st) {
     if (!general) {
         d2q9_batch_kernel<S, R, TX, TY><<<nblocks, TX * TY, 0, st>>>(b);
         return;
@@ -283,31 +303,38 @@ static void launch_batch_tile(const BatchArgs<S, R>& b, bool general, int nblock
             d2q9_batch_general_kernel<S, R, TX, TY, false><<<nblocks, TX * TY, 0, st>>>(b);
             return;
         }
+        if constexpr (TX * TY == 128)
+            if (room_for_large_tiles(nblocks, beside)) {
+                d2q9_batch_general_kernel<S, R, TX, TY, true, 96><<<nblocks, GenRoles<TX, TY>::THREADS, 0, st>>>(b);
+                return;
+            }
     }
     d2q9_batch_general_kernel<S, R, TX, TY, true><<<nblocks, GenRoles<TX, TY>::THREADS, 0, st>>>(b);
 }
 
 template <typename S, typename R>
-cudaError_t launch_d2q9_batch(const BatchArgs<S, R>& b, int variant, bool general, int nblocks, cudaStream_t st) {
+cudaError_t launch_d2q9_batch(const BatchArgs<S, R>& b, int variant, bool general, int nblocks, int beside,
+                              cudaStream_t st) {
     if (nblocks <= 0) return cudaSuccess;
     switch (d2q9_tile_kernel_variant(variant)) {
-    case 0: launch_batch_tile<S, R, 32, 8>(b, general, nblocks, st); break;
-    case 1: launch_batch_tile<S, R, 32, 4>(b, general, nblocks, st); break;
-    case 2: launch_batch_tile<S, R, 64, 4>(b, general, nblocks, st); break;
-    case 3: launch_batch_tile<S, R, 32, 16>(b, general, nblocks, st); break;
+    case 0: launch_batch_tile<S, R, 32, 8>(b, general, nblocks, beside, st); break;
+    case 1: launch_batch_tile<S, R, 32, 4>(b, general, nblocks, beside, st); break;
+    case 2: launch_batch_tile<S, R, 64, 4>(b, general, nblocks, beside, st); break;
+    case 3: launch_batch_tile<S, R, 32, 16>(b, general, nblocks, beside, st); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
 template <typename S, typename R>
-cudaError_t launch_d2q9_step(const D2Args<S, R>& a, int variant, bool general, int nblocks, cudaStream_t st) {
+cudaError_t launch_d2q9_step(const D2Args<S, R>& a, int variant, bool general, int nblocks, int beside,
+                             cudaStream_t st) {
     if (nblocks <= 0) return cudaSuccess;
     switch (d2q9_tile_kernel_variant(variant)) {
-    case 0: launch_tile<S, R, 32, 8>(a, general, nblocks, st); break;
-    case 1: launch_tile<S, R, 32, 4>(a, general, nblocks, st); break;
-    case 2: launch_tile<S, R, 64, 4>(a, general, nblocks, st); break;
-    case 3: launch_tile<S, R, 32, 16>(a, general, nblocks, st); break;
+    case 0: launch_tile<S, R, 32, 8>(a, general, nblocks, beside, st); break;
+    case 1: launch_tile<S, R, 32, 4>(a, general, nblocks, beside, st); break;
+    case 2: launch_tile<S, R, 64, 4>(a, general, nblocks, beside, st); break;
+    case 3: launch_tile<S, R, 32, 16>(a, general, nblocks, beside, st); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -339,12 +366,12 @@ cudaError_t launch_d2q9_diag(const S* f, const R* macro, const uint16_t* info, c
     return cudaGetLastError();
 }
 
-template cudaError_t launch_d2q9_batch<float, float>(const BatchArgs<float, float>&, int, bool, int, cudaStream_t);
-template cudaError_t launch_d2q9_batch<double, double>(const BatchArgs<double, double>&, int, bool, int, cudaStream_t);
-template cudaError_t launch_d2q9_batch<__half, float>(const BatchArgs<__half, float>&, int, bool, int, cudaStream_t);
-template cudaError_t launch_d2q9_step<float, float>(const D2Args<float, float>&, int, bool, int, cudaStream_t);
-template cudaError_t launch_d2q9_step<double, double>(const D2Args<double, double>&, int, bool, int, cudaStream_t);
-template cudaError_t launch_d2q9_step<__half, float>(const D2Args<__half, float>&, int, bool, int, cudaStream_t);
+template cudaError_t launch_d2q9_batch<float, float>(const BatchArgs<float, float>&, int, bool, int, int, cudaStream_t);
+template cudaError_t launch_d2q9_batch<double, double>(const BatchArgs<double, double>&, int, bool, int, int, cudaStream_t);
+template cudaError_t launch_d2q9_batch<__half, float>(const BatchArgs<__half, float>&, int, bool, int, int, cudaStream_t);
+template cudaError_t launch_d2q9_step<float, float>(const D2Args<float, float>&, int, bool, int, int, cudaStream_t);
+template cudaError_t launch_d2q9_step<double, double>(const D2Args<double, double>&, int, bool, int, int, cudaStream_t);
+template cudaError_t launch_d2q9_step<__half, float>(const D2Args<__half, float>&, int, bool, int, int, cudaStream_t);
 template cudaError_t launch_d2q9_outlet_chi<float, float>(const D2Args<float, float>&, cudaStream_t);
 template cudaError_t launch_d2q9_outlet_chi<double, double>(const D2Args<double, double>&, cudaStream_t);
 template cudaError_t launch_d2q9_outlet_chi<__half, float>(const D2Args<__half, float>&, cudaStream_t);

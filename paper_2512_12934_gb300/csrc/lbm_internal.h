@@ -131,7 +131,8 @@ struct BatchArgs {
 };
 
 template <typename S, typename R>
-cudaError_t launch_d2q9_batch(const BatchArgs<S, R>& b, int variant, bool general, int nblocks, cudaStream_t st);
+cudaError_t launch_d2q9_batch(const BatchArgs<S, R>& b, int variant, bool general, int nblocks, int beside,
+                              cudaStream_t st);
 
 // Persistent multi-step launch over a batch's tile list (lbm_d2q9_persist.cu).
 // Step s of the launch uses the argument blocks args[s & 1] (args_last[s & 1]
@@ -164,9 +165,11 @@ template <typename S, typename R>
 cudaError_t launch_d2q9_persist(const PersistArgs<S, R>& p, int variant, cudaStream_t st, int* grid_out);
 
 // Launch one list of tiles of one step: general = false -> fast kernel,
-// true -> general kernel; nblocks list entries starting at a.list_off.
+// true -> general kernel; nblocks list entries starting at a.list_off; beside:
+// entries of the step's other list.
 template <typename S, typename R>
-cudaError_t launch_d2q9_step(const D2Args<S, R>& a, int variant, bool general, int nblocks, cudaStream_t st);
+cudaError_t launch_d2q9_step(const D2Args<S, R>& a, int variant, bool general, int nblocks, int beside,
+                             cudaStream_t st);
 
 // Same-step chi: after the general tiles of a step, fold that step's flux
 // partials into chi (Eq. 23 at t + dt), set the outlet nodes' normal
