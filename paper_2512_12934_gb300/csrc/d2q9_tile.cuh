@@ -735,7 +735,8 @@ __device__ __forceinline__ void fold_finish(const D2Args<S, R>& a, const LamFold
     fold_finish(a, L, lam, chi, a.part_in, a.scal_in);
 }
 
-template <typename S, typename R, int TX, int TY>
+// EARLY: the own, ring and strip pulls' loads go out before the descriptors.
+template <typename S, typename R, int TX, int TY, bool EARLY>
 __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSmemGen<S, R, TX, TY>& sm, int x0,
                                                    int y0, unsigned strips, unsigned bflags, R (&f)[2][9],
                                                    unsigned& info, bool& fluid) {
@@ -766,8 +767,10 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         if (x >= 0 && x < a.nx && y >= 0 && y < a.ny) {
             info = a.info[y * a.pitch + x];
             R ref[2];
-            node_ref(a, y * a.pitch + x, ref);
-            pull_load_wrap(a, x, y, ref, f);
+            if constexpr (EARLY) {
+                node_ref(a, y * a.pitch + x, ref);
+                pull_load_wrap(a, x, y, ref, f);
+            }
             fluid = !(info & INFO_SOLID);
             if (fluid) {
                 sol = 0;
@@ -778,7 +781,8 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                     own_idx = side <= 1 ? ty : tx;
                     if (own_strip < 0) pending = true;
                 } else {
-                    pull_finish(a, x, y, info, ref, f);
+                    if constexpr (EARLY) pull_finish(a, x, y, info, ref, f);
+                    else pull_wrap(a, x, y, info, f);
                     r0 = rho_of(f[0]);
                     r1 = rho_of(f[1]);
                 }
@@ -802,8 +806,10 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         if (!resolve_site(a, gx, gy)) {
             const unsigned inf = a.info[gy * a.pitch + gx];
             R ref[2], g[2][9];
-            node_ref(a, gy * a.pitch + gx, ref);
-            pull_load_wrap(a, gx, gy, ref, g);
+            if constexpr (EARLY) {
+                node_ref(a, gy * a.pitch + gx, ref);
+                pull_load_wrap(a, gx, gy, ref, g);
+            }
             if (!(inf & INFO_SOLID)) {
                 hs = 0;
                 const int fid = (int)((inf >> INFO_FACE_SHIFT) & 7u);
@@ -825,7 +831,8 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                         pend_info = inf;
                     }
                 } else {
-                    pull_finish(a, gx, gy, inf, ref, g);
+                    if constexpr (EARLY) pull_finish(a, gx, gy, inf, ref, g);
+                    else pull_wrap(a, gx, gy, inf, g);
                     h0 = rho_of(g[0]);
                     h1 = rho_of(g[1]);
                 }
@@ -854,14 +861,16 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
                 // the inward neighbour along this strip's normal, read with
                 // the node's own word (a corner node may belong to the face of
                 // the other side; it is re-read below then).  Both pulls are in
-                // flight before either word is needed and before lambda is
-                // folded; only the blend of Eqs. 13-20 waits for it
+                // flight before lambda is folded (EARLY: before either word is
+                // needed); only the blend of Eqs. 13-20 waits for it
                 const int x2 = sx - side_ox(side), y2 = sy - side_oy(side);
                 inf2 = a.info[y2 * a.pitch + x2];
-                node_ref(a, sy * a.pitch + sx, ref);
-                node_ref(a, y2 * a.pitch + x2, ref2);
-                pull_load_wrap(a, sx, sy, ref, g);
-                pull_load_wrap(a, x2, y2, ref2, gn);
+                if constexpr (EARLY) {
+                    node_ref(a, sy * a.pitch + sx, ref);
+                    node_ref(a, y2 * a.pitch + x2, ref2);
+                    pull_load_wrap(a, sx, sy, ref, g);
+                    pull_load_wrap(a, x2, y2, ref2, gn);
+                }
             }
         }
         const bool face = !(inf & INFO_SOLID) && ((inf >> INFO_FACE_SHIFT) & 7u);
@@ -869,9 +878,15 @@ __device__ __forceinline__ void stage_tile_general(const D2Args<S, R>& a, TileSm
         const int fside = face ? a.face[fid].side : 0;
         if (face) {
             const int x2 = sx - side_ox(fside), y2 = sy - side_oy(fside);
-            pull_finish(a, sx, sy, inf, ref, g);
-            if (fside != side) pull_wrap(a, x2, y2, a.info[y2 * a.pitch + x2], gn);
-            else pull_finish(a, x2, y2, inf2, ref2, gn);
+            if constexpr (EARLY) {
+                pull_finish(a, sx, sy, inf, ref, g);
+                if (fside != side) pull_wrap(a, x2, y2, a.info[y2 * a.pitch + x2], gn);
+                else pull_finish(a, x2, y2, inf2, ref2, gn);
+            } else {
+                if (fside != side) inf2 = a.info[y2 * a.pitch + x2];
+                pull_wrap(a, sx, sy, inf, g);
+                pull_wrap(a, x2, y2, inf2, gn);
+            }
         }
         R lam = R(0);
         if (lam_on) {
@@ -1346,9 +1361,42 @@ __device__ __forceinline__ void collide_one(const D2Args<S, R>& a, int k, R r, R
         collide_scalar<R>(a.s[k], a.h[k], r, fx, fy, ux, uy, uu3, g, o);
 }
 
+// Register cap of a general tile, within the 64 K register file for every
+// variant.  FP32 tiles of more than 128 nodes with staging roles have an SM to
+// themselves at any cap and keep 96 (both strip pulls are in flight at once; at
+// 80 they spill 0.3 KB: 8.56 us per 1024x128 step with 32x8 tiles against 7.7).
+// Those of 32x4 nodes keep 80, at which two share an SM and more fast tiles fit
+// beside one.  us per step at 96 / 80: T-junction batches 8 x 24-38 wide 19.1 /
+// 16.7, 12 x 24-40 26.7 / 21.1, FP16 storage 24 x 24-72 96.4 / 82.5, one device
+// 100 wide 12.5 / 11.7.  A short list leaves the SMs to its tiles either way and
+// runs at 96 (launch_tile).  Serially staged tiles keep 80, which leaves three on
+// an SM (96: 292 -> 295 us per 4096x2048 step, 72.5 -> 75.9 for 24 T-junctions).
+template <int TX, int TY, bool ROLES>
+__host__ __device__ constexpr int gen_threads() {
+    return ROLES ? GenRoles<TX, TY>::THREADS : TX * TY;
+}
+
+// The warps of a CTA are spread over the SM's four sub-partitions, each with
+// 16 K registers, so the cap must let ceil(warps / 4) warps fit in 16 K (a
+// cap checked against the whole 64 K file alone can leave a block that does
+// not launch: 17 warps at 120 registers need 19,200 in one sub-partition).
+template <typename R, int TX, int TY, bool ROLES>
+__host__ __device__ constexpr int gen_maxreg() {
+    constexpr int warps = (gen_threads<TX, TY, ROLES>() + 31) / 32;
+    constexpr int fit = 16384 / (((warps + 3) / 4) * 32) / 8 * 8;
+    constexpr int want = sizeof(R) == 4 ? (ROLES && TX * TY > 128 ? 96 : 80) : 128;
+    return want < fit ? want : fit;
+}
+// Two 32x4 tiles with staging roles share an SM.
+static_assert(2 * ((GenRoles<32, 4>::THREADS / 32 + 3) / 4) * 32 * gen_maxreg<float, 32, 4, true>() <= 16384,
+              "a 32x4 general tile must leave half of the register file");
+
 // One tile of one step.  bxy = bx | by << 16; bflags = BLOCK_* flags; strips
 // and slot are used by general tiles only.  EARLY: fast tiles load before their
-// descriptors (see the pulls above).
+// descriptors (see the pulls above).  With FP16 storage general tiles do so only
+// at 96 registers: a thread's two pulls are converted at once, and at 80 the
+// 32x4 kernels lost more than the latency gains (us per step, early / not: one
+// T-junction 24 wide 9.3 / 8.5, a batch of 4, 24-40 wide, 12.8 / 11.5).
 template <typename S, typename R, int TX, int TY, bool GEN, bool ROLES = true, bool EARLY = true>
 __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsigned bflags, unsigned strips,
                                           int slot) {
@@ -1366,7 +1414,8 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
     unsigned info;
     bool fluid;
     if constexpr (GEN && ROLES)
-        stage_tile_general<S, R, TX, TY>(a, smx, x0, y0, strips, bflags, f, info, fluid);
+        stage_tile_general<S, R, TX, TY, !is_half_<S>() || gen_maxreg<R, TX, TY, ROLES>() >= 96>(
+            a, smx, x0, y0, strips, bflags, f, info, fluid);
     else if constexpr (GEN)
         stage_tile_compact<S, R, TX, TY>(a, smx, x0, y0, tx, ty, strips, bflags, f, info, fluid);
     else if (bflags & BLOCK_EDGE) stage_tile<S, R, TX, TY, 1, EARLY>(a, sm, x0, y0, tx, ty, f, info, fluid);
@@ -1593,36 +1642,6 @@ __device__ __forceinline__ void step_tile(const D2Args<S, R>& a, int bxy, unsign
         }
     }
 }
-
-// Register cap of a general tile, within the 64 K register file for every
-// variant.  FP32 tiles of more than 128 nodes with staging roles have an SM to
-// themselves at any cap and keep 96 (both strip pulls are in flight at once; at
-// 80 they spill 0.3 KB: 8.56 us per 1024x128 step with 32x8 tiles against 7.7).
-// Those of 32x4 nodes keep 80, at which two share an SM and more fast tiles fit
-// beside one.  us per step at 96 / 80: T-junction batches 8 x 24-38 wide 19.1 /
-// 16.7, 12 x 24-40 26.7 / 21.1, FP16 storage 24 x 24-72 96.4 / 82.5, one device
-// 100 wide 12.5 / 11.7.  A short list leaves the SMs to its tiles either way and
-// runs at 96 (launch_tile).  Serially staged tiles keep 80, which leaves three on
-// an SM (96: 292 -> 295 us per 4096x2048 step, 72.5 -> 75.9 for 24 T-junctions).
-template <int TX, int TY, bool ROLES>
-__host__ __device__ constexpr int gen_threads() {
-    return ROLES ? GenRoles<TX, TY>::THREADS : TX * TY;
-}
-
-// The warps of a CTA are spread over the SM's four sub-partitions, each with
-// 16 K registers, so the cap must let ceil(warps / 4) warps fit in 16 K (a
-// cap checked against the whole 64 K file alone can leave a block that does
-// not launch: 17 warps at 120 registers need 19,200 in one sub-partition).
-template <typename R, int TX, int TY, bool ROLES>
-__host__ __device__ constexpr int gen_maxreg() {
-    constexpr int warps = (gen_threads<TX, TY, ROLES>() + 31) / 32;
-    constexpr int fit = 16384 / (((warps + 3) / 4) * 32) / 8 * 8;
-    constexpr int want = sizeof(R) == 4 ? (ROLES && TX * TY > 128 ? 96 : 80) : 128;
-    return want < fit ? want : fit;
-}
-// Two 32x4 tiles with staging roles share an SM.
-static_assert(2 * ((GenRoles<32, 4>::THREADS / 32 + 3) / 4) * 32 * gen_maxreg<float, 32, 4, true>() <= 16384,
-              "a 32x4 general tile must leave half of the register file");
 
 }  // namespace
 }  // namespace lbm

@@ -35,7 +35,10 @@ __global__ void __launch_bounds__(TX * TY, (fast_min_blocks<R, TX, TY>())) d2q9_
     // one direction / alternating: 1024x1024 periodic 40.7 / 36.5, channels
     // 2048x512 45.6 / 42.8, 4096x2048 293 / 292, 24 T-junctions 76.8 / 75.6.
     const int li = a.list_off + (int)(a.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
-    step_tile<S, R, TX, TY, false>(a, a.blocks[li], a.block_flags[li], 0u, -1);
+    // FP16 tiles of four rows pull their ring in two passes; loaded early, those
+    // spill 0.2 KB at 64 registers (2048x512 channel, 32x4 tiles: 48.0 us per step
+    // early, 44.0 not)
+    step_tile<S, R, TX, TY, false, true, !(is_half_<S>() && TY == 4)>(a, a.blocks[li], a.block_flags[li], 0u, -1);
 }
 
 template <typename S, typename R, int TX, int TY, bool ROLES, int MAXREG = gen_maxreg<R, TX, TY, ROLES>()>
