@@ -220,10 +220,10 @@ lbm_status lbm_kernel_time_split(lbm_ctx* ctx, double* fast_ms, double* general_
 
 /* Tile shape of the fused step kernel: variant in [0, lbm_num_tile_variants()),
  * 0: 32x8, 1: 32x4, 2: 64x4, 3: 32x16 nodes per CTA (default: 0; 1 for
- * FP64 grids with open faces below 2^18 nodes and other grids with an open y
- * face below 2^22).  Bit-identical results on grids without open faces; with
- * open faces the FP64 flux partials are grouped per tile, so chi may differ
- * in its last bit.  Variant 4 tiles like variant 0 and, for FP32 storage,
+ * FP64 grids with open faces below 2^18 nodes or closed ones that spread more
+ * evenly over the SMs with it, and other grids with an open y face below 2^22).
+ * Bit-identical results on grids without open faces; with open faces the FP64
+ * flux partials are grouped per tile, so chi may differ in its last bit.  Variant 4 tiles like variant 0 and, for FP32 storage,
  * runs the interior tiles (those whose pulls and interaction stencil stay
  * inside the grid and away from open faces) through the column-marching
  * kernel: one CTA per run of up to 64 tiles of a tile column, one TMA bulk
@@ -335,9 +335,10 @@ lbm_status lbm_mass_noalloc(const void* f, int precision, int nx, int ny, int pi
  * precision); the caller keeps owning them and may still read them between
  * batch steps (lbm_get_macros, lbm_get_diagnostics, ...).  Every member takes
  * the batch's tile variant: the one set or autotuned for a member (the first
- * such member's), else 1 if that is any member's default, else 0.  A batch
- * step advances every member by one time step with exactly the arithmetic of
- * lbm_step on that member alone. */
+ * such member's), else 1 if a member with open faces defaults to it, else the
+ * default for all members' tiles together.  A batch step advances every
+ * member by one time step with exactly the arithmetic of lbm_step on that
+ * member alone. */
 typedef struct lbm_batch lbm_batch;
 
 /* members: n >= 1 distinct contexts of one precision; cuda_stream: the stream

@@ -956,34 +956,53 @@ lbm_status build_tiles(lbm_ctx* c, int v, bool sync_first) {
 
 
 // Default tile shape (lbm_set_tile_variant overrides): 32x8, whose halo ring
-// costs 0.69 pulls per node against 1.25 for 32x4 (variant 1).  Two kinds of
-// grid keep 32x4.  FP64 tiles hold half as many CTAs per SM: small FP64 grids
-// with open faces are faster with it.  With an open face on a y side the tile
-// height decides which nodes near it the general tiles collide (in packed
-// FP32x2 arithmetic, rounded differently in the last bit), and slow devices
-// amplify that to 2e-5 of u in 200 steps; their results are kept.  us per step,
-// 32x8 / 32x4: 100x100 periodic 3.70 / 4.02, 512x512 10.0 / 10.3, channels
-// 1024x128 7.9 / 9.0, 2048x512 46.1 / 46.7, 4096x1024 155 / 159, FP16 storage
-// 4001x1022 166 / 189, FP64 640x320 142.5 / 141.1, 960x320 194 / 201, 24
-// T-junctions in a batch 72.5 / 77.0.
-int default_variant(const lbm_ctx* c) {
-    const long long nodes = (long long)c->nx * c->ny;
-    if (c->precision == LBM_FP64) return c->nfaces > 0 && nodes < (1LL << 18) ? 1 : 0;
-    return (c->open_side[2] || c->open_side[3]) && nodes < (1LL << 22) ? 1 : 0;
+// costs 0.69 pulls per node against 1.25 for 32x4 (variant 1).  us per step,
+// 32x8 / 32x4: FP32 100x100 periodic 3.9 / 4.2, 512x512 10.3 / 10.7, channels
+// 1024x128 7.7 / 8.5, 2048x512 42.7 / 43.9, 4096x1024 155 / 159; FP16 storage
+// 512x512 10.6 / 12.6, channel 2048x512 41.4 / 44.1.  Three kinds of grid take
+// 32x4.
+// FP64 steps wait for the FP64 pipe of the busiest SM, and a 32x8 tile holds it
+// twice as long as a 32x4 tile (21.7 us against 10.8): closed grids take the
+// shape with fewer tile rows of four on that SM (100x100 25.7 / 16.0, 200x200
+// 47.3 / 37.5, 400x400 113 / 105, but 181x181 26.3 / 27.4).  With open faces the
+// general tiles, whose 32x8 form spills, decide up to about 2^18 nodes (channels
+// 300x48 39.0 / 24.3, 900x100 71.5 / 70.0, obstacle devices 480x160 75.2 / 61.8,
+// 640x320 140.7 / 140.3, 700x370 174.9 / 179.8, 960x320 194 / 201).
+// With an open face on a y side the tile height decides which nodes near it the
+// general tiles collide (in packed FP32x2 arithmetic, rounded differently in the
+// last bit), and slow devices amplify that to 2e-5 of u in 200 steps; grids below
+// 2^22 nodes keep the shape that their results were validated with.  It is the
+// faster one for small devices only: T-junctions 16 wide 8.1 / 7.8, 48 wide 8.8 /
+// 8.7, 160 wide 23.2 / 23.5; FP16 storage 48 wide 9.8 / 9.0, 160 wide 23.4 /
+// 24.0; 24 devices in a batch 72.5 / 76.3.
+// Members of a batch run as one list of tiles and decide together: 32x4 if one
+// of them takes it for its open faces, whatever their order.
+int default_variant(lbm_ctx* const* members, size_t n) {
+    const bool fp64 = members[0]->precision == LBM_FP64;
+    bool faces = false;
+    long long tiles8 = 0, tiles4 = 0;
+    for (size_t i = 0; i < n; ++i) {
+        const lbm_ctx* c = members[i];
+        const long long nodes = (long long)c->nx * c->ny, cols = (c->nx + 31) / 32;
+        faces = faces || c->nfaces > 0;
+        if (fp64 ? c->nfaces > 0 && nodes < (1LL << 18)
+                 : (c->open_side[2] || c->open_side[3]) && nodes < (1LL << 22))
+            return 1;
+        tiles8 += cols * ((c->ny + 7) / 8);
+        tiles4 += cols * ((c->ny + 3) / 4);
+    }
+    const long long sms = device_sms();
+    return fp64 && !faces && (tiles4 + sms - 1) / sms < 2 * ((tiles8 + sms - 1) / sms) ? 1 : 0;
 }
 
-// Tile variant of a new batch, whatever the order of its members: the one that
-// the caller chose for a member (the first such), else 32x4 if that is any
-// member's default.  A member with the 32x4 default keeps its results (see
-// above); those of the others do not depend on the shape but for the last bit
-// of chi (the grouping of its FP64 partials).
+// Tile variant of a new batch: the one that the caller chose for a member (the
+// first such), else the members' default.  A member with an open y face keeps
+// its results (see above); those of the others do not depend on the shape but
+// for the last bit of chi (the grouping of its FP64 partials).
 int batch_variant(const std::vector<lbm_ctx*>& members) {
-    int v = 0;
-    for (const lbm_ctx* c : members) {
+    for (const lbm_ctx* c : members)
         if (c->variant_chosen) return d2q9_tile_kernel_variant(c->variant);
-        v = std::max(v, default_variant(c));
-    }
-    return v;
+    return default_variant(members.data(), members.size());
 }
 
 // ---- snapshots (autotuning runs trial steps and then puts the state back) ----
@@ -1684,7 +1703,7 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
     c->host_solid_in.assign(sol.begin(), sol.end());
     c->h_faceid = faceid;
     c->h_nbrid = nbrid;
-    lbm_status st = build_tiles(c, default_variant(c), false);
+    lbm_status st = build_tiles(c, default_variant(&c, 1), false);
     if (st != LBM_OK) {
         const std::string msg = c->err;
         free_ctx(c);

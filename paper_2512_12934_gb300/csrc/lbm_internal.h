@@ -164,6 +164,8 @@ struct PersistArgs {
 template <typename S, typename R>
 cudaError_t launch_d2q9_persist(const PersistArgs<S, R>& p, int variant, cudaStream_t st, int* grid_out);
 
+int device_sms();  // SMs of the current device
+
 // Launch one list of tiles of one step: general = false -> fast kernel,
 // true -> general kernel; nblocks list entries starting at a.list_off; beside:
 // entries of the step's other list.
