@@ -52,17 +52,39 @@ void side_normal(int side, int* ox, int* oy) {
 // ones serve the rest of a call: a step launched on its own runs its two tile
 // lists one after the other (49 steps of 640x320 FP64: 17 of them at 200 us
 // instead of 171).
+// Capturing and instantiating a short graph costs 40 (one list) to 90 us (two
+// lists), what replaying it saves over 17 (100x100 periodic) or 8 steps (1024x128
+// channel).  It is made once kShortGraphAfter steps that it would have replayed
+// were launched one by one, so a context's first short call does not pay for it:
+// 46 us for 3 steps of 100x100 and 81 of the channel, 77 and 125 with graphs made
+// at once; 86 and 211 against 119 and 220 for 10 steps.
 constexpr int kGraphSizes = 3;
 constexpr int kGraphSteps[kGraphSizes] = {32, 8, 2};
+constexpr int kShortGraphAfter = 8;
 struct StepGraphs {
     cudaGraphExec_t exec[kGraphSizes][2] = {};
     int early[kGraphSizes][2] = {};  // the graph launches its steps early
+    int plain[kGraphSizes][2] = {};  // steps launched one by one for want of the graph
+    // The largest graph to replay next in a run of cnt steps from parity par,
+    // -1: launch *single steps one by one (and count them).
+    int next(int64_t cnt, int par, int* single) {
+        for (int q = 0; q < kGraphSizes; ++q) {
+            if (cnt < kGraphSteps[q]) continue;
+            if (q == 0 || exec[q][par] || plain[q][par] >= kShortGraphAfter) return q;
+            plain[q][par] += kGraphSteps[q];
+            *single = kGraphSteps[q];
+            return -1;
+        }
+        *single = (int)cnt;
+        return -1;
+    }
     void drop() {
         for (int q = 0; q < kGraphSizes; ++q)
             for (int p = 0; p < 2; ++p) {
                 if (exec[q][p]) cudaGraphExecDestroy(exec[q][p]);
                 exec[q][p] = nullptr;
                 early[q][p] = 0;
+                plain[q][p] = 0;
             }
     }
     bool early_in_use() const {
@@ -402,22 +424,26 @@ template <typename S, typename R>
 lbm_status run_plain(lbm_ctx* c, int64_t cnt) {
     const int per = (c->nfast > 0) + (c->ngeneral > 0) + (c->nmarch > 0) + (c->chi_same_step ? 1 : 0);
     const bool replay = cnt >= kGraphSteps[kGraphSizes - 1] && !stream_capturing(c->stream);
-    for (int size = 0; size < kGraphSizes && replay; ++size)
-        while (c->use_graphs && cnt >= kGraphSteps[size]) {
+    while (cnt > 0) {
+        int single = 1;
+        const int size = replay && c->use_graphs ? c->graphs.next(cnt, c->cur, &single) : -1;
+        if (size >= 0) {
             if (ensure_graph<S, R>(c, size, c->cur) != LBM_OK) {
                 c->use_graphs = 0;  // capture unavailable: keep launching the same kernel directly
                 cudaGetLastError();
-                break;
+                continue;
             }
             cudaError_t e = cudaGraphLaunch(c->graphs.exec[size][c->cur], c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "step graph launch");
             c->step += kGraphSteps[size];
             c->launches += (int64_t)kGraphSteps[size] * per;
             cnt -= kGraphSteps[size];
+            continue;
         }
-    for (; cnt > 0; --cnt) {
-        lbm_status st = launch_one<S, R>(c, false, c->stream);
-        if (st != LBM_OK) return st;
+        for (; single > 0; --single, --cnt) {
+            lbm_status st = launch_one<S, R>(c, false, c->stream);
+            if (st != LBM_OK) return st;
+        }
     }
     return LBM_OK;
 }
@@ -1321,9 +1347,9 @@ lbm_status batch_run(lbm_batch* b, int64_t n) {
     int64_t rem = n;
     const bool replay = rem > kGraphSteps[kGraphSizes - 1] && !stream_capturing(b->stream);
     while (rem > 1) {
-        int size = 0;
-        while (size < kGraphSizes && rem - 1 < kGraphSteps[size]) ++size;
-        if (replay && b->use_graphs && size < kGraphSizes) {
+        int single = 1;
+        const int size = replay && b->use_graphs ? b->graphs.next(rem - 1, b->bpar, &single) : -1;
+        if (size >= 0) {
             if (batch_graph<S, R>(b, size, b->bpar) != LBM_OK) {
                 b->use_graphs = 0;
                 cudaGetLastError();
@@ -1334,9 +1360,10 @@ lbm_status batch_run(lbm_batch* b, int64_t n) {
             rem -= kGraphSteps[size];
             continue;
         }
-        BCK((batch_launch<S, R>(b, false, b->stream, nullptr)));
-        batch_advance(b, 1);
-        --rem;
+        for (; single > 0; --single, --rem) {
+            BCK((batch_launch<S, R>(b, false, b->stream, nullptr)));
+            batch_advance(b, 1);
+        }
     }
     if (rem == 1) {
         BCK((batch_launch<S, R>(b, true, b->stream, nullptr)));
