@@ -764,21 +764,22 @@ static cudaError_t plain_step(Ctx3* c, bool write_u, cudaEvent_t a_ev, cudaEvent
 lbm_status step(Ctx3* c, int64_t nsteps) {
     if (nsteps < 0) return fail3(c, nullptr, LBM_ERR_INVALID_ARG, "nsteps must be >= 0");
     const int per = c->nslots > 0 ? 5 : 2;
-    int64_t s = 0;
-    // the call's last step writes u^eq and runs on its own; sampled runs and
+    // the call's last step writes u^eq and runs on its own, as do sampled steps;
     // streams under capture take plain launches throughout
-    while (c->use_graphs && c->time_every == 0 && nsteps - 1 - s >= kGraphSteps3) {
-        if (lbm::stream_capturing(c->stream)) break;
-        if (!ensure_graph3(c)) {
-            c->use_graphs = 0;
-            break;
+    const bool replay = nsteps > kGraphSteps3 && !lbm::stream_capturing(c->stream);
+    for (int64_t s = 0; s < nsteps;) {
+        const int64_t until = c->time_every > 0 ? (c->time_every - c->step % c->time_every) % c->time_every : nsteps;
+        if (replay && c->use_graphs && std::min(nsteps - 1 - s, until) >= kGraphSteps3) {
+            if (!ensure_graph3(c)) {
+                c->use_graphs = 0;
+                continue;
+            }
+            CK3(cudaGraphLaunch(c->gexec[c->cur], c->stream));
+            s += kGraphSteps3;
+            c->step += kGraphSteps3;
+            c->launches += (int64_t)per * kGraphSteps3;
+            continue;
         }
-        CK3(cudaGraphLaunch(c->gexec[c->cur], c->stream));
-        s += kGraphSteps3;
-        c->step += kGraphSteps3;
-        c->launches += (int64_t)per * kGraphSteps3;
-    }
-    for (; s < nsteps; ++s) {
         const bool timed = c->time_every > 0 && (c->step % c->time_every) == 0, last = s + 1 == nsteps;
         if (timed) cudaEventRecord(c->ev[0], c->stream);
         const cudaEvent_t ea = timed ? c->ev[1] : nullptr, eb = timed ? c->ev[2] : nullptr;
@@ -798,6 +799,7 @@ lbm_status step(Ctx3* c, int64_t nsteps) {
         c->launches += per;
         c->cur = 1 - c->cur;
         ++c->step;
+        ++s;
     }
     return LBM_OK;
 }

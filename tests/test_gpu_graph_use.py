@@ -4,7 +4,8 @@ sees what a run does, not how long it takes.
 
 A context's first short call makes no graph (making one costs as much as it
 saves over many steps); short graphs appear once their steps have been wanted
-often enough, and runs of 32 steps use one at once."""
+often enough, and runs of 32 steps use one at once.  In 3D, kernel timing
+interrupts the replay at the sampled steps only."""
 import json
 import os
 import subprocess
@@ -58,8 +59,17 @@ def solver(w):
 
 channel = W.channel(nx=130, ny=30, R=6, xc=40, u_max=0.02, G12=1.4, Gw=(0.3, -0.3))
 box = W.laplace(nx=70, ny=50, R=12, G12=1.2)
+drop = W.laplace3(n=20, R=5.0, G12=1.2)
 res = {"2d": calls(solver(channel), [10] * 4 + [34]),
        "batch": calls(lbm.Batch([solver(channel), solver(box)]), [10] * 4 + [34])}
+s = solver(drop)
+s.step(17)
+for every in (0, 40):
+    s.enable_kernel_timing(every)
+    t0 = s.diagnostics()["step"]
+    s.step(400)
+    s.sync()
+    res["3d_%d" % every] = (seen()[1], t0, s.kernel_time_split()[2])
 print("RESULT " + json.dumps(res))
 """
 
@@ -83,3 +93,18 @@ def test_first_short_calls_make_no_graph(result, kind):
     assert calls[0] == [0, 0]  # 8 of the 10 steps would have been replayed
     assert calls[1] == [1, 1] and calls[2] == [0, 1] and calls[3] == [0, 1]
     assert calls[4] == [1, 1]  # 32 steps at once
+
+
+def test_3d_timing_interrupts_replay_at_samples_only(result):
+    total0, _, _ = result["3d_0"]
+    total1, t0, samples = result["3d_40"]
+    first = -t0 % 40
+    want, s = 0, 0
+    while s < 400:  # runs of 16 before the next sample and before the call's last step
+        until = (first - s) % 40
+        if min(until, 399 - s) >= 16:
+            want, s = want + 1, s + 16
+        else:
+            s += 1
+    assert samples == len([q for q in range(400) if (t0 + q) % 40 == 0])
+    assert total1 - total0 == want > 0
