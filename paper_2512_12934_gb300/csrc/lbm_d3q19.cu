@@ -598,7 +598,6 @@ __device__ __forceinline__ void stencil_sums(Site site, R (&g1)[3], R (&g2)[3]) 
     }
 }
 
-// sum_e w s(x+e) e of Eq. 11 (geometry only; precomputed per near-solid node)
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 // Wait for phase `parity` of an mbarrier for at most about a second of SM
@@ -634,6 +633,7 @@ __device__ __forceinline__ void copy_box(const CUtensorMap* map, void* dst, unsi
         : "memory");
 }
 
+// sum_e w s(x+e) e of Eq. 11 (geometry only; precomputed per near-solid node)
 template <typename S>
 __device__ __forceinline__ void adhesion_vector(const D3Args<S>& a, long long n, uint32_t info,
                                                 typename Store<S>::R (&ad)[3]) {
@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
     __shared__ __half2 s_ref[is_half<S>() ? HN : 1];            // FP16 storage: the same rounded to half
     __shared__ R s_rate[2][Q];  // relaxation rates of both components (indexed by component below)
     // component 0's pulled populations, kept for its collision after
-    // component 1's (FP32 arithmetic; FP64 pulls them again, its tile would
+    // component 1's (FP16 storage; FP64 pulls them again, its tile would
     // exceed the static shared-memory limit)
     constexpr bool STASH = sizeof(R) == 4;
     __shared__ R s_f0[STASH ? Q : 1][STASH ? NT : 1];
@@ -799,8 +799,6 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
     }
     if constexpr (is_half<S>()) {
         for (int q = tid; q < HN; q += NT) s_ref[q] = __floats2half2_rn((float)s_rr[q].x, (float)s_rr[q].y);
-        __syncthreads();
-    } else if (tma) {
         __syncthreads();
     }
     if (info & INFO3_SOLID) return;  // solid, or outside the grid
@@ -904,8 +902,8 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
         a.rref_out[a.plane + n] = __float2half_rn(r2);
     }
     // collide component 1 (still in registers), then component 0 (from the
-    // shared-memory copy in FP32, pulled again in FP64): one loop body, so
-    // the unrolled collision is in the instruction stream once
+    // shared-memory copy with FP16 storage, pulled again in FP64): one loop body,
+    // so the unrolled collision is in the instruction stream once
 #pragma unroll 1
     for (int k = 1; k >= 0; --k) {
         if (k == 0) {
