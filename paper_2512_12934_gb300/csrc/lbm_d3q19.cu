@@ -616,6 +616,14 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* bar, unsigned parit
     }
 }
 
+// The density box has landed.  If the wait runs out the status word says so, and
+// the copy, which still writes this CTA's shared memory, is given as long again.
+__device__ __forceinline__ void wait_box(unsigned long long* bar, unsigned* status, bool report) {
+    if (bar_wait(bar, 0u)) return;
+    if (report) atomicOr(status, STATUS3_TIMEOUT);
+    bar_wait(bar, 0u);
+}
+
 __device__ __forceinline__ void bar_init(unsigned long long* bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -793,7 +801,7 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
         ref1 = __half2float(a.rref_in[a.plane + n]);
     }
     if (tma) {
-        if (!bar_wait(&s_bar, 0u) && tid == 0) atomicOr(a.status, STATUS3_TIMEOUT);
+        wait_box(&s_bar, a.status, tid == 0);
     } else {
         __syncthreads();
     }
@@ -1133,7 +1141,7 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
         }
     }
     if (tma) {
-        if (!bar_wait(&s_bar, 0u) && tid == 0) atomicOr(a.status, STATUS3_TIMEOUT);
+        wait_box(&s_bar, a.status, tid == 0);
     } else {
         __syncthreads();
     }
