@@ -146,15 +146,14 @@ __device__ __forceinline__ R feq_(int i, R rho, R ux, R uy) {
 // population planes exceed 2^31 elements).  Pull stream (Eq. 2): f_i(x) =
 // f*_i(x - e_i); a set bit i in `info` means that source is solid or outside
 // a closed edge, and halfway bounce-back (Eq. B1) takes f*_opp(i)(x).
-
 //
 // A pull is issued in two parts.  The loads take the plain neighbours (wrapped
 // on every axis, so always inside the grid) and need no descriptor: they go out
 // together with the descriptor's own load instead of one memory latency after
 // it, and cost no selects.  The few nodes with a blocked direction then replace
-// those values.  us per step, before -> now: 100x100 periodic 4.67 -> 3.70,
-// 512x512 10.6 -> 9.9, channels 1024x128 8.25 -> 7.9, 4096x2048 308 -> 292, 24
-// T-junctions in a batch 80.7 -> 77.0.
+// those values.  us per step, descriptor first / loads first, on otherwise equal
+// source: 100x100 periodic 4.67 / 3.70, 512x512 10.6 / 9.9, channels 1024x128
+// 8.25 / 7.9, 4096x2048 308 / 292.
 
 // Loads of an interior node: every source lies inside the grid, no wrap needed.
 template <typename S, typename R>

@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(Tile3<S>::NT, Tile3<S>::MIN_BLOCKS)
     __shared__ R s_f0[STASH ? Q : 1][STASH ? NT : 1];
     // from the last z on: the pull kernel has just read those planes (L2), and the
     // next one starts on the planes this kernel writes last (co-flow 250x64x64
-    // 112.7 -> 108.4 us per step, 512x96x96 400 -> 397)
+    // 112.7 us per step in ascending order, 108.4 in this one; 512x96x96 400, 397)
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (zblock + (int)(gridDim.z - 1 - blockIdx.z)) * TZ;
     const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
@@ -1086,8 +1086,7 @@ __device__ __forceinline__ void collide2(const Moments2& M, float2 r, float ux, 
 // result: 80 registers and three CTAs of 256 per SM instead of two at 126 with
 // the populations in registers (265 against 277 us on the 512x96x96 co-flow
 // device; one component after the other, 64 registers: 330).  The rest is load
-// latency and shared-memory throughput (l1tex 58 %, DRAM 51 %); the step went
-// from 530 to 408 us.
+// latency and shared-memory throughput (l1tex 58 %, DRAM 51 %).
 __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
     d3q_collide_f32_kernel(const __grid_constant__ D3Args<float> a, const __grid_constant__ CUtensorMap rho_map,
                            int use_tma, int zblock) {
@@ -1100,7 +1099,7 @@ __global__ void __launch_bounds__(Tile3<float>::NT, Tile3<float>::MIN_BLOCKS)
     __shared__ __align__(8) unsigned long long s_bar;
     // from the last z on: the pull kernel has just read those planes (L2), and the
     // next one starts on the planes this kernel writes last (co-flow 250x64x64
-    // 112.7 -> 108.4 us per step, 512x96x96 400 -> 397)
+    // 112.7 us per step in ascending order, 108.4 in this one; 512x96x96 400, 397)
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (zblock + (int)(gridDim.z - 1 - blockIdx.z)) * TZ;
     const int tid = threadIdx.x + TX * (threadIdx.y + TY * threadIdx.z);
     const unsigned s_f = smem_addr(s_rr + HN) + 8u * (unsigned)tid;

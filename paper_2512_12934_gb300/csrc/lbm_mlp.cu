@@ -62,8 +62,8 @@ __device__ __forceinline__ void adam_update(float& w, float& m, float& v, float 
 // took 11 us (8 CTAs) and 15 us (16 CTAs).  The form before this, one CTA per
 // 32 samples and three launches per step, left all but 10 SMs idle at a
 // minibatch of 64 and staged transposed weights with uncoalesced reads.
-// Step of 5 members, before -> now: minibatch 64 109 -> 15 us, 256 111 -> 28
-// us, 1024 161 -> 68 us, 4096 449 -> 206 us.
+// Step of 5 members, that form / this one: minibatch 64 109 / 15 us, 256 111 /
+// 28, 1024 161 / 68, 4096 449 / 206.
 constexpr int TT = 512;                        // threads per CTA
 constexpr int WS = H + 4;                      // padded weight row: 16-byte accesses of 8 rows or of one row
 constexpr int iW2 = 0, iW3 = iW2 + H * WS;     // shared parameter image (floats)
@@ -756,9 +756,9 @@ __device__ __forceinline__ void tc_issue_chunk(int c, uint32_t tmem, uint32_t wh
 // tiles x, x + gridDim.x, ... of that member.  The FP32 work between the layers
 // (GELU, operand splitting) bounds it, so the MMAs run under it: a layer's input
 // is produced in four chunks of 32 neurons (8 per warp quarter) and each chunk's
-// MMAs are issued while the next chunk is computed.  Before (erff, the whole
-// layer written, one barrier, 40 MMAs, a wait): 222 us for 65,536 points x 5
-// members with the tensor pipe idle 78 % of the time; now 140 us.
+// MMAs are issued while the next chunk is computed: 140 us for 65,536 points x 5
+// members (222 with erff and the whole layer written before one barrier, 40 MMAs
+// and a wait, the tensor pipe idle 78 % of the time).
 __global__ void __launch_bounds__(TCT, 1) mlp_infer_tc_kernel(const float* __restrict__ params,
                                                               const unsigned char* __restrict__ img,
                                                               const float* __restrict__ X, int B,
