@@ -241,7 +241,7 @@ lbm_status lbm_tile_stats(lbm_ctx* ctx, int* variant, int* fast_tiles, int* gene
 
 /* Step-replay mode: use_graphs != 0 (the default) replays runs of steps
  * from captured CUDA graphs (two launches per graph node pair; runs of 32
- * steps are captured on first use, of 8 and 2 once they have been wanted for 8
+ * steps are captured on first use, of 8 and 2 once they have been wanted for 16
  * steps); 0 launches every step individually.  Results are identical. */
 lbm_status lbm_set_graph_mode(lbm_ctx* ctx, int use_graphs);
 

@@ -53,14 +53,15 @@ void side_normal(int side, int* ox, int* oy) {
 // lists one after the other (49 steps of 640x320 FP64: 17 of them at 200 us
 // instead of 171).
 // Capturing and instantiating a short graph costs 40 (one list) to 90 us (two
-// lists), what replaying it saves over 17 (100x100 periodic) or 8 steps (1024x128
-// channel).  It is made once kShortGraphAfter steps that it would have replayed
-// were launched one by one, so a context's first short call does not pay for it:
-// 46 us for 3 steps of 100x100 and 81 of the channel, 77 and 125 with graphs made
-// at once; 86 and 211 against 119 and 220 for 10 steps.
+// lists), what replaying it saves over 17 (100x100 periodic), 8 (1024x128
+// channel) or 2 steps (640x320 FP64).  It is made once the steps that it replays
+// in this run and those launched one by one for want of it come to
+// kShortGraphAfter, so a context's first short call does not pay for it: 47 us
+// for 3 steps of 100x100 and 81 of the channel, 77 and 125 with graphs made at
+// once; 86 and 209 against 119 and 220 for 10 steps.
 constexpr int kGraphSizes = 3;
 constexpr int kGraphSteps[kGraphSizes] = {32, 8, 2};
-constexpr int kShortGraphAfter = 8;
+constexpr int kShortGraphAfter = 16;
 struct StepGraphs {
     cudaGraphExec_t exec[kGraphSizes][2] = {};
     int early[kGraphSizes][2] = {};  // the graph launches its steps early
@@ -70,7 +71,8 @@ struct StepGraphs {
     int next(int64_t cnt, int par, int* single) {
         for (int q = 0; q < kGraphSizes; ++q) {
             if (cnt < kGraphSteps[q]) continue;
-            if (q == 0 || exec[q][par] || plain[q][par] >= kShortGraphAfter) return q;
+            if (q == 0 || exec[q][par] || plain[q][par] + cnt / kGraphSteps[q] * kGraphSteps[q] >= kShortGraphAfter)
+                return q;
             plain[q][par] += kGraphSteps[q];
             *single = kGraphSteps[q];
             return -1;
@@ -999,8 +1001,8 @@ lbm_status build_tiles(lbm_ctx* c, int v, bool sync_first) {
 // last bit), and slow devices amplify that to 2e-5 of u in 200 steps; grids below
 // 2^22 nodes keep the shape that their results were validated with.  It is the
 // faster one for small devices only: T-junctions 16 wide 8.1 / 7.8, 48 wide 8.8 /
-// 8.7, 160 wide 23.2 / 23.5; FP16 storage 48 wide 9.8 / 9.0, 160 wide 23.4 /
-// 24.0; 24 devices in a batch 72.5 / 76.3.
+// 8.7, 160 wide 23.2 / 23.5, 24 devices of 24-72 in a batch 69.4 / 78.0; FP16
+// storage 48 wide 9.8 / 9.0, 160 wide 23.4 / 24.0, the batch 80.8 / 83.3.
 // Members of a batch run as one list of tiles and decide together: 32x4 if one
 // of them takes it for its open faces, whatever their order.
 int default_variant(lbm_ctx* const* members, size_t n) {

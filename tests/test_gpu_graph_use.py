@@ -61,6 +61,7 @@ channel = W.channel(nx=130, ny=30, R=6, xc=40, u_max=0.02, G12=1.4, Gw=(0.3, -0.
 box = W.laplace(nx=70, ny=50, R=12, G12=1.2)
 drop = W.laplace3(n=20, R=5.0, G12=1.2)
 res = {"2d": calls(solver(channel), [10] * 4 + [34]),
+       "long": calls(solver(channel), [18] * 2),
        "batch": calls(lbm.Batch([solver(channel), solver(box)]), [10] * 4 + [34])}
 s = solver(drop)
 s.step(17)
@@ -93,6 +94,10 @@ def test_first_short_calls_make_no_graph(result, kind):
     assert calls[0] == [0, 0]  # 8 of the 10 steps would have been replayed
     assert calls[1] == [1, 1] and calls[2] == [0, 1] and calls[3] == [0, 1]
     assert calls[4] == [1, 1]  # 32 steps at once
+
+
+def test_a_call_that_wants_a_short_graph_twice_makes_it(result):
+    assert result["long"] == [[1, 2], [0, 2]]
 
 
 def test_3d_timing_interrupts_replay_at_samples_only(result):
