@@ -989,7 +989,9 @@ namespace {
 // kernels read X and write the results over the host link themselves, two
 // launches and one synchronisation instead of those plus four copies (221
 // points: 63 -> 31 us a call; beyond a few thousand points the copy engine moves the
-// bytes faster than every member reading X over the link).
+// bytes faster than every member reading X over the link).  The pinned block costs
+// 110 us at creation and 160 when it is freed in a process that holds no other
+// pinned memory, 2 us otherwise.
 constexpr int kMappedPoints = 4096;
 
 lbm_status mfail(lbm_mlp* m, lbm_status st, const std::string& msg) {
