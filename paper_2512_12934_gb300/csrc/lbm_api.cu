@@ -394,6 +394,7 @@ lbm_status launch_one(lbm_ctx* c, bool macros, cudaStream_t st, cudaEvent_t mid 
 template <typename S, typename R>
 lbm_status ensure_graph(lbm_ctx* c, int size, int par) {
     if (c->graphs.exec[size][par]) return LBM_OK;
+    RelaxedCapture relaxed;
     if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     if (!c->side_stream) CK(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
     if (!c->ev_fork) CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
@@ -1307,6 +1308,7 @@ lbm_status batch_run_persistent(lbm_batch* b, int64_t n) {
 template <typename S, typename R>
 lbm_status batch_graph(lbm_batch* b, int size, int par) {
     if (b->graphs.exec[size][par]) return LBM_OK;
+    RelaxedCapture relaxed;
     if (!b->cap_stream) BCK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
     if (!b->side_stream) BCK(cudaStreamCreateWithFlags(&b->side_stream, cudaStreamNonBlocking));
     if (!b->ev_fork) BCK(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));

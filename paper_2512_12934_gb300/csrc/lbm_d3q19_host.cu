@@ -733,6 +733,7 @@ static cudaError_t capture_steps(Ctx3* c, cudaGraph_t* g) {
 // The graph of the current parity; false: stepping goes on with plain launches.
 static bool ensure_graph3(Ctx3* c) {
     if (c->gexec[c->cur]) return true;
+    lbm::RelaxedCapture relaxed;
     cudaError_t e = cudaSuccess;
     if (!c->cap_stream) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess && !c->side_stream) e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);

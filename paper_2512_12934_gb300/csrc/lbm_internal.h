@@ -224,6 +224,17 @@ inline bool stream_capturing(cudaStream_t st) {
     return true;
 }
 
+// While it lives, this thread may create streams, events and executable graphs
+// although another stream of the process is being captured: none of them touches
+// that stream, but outside the relaxed mode the runtime ends its capture.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+    RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 // Dense macroscopic fields rho [2][ny][nx], u [2][ny][nx] from macro [4][plane]
 // (0 at solid nodes); rho and u may be device or mapped host memory.  Nothing
 // is written when *status is set; *status_out (mapped host memory) receives it.

@@ -1,7 +1,9 @@
 """Steps recorded into a caller's stream capture: runs of every length a step
 graph would serve are recorded as plain launches, and a replay of the caller's
 graph leaves the state that the same steps leave when run at once, bit for
-bit (2D, batch and 3D; before and after the context has graphs of its own)."""
+bit (2D, batch and 3D; before and after the context has graphs of its own).
+Steps on one stream while another is being captured run at once, graphs of their
+own included, and leave that capture alone."""
 import numpy as np
 import pytest
 
@@ -52,3 +54,31 @@ def test_captured_steps_replay(kind, n, warm):
     plain.sync()
     for a, b in zip(pm, rm):
         assert np.array_equal(a.populations(), b.populations())
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("kind", ["2d", "batch", "3d"])
+def test_steps_beside_a_capture(kind, mode):
+    import torch
+
+    runs = (10, 10, 10, 40)
+    plain, pm = make(kind, None)
+    for n in runs:
+        plain.step(n)
+    plain.sync()
+    captured, own = torch.cuda.Stream(), torch.cuda.Stream()
+    run, rm = make(kind, own.cuda_stream)
+    run.sync()
+    x = torch.zeros(100, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=captured, capture_error_mode=mode):
+        x += 1
+        for n in runs:
+            run.step(n)
+        x += 1
+    run.sync()
+    for a, b in zip(pm, rm):
+        assert np.array_equal(a.populations(), b.populations())
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(x[0]) == 2.0
